@@ -101,15 +101,17 @@ typedef struct msf_projector msf_projector;
  * would lie inside the volume's circumscribed cylinder (dso and dsd-dso must
  * exceed its radius), or when a ray could be steeper than 45 deg to the
  * rotation plane (the z-major case, which this projector does not model).
- * Allocates the table, two z-paired copies of a 4D volume (the forward's
- * inputs, 16*N bytes) and a step-weighted sinogram. */
+ * Allocates the table, a copy of a 4D volume in lines along z (the forward's
+ * input, 4 bytes per voxel and per element of the lines' margins) and a
+ * step-weighted sinogram. */
 msf_status msf_projector_create(const msf_geom* geom, const msf_vol* vol, msf_projector** out);
 void msf_projector_destroy(msf_projector* p);
 /* Device bytes held by the plan. */
 size_t msf_projector_bytes(const msf_projector* p);
 
-/* Autotuner: times the forward projector with ray blocks of 32x4, 64x2 and
- * 16x8 (columns x rows) and the gather adjoint with voxel runs of 8, 16 and 32
+/* Autotuner: times the forward projector with its three launch shapes, named
+ * 32x4, 64x2 and 16x8 (4, 8 or 2 detector columns per block, one warp each over
+ * sets of 32 rows), and the gather adjoint with voxel runs of 8, 16 and 32
  * along z (and 64 when the gather grid of 64-voxel runs is still at least 24
  * waves of 8 blocks per SM deep) on this plan's geometry, and keeps the
  * fastest of each for the plan.

@@ -106,49 +106,45 @@ __global__ void column_table_kernel(const double* __restrict__ angles, float4* _
     (void)na;
 }
 
-// ------------------------------------------------------------------ z-paired copies
+// ------------------------------------------------------------------ z-contiguous copies
 
-// Per frame and z-slice, the two copies of a volume v that the forward reads:
-// py[z][y][x] = (v(z, y, x), v(z + 1, y, x)) and px[z][x][y], the same pairs
-// transposed (x-major rays read y-contiguous data), with v(nz, ., .) = 0, so
-// that a ray's four bilinear taps are two 8-byte loads.
+// The forward reads a frame as lines of voxels along z: line (y, x) of frame t
+// starts at ((t*ny + y)*nx + x) * nzp, voxel z at element VZ_FRONT + z.  The
+// elements before and after the nz voxels are zeros that nothing writes (the
+// buffers are cleared when they are allocated), so that a tap outside the
+// volume in z reads 0 without a check.
+constexpr int VZ_FRONT = 4;
+__host__ __device__ __forceinline__ int vz_pitch(int nz) { return (nz + VZ_FRONT + 2 + 7) & ~7; }
+
+// Copies [nt][nz][ny][nx] -> z-contiguous lines, through 32 x 32 shared tiles
+// of one (t, y) plane.  Bound by HBM (8 bytes per voxel).
 // FUSED: v = r + beta_t p (the CG direction update) with p = in; v is also
-// written to pnext (a different buffer: neighbouring slices still read p).
+// written to pnext.
 template <bool FUSED>
-__global__ void pair_kernel(const float* __restrict__ in, float2* __restrict__ px, float2* __restrict__ py,
-                            const float* __restrict__ r, float* __restrict__ pnext, const double* __restrict__ beta,
-                            int nx, int ny, int nz) {
-    __shared__ float2 tile[32][33];
-    const int slice = blockIdx.z;             // t * nz + z
-    const int t = slice / nz, z = slice % nz;
-    const size_t plane = (size_t)nx * ny;
-    const size_t base = (size_t)slice * plane;
-    const bool up = z + 1 < nz;
-    const int x0 = blockIdx.x * 32, y0 = blockIdx.y * 32;
+__global__ void lines_kernel(const float* __restrict__ in, float* __restrict__ vz, const float* __restrict__ r,
+                             float* __restrict__ pnext, const double* __restrict__ beta, int nx, int ny, int nz) {
+    __shared__ float tile[32][33];
+    const int t = blockIdx.x / ny, y = blockIdx.x % ny;
+    const int x0 = blockIdx.y * 32, z0 = blockIdx.z * 32;
+    const int nzp = vz_pitch(nz);
     float bt = 0.0f;
     if (FUSED) bt = (float)beta[t];
     for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-        const int x = x0 + threadIdx.x, y = y0 + k;
-        if (x < nx && y < ny) {
-            const size_t i = base + (size_t)y * nx + x;
-            float lo, hi = 0.0f;
+        const int x = x0 + threadIdx.x, z = z0 + k;
+        if (x < nx && z < nz) {
+            const size_t i = (((size_t)t * nz + z) * ny + y) * nx + x;
+            float v = in[i];
             if (FUSED) {
-                lo = __fmaf_rn(bt, in[i], r[i]);
-                if (up) hi = __fmaf_rn(bt, in[i + plane], r[i + plane]);
-                pnext[i] = lo;
-            } else {
-                lo = in[i];
-                if (up) hi = in[i + plane];
+                v = __fmaf_rn(bt, v, r[i]);
+                pnext[i] = v;
             }
-            const float2 v = make_float2(lo, hi);
-            py[i] = v;
             tile[k][threadIdx.x] = v;
         }
     }
     __syncthreads();
     for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-        const int y = y0 + threadIdx.x, x = x0 + k;
-        if (x < nx && y < ny) px[base + (size_t)x * ny + y] = tile[threadIdx.x][k];
+        const int x = x0 + k, z = z0 + threadIdx.x;
+        if (x < nx && z < nz) vz[(((size_t)t * ny + y) * nx + x) * nzp + VZ_FRONT + z] = tile[threadIdx.x][k];
     }
 }
 
@@ -156,168 +152,227 @@ __global__ void pair_kernel(const float* __restrict__ in, float2* __restrict__ p
 
 enum FwdMode { FWD_PLAIN = 0, FWD_LAMBDA = 1, FWD_RESIDUAL = 2 };
 
-// Rays per thread of the forward: consecutive detector rows of one column,
-// which share the column's in-plane crossing (f_a, its floor and weight).
-constexpr int FWD_R = 2;
+// Row sets (32 detector rows each) of one warp.  Five sets share a plane's
+// in-plane arithmetic among the most rays (160 rows: 0.67 ms in one chunk of
+// five, 0.86 in two of three); up to four sets two planes are unrolled under a
+// limit of three blocks per SM, which keeps their loads in flight (384 rows:
+// 2.43 ms in chunks of four, 2.76 without the limit, 2.69 in chunks of six,
+// whose slab of z-slices also leaves L2).
+constexpr int FWD_MAX_R = 5;
 
-// Narrows [kmin, kmax] to the planes k where f(k) = f0 + (k - cmaj) b lies in
-// [lo, hi], one plane inside the exact bounds on each side (so that FP32
-// rounding of f never leaves [lo, hi] inside the range).
-__device__ __forceinline__ void planes_within(float f0, float b, float lo, float hi, float cmaj, float& kmin,
-                                              float& kmax) {
-    if (fabsf(b) > 1e-12f) {
-        const float k1 = (lo - f0) / b + cmaj, k2 = (hi - f0) / b + cmaj;
-        kmin = fmaxf(kmin, ceilf(fminf(k1, k2)) + 1.0f);
-        kmax = fminf(kmax, floorf(fmaxf(k1, k2)) - 1.0f);
-    } else if (!(f0 >= lo && f0 <= hi)) {
-        kmax = kmin - 1.0f;
-    }
+// 2^23 + 2^22: adding it in round-down mode leaves floor(f) in the low mantissa
+// bits for |f| < 2^22, so the floor and its integer cost two additions instead
+// of two conversions.
+constexpr float FLOOR_MAGIC = 12582912.0f;
+constexpr int FLOOR_MAGIC_BITS = 0x4B400000;
+
+// Two FP32 values in one 64-bit register: one instruction issues both lanes'
+// operation, each rounded as its scalar form (sm_100 and later).
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2_rd(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rm.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
 }
 
-// One thread per FWD_R rays (detector rows FWD_R*i .. FWD_R*i + FWD_R - 1 of one
-// column); a block covers blockDim.x columns x FWD_R*blockDim.y rows of one view
-// (128 threads; the shape is chosen per plan by msf_projector_autotune).  x-major
-// rays read the z-paired transposed frame px [nz][nx][ny], y-major rays the
-// z-paired natural frame py [nz][ny][nx] (pair_kernel), so the minor in-plane
-// axis is contiguous and each (a, z) tap pair is one 8-byte load.  Planes
-// where every bilinear tap of every ray of the thread lies inside the grid run
-// without bounds checks; the planes at either end check each tap.  The
-// interpolation is v00 + w_a (v01 - v00) along a, then the same along z.
+// A warp takes one detector column and R sets of 32 consecutive rows (lane =
+// row in a set); a block takes blockDim.y neighbouring columns.  All rays of a
+// column lie in one vertical plane: on voxel plane k of the major axis they
+// share the in-plane crossing f_a, so the warp forms it once for its R sets and
+// reads two z-lines (a0 and a0 + 1), along which the lanes step by the row
+// spacing.  Bound by L1 wavefronts: a crossing is four 4-byte loads, and a load
+// of 32 lanes (a span of 32 row spacings, on any alignment) takes 1.86.  With
+// lanes along u and 8-byte loads of z-paired copies (16 bytes of copies per
+// voxel) it took 8.8 for each of two loads: 30.1 -> 16.6 ms at 384^3 x 16, 512 x
+// 384 detector, 24 views (740 G crossings/s); 0.90 -> 0.62 ms at 128^3 x 8, 192 x
+// 160, 32 views; 25 -> 10 us at 24^3 x 4, 32 x 32, 12 views.  Pairs of sets
+// share instructions (f32x2), since at 30 instructions per crossing the issue
+// slots bound it as much (2.43 against 2.59 ms at 384^3 x 2).
+// The interpolation is v00 + w_a (v01 - v00) along a, then the same along z,
+// summed over increasing planes.  A line outside the volume in a is the zero
+// line; f_z is clamped to [-2, nz], where both taps are zeros of the line's
+// margins, so a lane outside the volume adds exactly zero.
 //   FWD_PLAIN:    out = A x
 //   FWD_LAMBDA:   out = step * Lambda * (A x)
 //   FWD_RESIDUAL: out = step * Lambda * (meas - A x)
 // (the CG modes write the step-weighted sinogram e' = step * e that the gather
-// adjoint consumes)
+// adjoint consumes).  The sums go through shared memory so that the sinogram is
+// read and written in 32-byte pieces along u.
+// Blocks run over the columns and views of one set of rows before the next:
+// the rows of a set cross a slab of z-slices that stays in L2 for all views.
 // PAR (the ICD agent's projection of a group step): x is zero outside one
 // voxel parity group, so an x-major ray only visits planes x = kpx (mod 2) and
 // a y-major ray planes y = kpy (mod 2), and on a visited plane it loads only
-// the z-pair of the minor-axis tap with the group's parity (the other is zero);
+// the line of the minor-axis tap with the group's parity (the other is zero);
 // the skipped terms are exact zeros, so the result equals the full projection
 // bit for bit.
-template <int MODE, bool PAR = false>
-__global__ void __launch_bounds__(128) joseph_fwd_kernel(
-    const float2* __restrict__ px, const float2* __restrict__ py, const float4* __restrict__ col,
-    float* __restrict__ out, const float* __restrict__ lam, const float* __restrict__ meas,
-    ProjDims d, int kpx = 0, int kpy = 0) {
-    const int iu = blockIdx.x * blockDim.x + threadIdx.x;
-    const int iv0 = (blockIdx.y * blockDim.y + threadIdx.y) * FWD_R;
-    const int g = blockIdx.z;
-    if (iu >= d.nu || iv0 >= d.nv) return;
-    const int t = g / d.views;
-    const ColParams c = load_col(col, (size_t)g * d.nu + iu);
-    const bool xmaj = c.xmajor != 0.0f;
-    const int nmaj = xmaj ? d.nx : d.ny, na = xmaj ? d.ny : d.nx;
-    const size_t fs = (size_t)d.nx * d.ny * d.nz;
-    const float2* __restrict__ vol = (xmaj ? px : py) + (size_t)t * fs;   // (v(z), v(z+1)) pairs
-    const float cmaj = xmaj ? d.cx : d.cy;
-    const int zs = nmaj * na;    // z stride of the frame
-
-    RayZ rz[FWD_R];
+template <int MODE, int R, bool PAR>
+__global__ void __launch_bounds__(256, R == 5 ? 1 : 3) joseph_fwd_kernel(
+    const float* __restrict__ vz, const float* __restrict__ zero_line, const float4* __restrict__ col,
+    float* __restrict__ out, const float* __restrict__ lam, const float* __restrict__ meas, ProjDims d, int kpx,
+    int kpy) {
+    extern __shared__ float fwd_sum[];   // [32 R rows][columns + 1]
+    const int lane = threadIdx.x, ncol = blockDim.y;
+    const int ublocks = (d.nu + ncol - 1) / ncol;
+    const int iu0 = (blockIdx.x % ublocks) * ncol, iu = iu0 + threadIdx.y;
+    const int iv0 = blockIdx.y * 32 * R;
+    const int t = blockIdx.z, g = t * d.views + blockIdx.x / ublocks;
+    if (iu < d.nu) {
+        const ColParams c = load_col(col, (size_t)g * d.nu + iu);
+        const bool xmaj = c.xmajor != 0.0f;
+        const int nmaj = xmaj ? d.nx : d.ny, na = xmaj ? d.ny : d.nx;
+        const int nzp = vz_pitch(d.nz);
+        // element strides of the major and the minor in-plane axis
+        const ptrdiff_t smaj = xmaj ? nzp : (ptrdiff_t)d.nx * nzp, smin = xmaj ? (ptrdiff_t)d.nx * nzp : nzp;
+        const float* vol = vz + (size_t)t * d.ny * d.nx * nzp + VZ_FRONT;
+        const float* zl = zero_line + VZ_FRONT;
+        const float cmaj = xmaj ? d.cx : d.cy;
+        const float zmax = (float)d.nz;
+        // f_z of the rows, packed by pairs of sets; the last set of an odd R alone
+        float f_mid[R], f_b[R];
+        // planes where a crossing of the warp can touch the grid (-1 < f < n on
+        // both minor axes, one plane of margin)
+        int K0 = nmaj, K1 = -1;
 #pragma unroll
-    for (int r = 0; r < FWD_R; ++r) rz[r] = ray_z(c, det_v(min(iv0 + r, d.nv - 1), d), d.cz);
-
-    // planes where some crossing can touch the grid (-1 < f < n on both minor
-    // axes, one plane of margin), and the inner planes where all four taps of
-    // every ray are inside (0.5 <= f <= n - 1.5)
-    float klo = (float)(nmaj - 1), khi = 0.0f;
-    float kin_lo = 0.0f, kin_hi = (float)(nmaj - 1);
-    planes_within(c.fa_mid, c.ba, 0.5f, (float)na - 1.5f, cmaj, kin_lo, kin_hi);
+        for (int r = 0; r < R; ++r) {
+            const RayZ rz = ray_z(c, det_v(min(iv0 + 32 * r + lane, d.nv - 1), d), d.cz);
+            f_mid[r] = rz.fz_mid;
+            f_b[r] = rz.bz;
+            float lo = 0.0f, hi = (float)(nmaj - 1);
+            const float fm[2] = {c.fa_mid, rz.fz_mid}, bb[2] = {c.ba, rz.bz};
+            const float top[2] = {(float)na, (float)d.nz};
 #pragma unroll
-    for (int r = 0; r < FWD_R; ++r) {
-        float lo = 0.0f, hi = (float)(nmaj - 1);
-        const float fm[2] = {c.fa_mid, rz[r].fz_mid}, bb[2] = {c.ba, rz[r].bz};
-        const float top[2] = {(float)na, (float)d.nz};
-        for (int a = 0; a < 2; ++a) {
-            if (fabsf(bb[a]) > 1e-12f) {
-                const float k1 = (-1.0f - fm[a]) / bb[a] + cmaj, k2 = (top[a] - fm[a]) / bb[a] + cmaj;
-                lo = fmaxf(lo, floorf(fminf(k1, k2)) - 1.0f);
-                hi = fminf(hi, ceilf(fmaxf(k1, k2)) + 1.0f);
-            } else if (!(fm[a] > -1.0f && fm[a] < top[a])) {
-                hi = -1.0f;
+            for (int a = 0; a < 2; ++a) {
+                if (fabsf(bb[a]) > 1e-12f) {
+                    const float k1 = (-1.0f - fm[a]) / bb[a] + cmaj, k2 = (top[a] - fm[a]) / bb[a] + cmaj;
+                    lo = fmaxf(lo, floorf(fminf(k1, k2)) - 1.0f);
+                    hi = fminf(hi, ceilf(fmaxf(k1, k2)) + 1.0f);
+                } else if (!(fm[a] > -1.0f && fm[a] < top[a])) {
+                    hi = -1.0f;
+                }
+            }
+            if (lo <= hi) {
+                K0 = min(K0, (int)lo);
+                K1 = max(K1, (int)hi);
             }
         }
-        if (lo <= hi) {
-            klo = fminf(klo, lo);
-            khi = fmaxf(khi, hi);
+        f32x2 fzm[R / 2 + 1], bz[R / 2 + 1], acc[R / 2 + 1];
+#pragma unroll
+        for (int r = 0; r < R / 2; ++r) {
+            fzm[r] = pack2(f_mid[2 * r], f_mid[2 * r + 1]);
+            bz[r] = pack2(f_b[2 * r], f_b[2 * r + 1]);
+            acc[r] = 0;
         }
-        planes_within(rz[r].fz_mid, rz[r].bz, 0.5f, (float)d.nz - 1.5f, cmaj, kin_lo, kin_hi);
-    }
-    float acc[FWD_R];
-#pragma unroll
-    for (int r = 0; r < FWD_R; ++r) acc[r] = 0.0f;
-    if (klo <= khi) {
-        const int K0 = (int)klo, K1 = (int)khi;
-        int F0 = (int)fmaxf(kin_lo, klo), F1 = (int)fminf(kin_hi, khi);
-        if (F0 > F1) F0 = K1 + 1, F1 = K1;
-
-        // one plane with every tap checked against the grid
-        auto checked = [&](int k) {
-            const float tk = __fsub_rn((float)k, cmaj);
+        const float fzm1 = f_mid[R - 1], bz1 = f_b[R - 1];
+        float acc1 = 0.0f;
+        K0 = __reduce_min_sync(0xffffffffu, K0);
+        K1 = __reduce_max_sync(0xffffffffu, K1);
+        const int kp = xmaj ? kpx : kpy, ka = xmaj ? kpy : kpx;
+        if (PAR) K0 += (K0 ^ kp) & 1;
+        const float* lk = vol + K0 * smaj;   // lines of plane k
+        float tk = __fsub_rn((float)K0, cmaj);
+#pragma unroll(R == 5 ? 1 : R == 1 ? 4 : 2)
+        for (int k = K0; k <= K1; k += PAR ? 2 : 1) {
             const float fa = __fmaf_rn(tk, c.ba, c.fa_mid);
-            const float a0f = floorf(fa);
-            const float wa1 = __fsub_rn(fa, a0f);
-            const int ia = (int)a0f;
-            const bool a_in0 = ia >= 0 && ia < na, a_in1 = ia + 1 >= 0 && ia + 1 < na;
+            const float am = __fadd_rd(fa, FLOOR_MAGIC);
+            const float wa1 = __fsub_rn(fa, __fsub_rn(am, FLOOR_MAGIC));
+            const int ia = __float_as_int(am) - FLOOR_MAGIC_BITS;
+            const float* l0 = lk + ia * smin;
+            const float* l1 = l0 + smin;
+            if ((unsigned)ia >= (unsigned)na) l0 = zl;
+            if ((unsigned)(ia + 1) >= (unsigned)na) l1 = zl;
+            // PAR: the line of the tap with the group's parity
+            const bool first = (ia & 1) == ka;
+            // the lines' addresses less the bits of FLOOR_MAGIC, which every index carries
+            l0 -= FLOOR_MAGIC_BITS;
+            l1 -= FLOOR_MAGIC_BITS;
+            const f32x2 tk2 = pack2(tk, tk), wa2 = pack2(wa1, wa1), m2 = pack2(FLOOR_MAGIC, FLOOR_MAGIC);
 #pragma unroll
-            for (int r = 0; r < FWD_R; ++r) {
-                const float fz = __fmaf_rn(tk, rz[r].bz, rz[r].fz_mid);
-                const float z0f = floorf(fz);
-                const float wz1 = __fsub_rn(fz, z0f);
-                const int iz = (int)z0f;
-                // the pair of slice iz holds taps iz and iz + 1 (0 above the
-                // grid); below it (iz = -1) only the upper tap, from slice 0
-                float v00 = 0.0f, v01 = 0.0f, v10 = 0.0f, v11 = 0.0f;
-                if (iz >= 0 && iz < d.nz) {
-                    const float2* row = vol + ((ptrdiff_t)iz * nmaj + k) * na;
-                    if (a_in0) { const float2 q = __ldg(row + ia); v00 = q.x; v10 = q.y; }
-                    if (a_in1) { const float2 q = __ldg(row + ia + 1); v01 = q.x; v11 = q.y; }
-                } else if (iz == -1) {
-                    const float2* row = vol + (ptrdiff_t)k * na;
-                    if (a_in0) v10 = __ldg(row + ia).x;
-                    if (a_in1) v11 = __ldg(row + ia + 1).x;
+            for (int r = 0; r < R / 2; ++r) {
+                float f0, f1;
+                unpack2(fma2(tk2, bz[r], fzm[r]), f0, f1);
+                const f32x2 fz = pack2(fminf(fmaxf(f0, -2.0f), zmax), fminf(fmaxf(f1, -2.0f), zmax));
+                const f32x2 zm = add2_rd(fz, m2);
+                const f32x2 wz = sub2(fz, sub2(zm, m2));
+                float i0, i1;
+                unpack2(zm, i0, i1);
+                const int j0 = __float_as_int(i0), j1 = __float_as_int(i1);
+                f32x2 v00 = 0, v10 = 0, v01 = 0, v11 = 0;
+                if (!PAR || first) {
+                    v00 = pack2(__ldg(l0 + j0), __ldg(l0 + j1));
+                    v10 = pack2(__ldg(l0 + j0 + 1), __ldg(l0 + j1 + 1));
+                }
+                if (!PAR || !first) {
+                    v01 = pack2(__ldg(l1 + j0), __ldg(l1 + j1));
+                    v11 = pack2(__ldg(l1 + j0 + 1), __ldg(l1 + j1 + 1));
+                }
+                const f32x2 top = fma2(wa2, sub2(v01, v00), v00);
+                const f32x2 bot = fma2(wa2, sub2(v11, v10), v10);
+                acc[r] = add2(acc[r], fma2(wz, sub2(bot, top), top));
+            }
+            if (R & 1) {
+                const float fz = fminf(fmaxf(__fmaf_rn(tk, bz1, fzm1), -2.0f), zmax);
+                const float zm = __fadd_rd(fz, FLOOR_MAGIC);
+                const float wz1 = __fsub_rn(fz, __fsub_rn(zm, FLOOR_MAGIC));
+                const int j = __float_as_int(zm);
+                float v00 = 0.0f, v10 = 0.0f, v01 = 0.0f, v11 = 0.0f;
+                if (!PAR || first) {
+                    v00 = __ldg(l0 + j);
+                    v10 = __ldg(l0 + j + 1);
+                }
+                if (!PAR || !first) {
+                    v01 = __ldg(l1 + j);
+                    v11 = __ldg(l1 + j + 1);
                 }
                 const float top = __fmaf_rn(wa1, __fsub_rn(v01, v00), v00);
                 const float bot = __fmaf_rn(wa1, __fsub_rn(v11, v10), v10);
-                acc[r] = __fadd_rn(acc[r], __fmaf_rn(wz1, __fsub_rn(bot, top), top));
+                acc1 = __fadd_rn(acc1, __fmaf_rn(wz1, __fsub_rn(bot, top), top));
             }
-        };
-        const int kp = xmaj ? kpx : kpy, ka = xmaj ? kpy : kpx;
-        for (int k = K0; k < F0; ++k)
-            if (!PAR || (k & 1) == kp) checked(k);
-        for (int k = PAR ? F0 + ((F0 ^ kp) & 1) : F0; k <= F1; k += PAR ? 2 : 1) {
-            const float tk = __fsub_rn((float)k, cmaj);
-            const float fa = __fmaf_rn(tk, c.ba, c.fa_mid);
-            const float a0f = floorf(fa);
-            const float wa1 = __fsub_rn(fa, a0f);
-            const float2* pk = vol + k * na + (int)a0f;
-            const bool lo = (((int)a0f) & 1) == ka;   // PAR: the tap at a0 has the group's parity
-#pragma unroll
-            for (int r = 0; r < FWD_R; ++r) {
-                const float fz = __fmaf_rn(tk, rz[r].bz, rz[r].fz_mid);
-                const float z0f = floorf(fz);
-                const float wz1 = __fsub_rn(fz, z0f);
-                const float2* p0 = pk + (ptrdiff_t)((int)z0f) * zs;
-                const float2 zero = make_float2(0.0f, 0.0f);
-                const float2 q0 = (!PAR || lo) ? __ldg(p0) : zero;
-                const float2 q1 = (!PAR || !lo) ? __ldg(p0 + 1) : zero;
-                const float v00 = q0.x, v10 = q0.y, v01 = q1.x, v11 = q1.y;
-                const float top = __fmaf_rn(wa1, __fsub_rn(v01, v00), v00);
-                const float bot = __fmaf_rn(wa1, __fsub_rn(v11, v10), v10);
-                acc[r] = __fadd_rn(acc[r], __fmaf_rn(wz1, __fsub_rn(bot, top), top));
-            }
+            lk += PAR ? 2 * smaj : smaj;
+            tk += PAR ? 2.0f : 1.0f;
         }
-        for (int k = F1 + 1; k <= K1; ++k)
-            if (!PAR || (k & 1) == kp) checked(k);
-    }
 #pragma unroll
-    for (int r = 0; r < FWD_R; ++r) {
-        const int iv = iv0 + r;
-        if (iv >= d.nv) break;
-        const float val = acc[r] * rz[r].step;
-        const size_t ray = ((size_t)g * d.nv + iv) * d.nu + iu;
+        for (int r = 0; r < R / 2; ++r) {
+            float a0, a1;
+            unpack2(acc[r], a0, a1);
+            fwd_sum[(64 * r + lane) * (ncol + 1) + threadIdx.y] = a0;
+            fwd_sum[(64 * r + 32 + lane) * (ncol + 1) + threadIdx.y] = a1;
+        }
+        if (R & 1) fwd_sum[(32 * (R - 1) + lane) * (ncol + 1) + threadIdx.y] = acc1;
+    }
+    __syncthreads();
+    for (int i = threadIdx.y * 32 + lane; i < 32 * R * ncol; i += 32 * ncol) {
+        const int cu = i % ncol, row = i / ncol, iv = iv0 + row, ju = iu0 + cu;
+        if (iv >= d.nv || ju >= d.nu) continue;
+        const float step = ray_z(load_col(col, (size_t)g * d.nu + ju), det_v(iv, d), d.cz).step;
+        const float val = fwd_sum[row * (ncol + 1) + cu] * step;
+        const size_t ray = ((size_t)g * d.nv + iv) * d.nu + ju;
         if (MODE == FWD_PLAIN) out[ray] = val;
-        else if (MODE == FWD_LAMBDA) out[ray] = rz[r].step * (lam[ray] * val);
-        else out[ray] = rz[r].step * (lam[ray] * (meas[ray] - val));
+        else if (MODE == FWD_LAMBDA) out[ray] = step * (lam[ray] * val);
+        else out[ray] = step * (lam[ray] * (meas[ray] - val));
     }
 }
 
@@ -902,10 +957,10 @@ struct msf_projector {
     float4* d_col = nullptr;
     float2* d_trig = nullptr;
     int* d_vflag = nullptr;
-    float2* d_px = nullptr;    // z-paired volume, [nt][nz][nx][ny] (x-major rays)
-    float2* d_py = nullptr;    // z-paired volume, [nt][nz][ny][nx] (y-major rays)
+    float* d_vz = nullptr;     // z-contiguous lines of a volume (the forward's input)
+    float* d_zero = nullptr;   // one line of zeros
     float* d_sw = nullptr;     // step-weighted sinogram for msf_backproject
-    int fwd_bx = 32, fwd_by = 4;   // forward ray block (columns x rows)
+    int fwd_bx = 32, fwd_by = 4;   // forward launch shape (fwd_cols_of: detector columns per block)
     int adj_zb = 16;               // gather z-run length
     uint64_t tuning_gen = 0;       // advanced whenever the launch shapes change
     size_t bytes = 0;
@@ -932,48 +987,67 @@ static size_t sino_size(const msf_projector* p) {
     return (size_t)p->geom.nu * p->geom.nv * p->geom.views * p->vol.nt;
 }
 
-static msf_status launch_pairs(msf_projector* p, const float* in, cudaStream_t st) {
+static dim3 lines_grid(const msf_vol& v) { return dim3(v.ny * v.nt, (v.nx + 31) / 32, (v.nz + 31) / 32); }
+
+static msf_status launch_lines(msf_projector* p, const float* in, cudaStream_t st) {
     const msf_vol& v = p->vol;
-    dim3 grid((v.nx + 31) / 32, (v.ny + 31) / 32, v.nz * v.nt);
     MSF_PROF("transpose", st);
-    pair_kernel<false><<<grid, dim3(32, 8), 0, st>>>(in, p->d_px, p->d_py, nullptr, nullptr, nullptr, v.nx, v.ny, v.nz);
+    lines_kernel<false><<<lines_grid(v), dim3(32, 8), 0, st>>>(in, p->d_vz, nullptr, nullptr, nullptr, v.nx, v.ny, v.nz);
     MSF_LAUNCH_CHECK();
     return MSF_OK;
 }
 
-// Forward grid: blockDim.x columns x FWD_R*blockDim.y rows per block, one z per view.
-static dim3 fwd_grid(const ProjDims& d, dim3 block) {
-    const unsigned rows = block.y * FWD_R;
-    return dim3((d.nu + block.x - 1) / block.x, (d.nv + rows - 1) / rows, d.nt * d.views);
+template <int MODE, bool PAR>
+static void launch_fwd_kernel(msf_projector* p, const float* vz, float* out, const float* lam, const float* meas,
+                              int kpx, int kpy, cudaStream_t st) {
+    const ProjDims& d = p->dims;
+    // detector columns (warps) per block; row sets of 32 rows, split evenly
+    // over as few chunks as FWD_MAX_R allows
+    const int ncol = p->fwd_bx / 8;
+    const int sets = (d.nv + 31) / 32, chunks = (sets + FWD_MAX_R - 1) / FWD_MAX_R, R = (sets + chunks - 1) / chunks;
+    const dim3 block(32, ncol), grid((d.nu + ncol - 1) / ncol * d.views, chunks, d.nt);
+    const size_t smem = (size_t)32 * R * (ncol + 1) * sizeof(float);
+#define MSF_FWD_CASE(N)                                                                                            \
+    case N:                                                                                                        \
+        joseph_fwd_kernel<MODE, N, PAR><<<grid, block, smem, st>>>(vz, p->d_zero, p->d_col, out, lam, meas, d,     \
+                                                                    kpx, kpy);                                     \
+        break;
+    switch (R) {
+        MSF_FWD_CASE(1)
+        MSF_FWD_CASE(2)
+        MSF_FWD_CASE(3)
+        MSF_FWD_CASE(4)
+        MSF_FWD_CASE(5)
+    }
+#undef MSF_FWD_CASE
+}
+
+// A of the volume whose lines are vz.
+static msf_status launch_fwd_lines(msf_projector* p, int mode, const float* vz, float* out, const float* lam,
+                                   const float* meas, cudaStream_t st) {
+    MSF_PROF("joseph_fwd", st);
+    if (mode == FWD_PLAIN)
+        launch_fwd_kernel<FWD_PLAIN, false>(p, vz, out, lam, meas, 0, 0, st);
+    else if (mode == FWD_LAMBDA)
+        launch_fwd_kernel<FWD_LAMBDA, false>(p, vz, out, lam, meas, 0, 0, st);
+    else
+        launch_fwd_kernel<FWD_RESIDUAL, false>(p, vz, out, lam, meas, 0, 0, st);
+    MSF_LAUNCH_CHECK();
+    return MSF_OK;
 }
 
 static msf_status launch_fwd(msf_projector* p, int mode, const float* x, float* out,
                              const float* lam, const float* meas, cudaStream_t st) {
-    MSF_TRY(launch_pairs(p, x, st));
-    const ProjDims& d = p->dims;
-    dim3 block(p->fwd_bx, p->fwd_by);
-    dim3 grid = fwd_grid(d, block);
-    MSF_PROF("joseph_fwd", st);
-    if (mode == FWD_PLAIN)
-        joseph_fwd_kernel<FWD_PLAIN><<<grid, block, 0, st>>>(p->d_px, p->d_py, p->d_col, out, lam, meas, d);
-    else if (mode == FWD_LAMBDA)
-        joseph_fwd_kernel<FWD_LAMBDA><<<grid, block, 0, st>>>(p->d_px, p->d_py, p->d_col, out, lam, meas, d);
-    else
-        joseph_fwd_kernel<FWD_RESIDUAL><<<grid, block, 0, st>>>(p->d_px, p->d_py, p->d_col, out, lam, meas, d);
-    MSF_LAUNCH_CHECK();
-    return MSF_OK;
+    MSF_TRY(launch_lines(p, x, st));
+    return launch_fwd_lines(p, mode, p->d_vz, out, lam, meas, st);
 }
 
 // A x for an x that is zero outside the voxels with x = kpx and y = kpy (mod 2)
 // (the ICD agent's group step), visiting only the planes that can touch them.
 static msf_status launch_fwd_parity(msf_projector* p, const float* x, float* out, int kpx, int kpy, cudaStream_t st) {
-    MSF_TRY(launch_pairs(p, x, st));
-    const ProjDims& d = p->dims;
-    dim3 block(p->fwd_bx, p->fwd_by);
-    dim3 grid = fwd_grid(d, block);
+    MSF_TRY(launch_lines(p, x, st));
     MSF_PROF("joseph_fwd", st);
-    joseph_fwd_kernel<FWD_PLAIN, true><<<grid, block, 0, st>>>(p->d_px, p->d_py, p->d_col, out, nullptr, nullptr, d,
-                                                               kpx, kpy);
+    launch_fwd_kernel<FWD_PLAIN, true>(p, p->d_vz, out, nullptr, nullptr, kpx, kpy, st);
     MSF_LAUNCH_CHECK();
     return MSF_OK;
 }
@@ -1063,17 +1137,18 @@ extern "C" msf_status msf_projector_create(const msf_geom* geom, const msf_vol* 
 
     auto cleanup = [&](msf_status st) { msf_projector_destroy(p); return st; };
     const size_t col_bytes = (size_t)G * geom->nu * 2 * sizeof(float4);
-    const size_t vol_bytes = vol_size(*vol) * sizeof(float);
+    const size_t line_bytes = vz_pitch(vol->nz) * sizeof(float);
+    const size_t vz_bytes = (size_t)vol->nt * vol->ny * vol->nx * line_bytes;
     if (cudaMalloc(&p->d_angles, G * sizeof(double)) != cudaSuccess ||
         cudaMalloc(&p->d_col, col_bytes) != cudaSuccess ||
         cudaMalloc(&p->d_trig, G * sizeof(float2)) != cudaSuccess ||
         cudaMalloc(&p->d_vflag, G * sizeof(int)) != cudaSuccess ||
-        cudaMalloc(&p->d_px, 2 * vol_bytes) != cudaSuccess || cudaMalloc(&p->d_py, 2 * vol_bytes) != cudaSuccess ||
+        cudaMalloc(&p->d_vz, vz_bytes) != cudaSuccess || cudaMalloc(&p->d_zero, line_bytes) != cudaSuccess ||
         cudaMalloc(&p->d_sw, sino_size(p) * sizeof(float)) != cudaSuccess) {
         cudaGetLastError();
         return cleanup(fail(MSF_ERR_NOMEM, "msf_projector_create: out of device memory"));
     }
-    p->bytes = G * sizeof(double) + col_bytes + G * (sizeof(float2) + sizeof(int)) + 4 * vol_bytes +
+    p->bytes = G * sizeof(double) + col_bytes + G * (sizeof(float2) + sizeof(int)) + vz_bytes + line_bytes +
                sino_size(p) * sizeof(float);
     std::vector<float2> trig(G);
     for (int g = 0; g < G; ++g) trig[g] = make_float2((float)cos(p->angles[g]), (float)sin(p->angles[g]));
@@ -1082,6 +1157,8 @@ extern "C" msf_status msf_projector_create(const msf_geom* geom, const msf_vol* 
     cudaError_t e = cudaMemcpy(p->d_angles, p->angles.data(), G * sizeof(double), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(p->d_trig, trig.data(), G * sizeof(float2), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(p->d_vflag, 0, G * sizeof(int));
+    if (e == cudaSuccess) e = cudaMemset(p->d_vz, 0, vz_bytes);
+    if (e == cudaSuccess) e = cudaMemset(p->d_zero, 0, line_bytes);
     if (e == cudaSuccess) e = cudaMalloc(&d_bad, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(d_bad, 0, sizeof(int));
     if (e == cudaSuccess) {
@@ -1104,8 +1181,8 @@ extern "C" void msf_projector_destroy(msf_projector* p) {
     cudaFree(p->d_col);
     cudaFree(p->d_trig);
     cudaFree(p->d_vflag);
-    cudaFree(p->d_px);
-    cudaFree(p->d_py);
+    cudaFree(p->d_vz);
+    cudaFree(p->d_zero);
     cudaFree(p->d_sw);
     delete p;
 }
@@ -1196,30 +1273,22 @@ extern "C" msf_status msf_prox_data(msf_dataprox* dp, const float* d_y, const fl
         MSF_LAUNCH_CHECK();
     }
     const msf_vol& v = p->vol;
-    const dim3 tgrid((v.nx + 31) / 32, (v.ny + 31) / 32, v.nz * v.nt);
-    // the direction p alternates between two buffers: the fused update reads
-    // p at slices z and z + 1 while writing the new p
+    // the direction p alternates between two buffers
     float* pc = dp->d_p;
     for (int it = 0; it < n_cg; ++it) {
-        // z-paired copies of p for the forward pass (fused with p = r + beta p after the first pass)
+        // lines of p for the forward (fused with p = r + beta p after the first pass)
         if (it == 0) {
-            MSF_TRY(launch_pairs(p, pc, st));
+            MSF_TRY(launch_lines(p, pc, st));
         } else {
             float* pn = pc == dp->d_p ? dp->d_p2 : dp->d_p;
             MSF_PROF("transpose_pupdate", st);
-            pair_kernel<true><<<tgrid, dim3(32, 8), 0, st>>>(pc, p->d_px, p->d_py, dp->d_r, pn, dp->d_beta, v.nx,
-                                                             v.ny, v.nz);
+            lines_kernel<true><<<lines_grid(v), dim3(32, 8), 0, st>>>(pc, p->d_vz, dp->d_r, pn, dp->d_beta, v.nx, v.ny,
+                                                                      v.nz);
             MSF_LAUNCH_CHECK();
             pc = pn;
         }
-        {   // s = Lambda A p  (pairs already built)
-            const ProjDims& d = p->dims;
-            dim3 block(p->fwd_bx, p->fwd_by);
-            dim3 grid = fwd_grid(d, block);
-            MSF_PROF("joseph_fwd", st);
-            joseph_fwd_kernel<FWD_LAMBDA><<<grid, block, 0, st>>>(p->d_px, p->d_py, p->d_col, dp->d_s, d_lambda, nullptr, d);
-            MSF_LAUNCH_CHECK();
-        }
+        // s = Lambda A p
+        MSF_TRY(launch_fwd_lines(p, FWD_LAMBDA, p->d_vz, dp->d_s, d_lambda, nullptr, st));
         // q = A^T s + p/sigma^2 ; alpha = rr / p.q
         MSF_TRY(launch_adj(p, ADJ_CG_Q, dp->d_s, dp->d_q, pc, nullptr, nullptr, dp->d_partial, inv_s2, st));
         {
@@ -1550,8 +1619,6 @@ extern "C" msf_status msf_projector_autotune(msf_projector* p, void* stream, int
         cudaEventElapsedTime(&ms, e0, e1);
         return ms;
     };
-    MSF_TRY_CUDA(cudaMemsetAsync(p->d_px, 0, nv * sizeof(float2), st));
-    MSF_TRY_CUDA(cudaMemsetAsync(p->d_py, 0, nv * sizeof(float2), st));
     MSF_TRY_CUDA(cudaMemsetAsync(p->d_sw, 0, ns * sizeof(float), st));
     const int shapes[3][2] = {{32, 4}, {64, 2}, {16, 8}};
     float best = 1e30f;
@@ -1559,12 +1626,7 @@ extern "C" msf_status msf_projector_autotune(msf_projector* p, void* stream, int
     for (int i = 0; i < 3; ++i) {
         p->fwd_bx = shapes[i][0];
         p->fwd_by = shapes[i][1];
-        const float ms = time_it([&] {
-            const ProjDims& d = p->dims;
-            dim3 block(p->fwd_bx, p->fwd_by);
-            dim3 grid = fwd_grid(d, block);
-            joseph_fwd_kernel<FWD_PLAIN><<<grid, block, 0, st>>>(p->d_px, p->d_py, p->d_col, tmp, nullptr, nullptr, d);
-        });
+        const float ms = time_it([&] { launch_fwd_kernel<FWD_PLAIN, false>(p, p->d_vz, tmp, nullptr, nullptr, 0, 0, st); });
         if (ms < best) { best = ms; bi = i; }
     }
     p->fwd_bx = shapes[bi][0];
