@@ -111,10 +111,10 @@ size_t msf_projector_bytes(const msf_projector* p);
 
 /* Autotuner: times the forward projector with its three launch shapes, named
  * 32x4, 64x2 and 16x8 (4, 8 or 2 detector columns per block, one warp each over
- * sets of 32 rows), and the gather adjoint with voxel runs of 8, 16 and 32
- * along z (and 64 when the gather grid of 64-voxel runs is still at least 24
- * waves of 8 blocks per SM deep) on this plan's geometry, and keeps the
- * fastest of each for the plan.
+ * sets of 32 rows), and the gather adjoint with the z-runs 8, 16 and 32 (at most
+ * 2, 4 or 6 voxels per lane of a block's lines, 32 lanes) and, when its grid is
+ * still at least 24 waves of 8 blocks per SM deep, 64 (at most 12), on this
+ * plan's geometry, and keeps the fastest of each for the plan.
  * Results do not depend on the choice (same per-ray arithmetic and the same
  * per-voxel summation order).  Synchronises; allocates a temporary buffer.
  * h_choice (optional, 3 ints) receives {block columns, block rows, z-run}. */
@@ -137,8 +137,9 @@ msf_status msf_projector_set_tuning(msf_projector* p, int fwd_cols, int fwd_rows
 msf_status msf_project(msf_projector* p, const float* d_x, float* d_y, void* stream);
 
 /* x = A^T y for every time-point: the matched adjoint of msf_project, computed
- * as a voxel-driven gather (no atomics) that re-derives, bit for bit, the
- * forward's interpolation weights for every ray touching the voxel.
+ * as a voxel-driven gather (no atomics) that re-derives the forward's
+ * interpolation weights for every ray touching the voxel: those along the minor
+ * in-plane axis bit for bit, those along z to the rounding of the crossing.
  * d_y: sinogram; d_x: 4D volume (overwritten). */
 msf_status msf_backproject(msf_projector* p, const float* d_y, float* d_x, void* stream);
 

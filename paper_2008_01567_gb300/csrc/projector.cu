@@ -160,6 +160,13 @@ enum FwdMode { FWD_PLAIN = 0, FWD_LAMBDA = 1, FWD_RESIDUAL = 2 };
 // whose slab of z-slices also leaves L2).
 constexpr int FWD_MAX_R = 5;
 
+// The step-weighted sinogram e' as the gather reads it: lines of detector rows,
+// row iv of (view g, column iu) at (g*nu + iu) * sino_pitch + SINO_FRONT + iv.
+// The margins are zeros that nothing writes: rows a voxel's window reaches
+// beyond the detector read 0.
+constexpr int SINO_FRONT = 4, SINO_BACK = 4;
+__host__ __device__ __forceinline__ int sino_pitch(int nv) { return (nv + SINO_FRONT + SINO_BACK + 7) & ~7; }
+
 // 2^23 + 2^22: adding it in round-down mode leaves floor(f) in the low mantissa
 // bits for |f| < 2^22, so the floor and its integer cost two additions instead
 // of two conversions.
@@ -219,8 +226,9 @@ __device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
 //   FWD_LAMBDA:   out = step * Lambda * (A x)
 //   FWD_RESIDUAL: out = step * Lambda * (meas - A x)
 // (the CG modes write the step-weighted sinogram e' = step * e that the gather
-// adjoint consumes).  The sums go through shared memory so that the sinogram is
-// read and written in 32-byte pieces along u.
+// adjoint consumes; ROWS: as lines of detector rows, sino_pitch).  The sums go
+// through shared memory so that the sinogram is read and written in 16-byte
+// pieces along u.
 // Blocks run over the columns and views of one set of rows before the next:
 // the rows of a set cross a slab of z-slices that stays in L2 for all views.
 // PAR (the ICD agent's projection of a group step): x is zero outside one
@@ -229,7 +237,7 @@ __device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
 // the line of the minor-axis tap with the group's parity (the other is zero);
 // the skipped terms are exact zeros, so the result equals the full projection
 // bit for bit.
-template <int MODE, int R, bool PAR>
+template <int MODE, int R, bool PAR, bool ROWS>
 __global__ void __launch_bounds__(256, R == 5 ? 1 : 3) joseph_fwd_kernel(
     const float* __restrict__ vz, const float* __restrict__ zero_line, const float4* __restrict__ col,
     float* __restrict__ out, const float* __restrict__ lam, const float* __restrict__ meas, ProjDims d, int kpx,
@@ -368,11 +376,21 @@ __global__ void __launch_bounds__(256, R == 5 ? 1 : 3) joseph_fwd_kernel(
         const int cu = i % ncol, row = i / ncol, iv = iv0 + row, ju = iu0 + cu;
         if (iv >= d.nv || ju >= d.nu) continue;
         const float step = ray_z(load_col(col, (size_t)g * d.nu + ju), det_v(iv, d), d.cz).step;
-        const float val = fwd_sum[row * (ncol + 1) + cu] * step;
+        float* sum = fwd_sum + row * (ncol + 1) + cu;
+        const float val = *sum * step;
         const size_t ray = ((size_t)g * d.nv + iv) * d.nu + ju;
-        if (MODE == FWD_PLAIN) out[ray] = val;
-        else if (MODE == FWD_LAMBDA) out[ray] = step * (lam[ray] * val);
-        else out[ray] = step * (lam[ray] * (meas[ray] - val));
+        float res = val;
+        if (MODE == FWD_LAMBDA) res = step * (lam[ray] * val);
+        if (MODE == FWD_RESIDUAL) res = step * (lam[ray] * (meas[ray] - val));
+        if (ROWS) *sum = res;
+        else out[ray] = res;
+    }
+    if (ROWS) {
+        __syncthreads();
+        if (iu >= d.nu) return;
+        float* o = out + ((size_t)g * d.nu + iu) * sino_pitch(d.nv) + SINO_FRONT;
+        for (int row = lane; row < 32 * R && iv0 + row < d.nv; row += 32)
+            o[iv0 + row] = fwd_sum[row * (ncol + 1) + threadIdx.y];
     }
 }
 
@@ -380,162 +398,333 @@ __global__ void __launch_bounds__(256, R == 5 ? 1 : 3) joseph_fwd_kernel(
 
 enum AdjMode { ADJ_PLAIN = 0, ADJ_CG_INIT = 1, ADJ_CG_Q = 2 };
 
-// Voxels of one z-run handled by one thread of the gather: 8, 16, 32 or 64,
-// chosen per plan (default 16).
+constexpr int ADJ_T = 4;           // a block's tile: ADJ_T x ADJ_T voxel lines in (x, y), one warp per ADJ_T
+constexpr int ADJ_ENTRIES = 32;    // columns of a warp's list
+// floats of one line in a block's tile: its 32 J voxels, and 8 that put the
+// lines read together on different banks
+__host__ __device__ constexpr int adj_line(int J) { return 32 * J + 8; }
 
 // Detector u coordinate (in pixels) of the point (x, y, .) for view (cs, sn);
 // only used to bound candidate columns, so a fast division is enough.
 __device__ __forceinline__ float u_pixel(float x, float y, float cs, float sn, const ProjDims& d) {
     const float lat = -x * sn + y * cs;
     const float depth = d.dso - x * cs - y * sn;
-    return __fdividef(d.dsd * lat, depth) / d.du + d.cu;
+    return __fdividef(d.dsd * lat, depth * d.du) + d.cu;
 }
 
-// Adds, for the rays of one view whose major axis is XMAJ, w(ray, voxel) *
-// e'(ray) to the ZB accumulators of the voxel run (ix, iy, iz_lo ..
-// iz_lo+ZB-1), where e' = step * e is the step-weighted sinogram.
-//
-// An x-major ray touches column (ix, iy) on plane k = ix when floor(f_y) is
-// iy-1 or iy.  Candidate detector columns come from the exact projection of
-// the segment {x = x_ix, |y - y_iy| <= voxel} (plus one column of margin); on
-// a column that qualifies, the rows whose f_z(k) can fall within one voxel of
-// the run follow from f_z(v) = c_z + v (c1 + tk inv_dmaj).  Each ray's f_a is
-// recomputed with the forward's own operations (bit for bit); f_z of row 0
-// likewise, and of a row iv by one FMA from it (a few 1e-5 voxel from the
-// forward's value, so the taps agree except within that distance of a voxel
-// boundary, where the weights are continuous; the value depends on the ray
-// alone, not on the run length the plan's autotuner picks).
-// Every ray-plane crossing of the forward is visited by the two runs that hold
-// its a-taps, so the work tracks the forward's.
-template <bool XMAJ, int ZB>
-__device__ __forceinline__ void gather_runs(const float4* __restrict__ col, const float* __restrict__ e,
-                                            int g, int ix, int iy, int iz_lo, float cs, float sn,
-                                            const ProjDims& d, float (*acc)[128], int tid) {
-    const int kpl = XMAJ ? ix : iy;             // plane index along the major axis
-    const int ia = XMAJ ? iy : ix;              // voxel index on the minor axis
-    const float cmaj = XMAJ ? d.cx : d.cy;
-    const float xc = (ix - d.cx) * d.vox, yc = (iy - d.cy) * d.vox;
-    float u1, u2;
-    if (XMAJ) {
-        u1 = u_pixel(xc, yc - d.vox, cs, sn, d);
-        u2 = u_pixel(xc, yc + d.vox, cs, sn, d);
-    } else {
-        u1 = u_pixel(xc - d.vox, yc, cs, sn, d);
-        u2 = u_pixel(xc + d.vox, yc, cs, sn, d);
+// One detector column that crosses a warp's run of voxel lines; what the packed
+// operations take is stored twice.
+struct __align__(16) AdjEntry {
+    float2 dfz, nrdfz;   // row spacing along z on this plane (voxels), and minus its reciprocal
+    float2 c0, wa;       // cv + 1 - 1/dfz; weight of the line after the crossing
+    float2 wb;           // 1 - wa: weight of the line before it
+    const float* row0;   // the column's row 0, less FLOOR_MAGIC_BITS elements
+};
+constexpr int ADJ_FAST = 32;   // slot flag: two rows per footprint, none outside the line's margins
+
+__device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ f32x2 vfma(f32x2 a, f32x2 b, f32x2 c) { return fma2(a, b, c); }
+__device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ f32x2 vadd(f32x2 a, f32x2 b) { return add2(a, b); }
+__device__ __forceinline__ float vadd_rd(float a, float b) { return __fadd_rd(a, b); }
+__device__ __forceinline__ f32x2 vadd_rd(f32x2 a, f32x2 b) { return add2_rd(a, b); }
+__device__ __forceinline__ float vsub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ f32x2 vsub(f32x2 a, f32x2 b) { return sub2(a, b); }
+template <typename V> struct Lanes;
+template <> struct Lanes<float> {
+    static constexpr int N = 1;
+    __device__ static __forceinline__ float all(float a) { return a; }
+    __device__ static __forceinline__ float pack(const float* a) { return a[0]; }
+    __device__ static __forceinline__ void unpack(float v, float* a) { a[0] = v; }
+};
+template <> struct Lanes<f32x2> {
+    static constexpr int N = 2;
+    __device__ static __forceinline__ f32x2 all(float a) { return pack2(a, a); }
+    __device__ static __forceinline__ f32x2 pack(const float* a) { return pack2(a[0], a[1]); }
+    __device__ static __forceinline__ void unpack(f32x2 v, float* a) { unpack2(v, a[0], a[1]); }
+};
+
+__device__ __forceinline__ float vbc(float2 a, float) { return a.x; }
+__device__ __forceinline__ f32x2 vbc(float2 a, f32x2) { return pack2(a.x, a.y); }
+
+// sum over the rows iv of one column of max(0, 1 - |f_z(iv) - z|) e'(iv) for
+// the voxels V of a lane (one, or two packed).  f_z(iv) - z = (iv - cv) dfz +
+// (cz - z), both bracketed terms exact, so only dfz carries a rounding.  The
+// window starts at the first row with f_z > z - 1 and holds NR rows (NR = 0:
+// `rows`, any number); all but its last lie inside the voxel's footprint, and
+// the last is dropped where it does not, so that a non-finite reading reaches
+// the voxels of its own footprint only.  CLAMP: the window may lie outside the
+// detector.
+template <int NR, bool CLAMP, typename V>
+__device__ __forceinline__ V row_sum(const AdjEntry& q, int rows, V zc, const ProjDims& d) {
+    using L = Lanes<V>;
+    float lo[L::N], w[L::N], ev[L::N];
+    const V dfz = vbc(q.dfz, V());
+    V t = vfma(zc, vbc(q.nrdfz, V()), vbc(q.c0, V()));
+    if (CLAMP) {
+        float tt[L::N];
+        L::unpack(t, tt);
+#pragma unroll
+        for (int k = 0; k < L::N; ++k) tt[k] = fminf(fmaxf(tt[k], (float)-SINO_FRONT), (float)d.nv);
+        t = L::pack(tt);
     }
-    const int iu_lo = max(0, (int)floorf(fminf(u1, u2)) - 1);
-    const int iu_hi = min(d.nu - 1, (int)ceilf(fmaxf(u1, u2)) + 1);
-    const float tk = __fsub_rn((float)kpl, cmaj);
-    const float inv_dv = 1.0f / d.dv;
-    for (int iu = iu_lo; iu <= iu_hi; ++iu) {
-        const ColParams c = load_col(col, (size_t)g * d.nu + iu);
-        if ((c.xmajor != 0.0f) != XMAJ) continue;
-        const float fa = __fmaf_rn(tk, c.ba, c.fa_mid);
-        const float a0f = floorf(fa);
-        const int a0 = (int)a0f;
-        if (ia != a0 && ia != a0 + 1) continue;
-        const float wa1 = __fsub_rn(fa, a0f);
-        const float wa = (ia == a0) ? __fsub_rn(1.0f, wa1) : wa1;
-        // rows with f_z in (iz_lo - 1, iz_lo + ZB); gz > 0 (planes lie
-        // between source and detector)
-        const float rgz = __fdividef(1.0f, c.c1 + tk * c.inv_dmaj);
-        const float va = (iz_lo - 1 - d.cz) * rgz * inv_dv + d.cv;
-        const float vb = (iz_lo + ZB - d.cz) * rgz * inv_dv + d.cv;
-        const int iv_lo = max(0, (int)floorf(va) - 1);
-        const int iv_hi = min(d.nv - 1, (int)ceilf(vb) + 1);
-        const float* erow = e + ((size_t)g * d.nv) * d.nu + iu;
-        // f_z is affine in the row: f_z(iv) = f_z(0) + iv dfz, with f_z(0) the
-        // forward's crossing of detector row 0 (so a ray's value does not
-        // depend on the run that evaluates it; within a few 1e-5 voxel of the
-        // forward's own FP32 value)
-        const RayZ rzb = ray_z(c, det_v(0, d), d.cz);
-        const float fzb = __fmaf_rn(tk, rzb.bz, rzb.fz_mid);
-        const float dfz = d.dv * __fmaf_rn(tk, c.inv_dmaj, c.c1);   // > 0
-        // rows in [iva, ivb) have both z taps inside the run (f_z in
-        // [iz_lo + 0.01, iz_lo + ZB - 1.01]); the others are checked
-        const float rdfz = __fdividef(1.0f, dfz);
-        const int iva = min(max((int)ceilf(((float)iz_lo + 0.01f - fzb) * rdfz), iv_lo), iv_hi + 1);
-        const int ivb = min(max((int)floorf(((float)(iz_lo + ZB) - 1.01f - fzb) * rdfz) + 1, iva), iv_hi + 1);
-        // explicit roundings: both loops must form a row's terms identically
-        auto checked = [&](int iv) {
-            const float fz = __fmaf_rn((float)iv, dfz, fzb);
-            const float z0f = floorf(fz);
-            const int k0 = (int)z0f - iz_lo;
-            if (k0 < -1 || k0 >= ZB) return;
-            const float ev = __fmul_rn(wa, __ldg(erow + (size_t)iv * d.nu));
-            const float c1 = __fmul_rn(__fsub_rn(fz, z0f), ev);
-            if (k0 >= 0) acc[k0][tid] = __fadd_rn(acc[k0][tid], __fsub_rn(ev, c1));
-            if (k0 + 1 < ZB) acc[k0 + 1][tid] = __fadd_rn(acc[k0 + 1][tid], c1);
-        };
-        for (int iv = iv_lo; iv < iva; ++iv) checked(iv);
-        for (int iv = iva; iv < ivb; ++iv) {
-            const float fz = __fmaf_rn((float)iv, dfz, fzb);
-            const float z0f = floorf(fz);
-            const int k0 = min(max((int)z0f - iz_lo, 0), ZB - 2);   // in range by the choice of [iva, ivb)
-            const float ev = __fmul_rn(wa, __ldg(erow + (size_t)iv * d.nu));
-            const float c1 = __fmul_rn(__fsub_rn(fz, z0f), ev);
-            acc[k0][tid] = __fadd_rn(acc[k0][tid], __fsub_rn(ev, c1));
-            acc[k0 + 1][tid] = __fadd_rn(acc[k0 + 1][tid], c1);
+    const V m = vadd_rd(t, L::all(FLOOR_MAGIC));
+    const V iv = vsub(m, L::all(FLOOR_MAGIC));
+    V df = vfma(vsub(iv, L::all(d.cv)), dfz, zc);
+    L::unpack(m, lo);
+    V s = L::all(0.0f);
+    const int n = NR ? NR : rows;
+#pragma unroll(NR ? NR : 1)
+    for (int i = 0; i < n; ++i) {
+        float dd[L::N];
+        L::unpack(df, dd);
+#pragma unroll
+        for (int k = 0; k < L::N; ++k) {
+            const int row = __float_as_int(lo[k]) + i;
+            w[k] = __saturatef(__fsub_rn(1.0f, fabsf(dd[k])));
+            if (NR) ev[k] = __ldg(q.row0 + row);
+            else ev[k] = (unsigned)(row - FLOOR_MAGIC_BITS) < (unsigned)d.nv ? __ldg(q.row0 + row) : 0.0f;
+            if (i == n - 1 || !NR) ev[k] = w[k] > 0.0f ? ev[k] : 0.0f;
         }
-        for (int iv = ivb; iv <= iv_hi; ++iv) checked(iv);
+        s = vfma(L::pack(w), L::pack(ev), s);
+        if (i + 1 < n) df = vadd(df, dfz);
+    }
+    return s;
+}
+
+// The gather's sums of J voxels per lane: J / 2 pairs, and one alone if J is odd.
+template <int J>
+struct AdjAcc {
+    f32x2 p[J / 2 + 1];
+    float o;
+    __device__ __forceinline__ void zero() {
+#pragma unroll
+        for (int j = 0; j < J / 2; ++j) p[j] = 0;
+        o = 0.0f;
+    }
+    __device__ __forceinline__ void add(float2 w, const AdjAcc& s) {
+#pragma unroll
+        for (int j = 0; j < J / 2; ++j) p[j] = fma2(pack2(w.x, w.y), s.p[j], p[j]);
+        if (J & 1) o = __fmaf_rn(w.x, s.o, o);
+    }
+    __device__ __forceinline__ void get(float* v) const {
+#pragma unroll
+        for (int j = 0; j < J / 2; ++j) unpack2(p[j], v[2 * j], v[2 * j + 1]);
+        if (J & 1) v[J - 1] = o;
+    }
+    __device__ __forceinline__ void set(const float* v) {
+#pragma unroll
+        for (int j = 0; j < J / 2; ++j) p[j] = pack2(v[2 * j], v[2 * j + 1]);
+        if (J & 1) o = v[J - 1];
+    }
+};
+
+template <int NR, bool CLAMP, int J>
+__device__ __forceinline__ void row_sums(const AdjEntry& q, int rows, const AdjAcc<J>& zc, const ProjDims& d,
+                                         AdjAcc<J>& s) {
+#pragma unroll
+    for (int j = 0; j < J / 2; ++j) s.p[j] = row_sum<NR, CLAMP, f32x2>(q, rows, zc.p[j], d);
+    if (J & 1) s.o = row_sum<NR, CLAMP, float>(q, rows, zc.o, d);
+}
+
+// Adds to the ADJ_T voxel lines a_lo .. a_lo + ADJ_T - 1 of plane kpl (x for
+// x-major rays, else y) the terms of every ray whose major axis is XMAJ.
+//
+// A column's ray plane crosses the voxel plane at f_a between the lines a0 and
+// a0 + 1, to which it adds (1 - w_a) s and w_a s with the same sums s over its
+// rows.  The lanes first build a list: `slots` columns of 32 / slots views at a
+// time (adj_slots: about as many as a run has), those that the projection of the
+// run's ends brackets (with a margin far above that projection's rounding) and
+// whose f_a, formed with the forward's own operations (bit for bit), touches the
+// run.  The warp then walks the list, its lanes taking voxels along z.  The order
+// of a voxel's terms (groups of views, columns in each) does not depend on J.
+template <bool XMAJ, int J>
+__device__ __forceinline__ void gather_run(const float4* __restrict__ col, const float2* __restrict__ trig,
+                                           const int* __restrict__ vflag, const float* __restrict__ e, int t, int kpl,
+                                           int a_lo, int z_lo, const AdjAcc<J>& zc, const ProjDims& d, int slots,
+                                           AdjEntry* __restrict__ list, int* __restrict__ slot, AdjAcc<J>* acc) {
+    const int lane = threadIdx.x;
+    const int na = XMAJ ? d.ny : d.nx, nvp = sino_pitch(d.nv);
+    const int a_hi = min(a_lo + ADJ_T, na);
+    const float tk = __fsub_rn((float)kpl, XMAJ ? d.cx : d.cy);
+    const float maj = tk * d.vox, lo = (a_lo - 1 - (XMAJ ? d.cy : d.cx)) * d.vox, hi = (a_hi - (XMAJ ? d.cy : d.cx)) * d.vox;
+    const float margin = 0.01f + 4e-6f * d.nu;
+    const int vstep = 32 / slots, vi = lane / slots, ci = lane - vi * slots;
+    for (int v0 = 0; v0 < d.views; v0 += vstep) {
+        const int v = v0 + vi, g = t * d.views + v;
+        int iu = d.nu, iu_hi = -1, flags = 0;
+        if (vi < vstep && v < d.views) flags = __ldg(vflag + g);
+        if (flags & (XMAJ ? 1 : 2)) {
+            const float2 cs = __ldg(trig + g);
+            const float x1 = XMAJ ? maj : lo, y1 = XMAJ ? lo : maj, x2 = XMAJ ? maj : hi, y2 = XMAJ ? hi : maj;
+            // an end beside the source projects anywhere: try every column
+            const bool near = fminf(d.dso - x1 * cs.x - y1 * cs.y, d.dso - x2 * cs.x - y2 * cs.y) < 0.05f * d.dso;
+            const float u1 = u_pixel(x1, y1, cs.x, cs.y, d), u2 = u_pixel(x2, y2, cs.x, cs.y, d);
+            iu = (near ? 0 : max(0, (int)ceilf(fminf(u1, u2) - margin))) + ci;
+            iu_hi = near ? d.nu - 1 : min(d.nu - 1, (int)floorf(fmaxf(u1, u2) + margin));
+        }
+        while (__any_sync(0xffffffffu, iu <= iu_hi)) {
+            bool ok = iu <= iu_hi;
+            AdjEntry q;
+            int al = 0, fast = 0;
+            if (ok) {
+                const size_t gcol = (size_t)g * d.nu + iu;
+                const float4 c = __ldg(col + 2 * gcol);   // fa_mid, ba, c1, inv_dmaj
+                if (flags == 3) ok = (__ldg(col + 2 * gcol + 1).z != 0.0f) == XMAJ;
+                const float fa = __fmaf_rn(tk, c.y, c.x);
+                const float a0f = floorf(fa);
+                const float wa = __fsub_rn(fa, a0f), wb = __fsub_rn(1.0f, wa);
+                al = (int)a0f - a_lo;
+                ok = ok && al >= -1 && al < ADJ_T;
+                const float dfz = d.dv * __fmaf_rn(tk, c.w, c.z), rdfz = __fdividef(1.0f, dfz);
+                const float c0 = d.cv + 1.0f - rdfz;
+                q.dfz = make_float2(dfz, dfz);
+                q.nrdfz = make_float2(-rdfz, -rdfz);
+                q.c0 = make_float2(c0, c0);
+                q.wa = make_float2(wa, wa);
+                q.wb = make_float2(wb, wb);
+                q.row0 = e + gcol * nvp + SINO_FRONT - FLOOR_MAGIC_BITS;
+                // two rows per footprint (1 <= dfz < 2) and every window of the
+                // run inside the line's margins
+                const float t_lo = __fmaf_rn(d.cz - (float)z_lo, -rdfz, c0);
+                const float t_hi = __fmaf_rn(d.cz - (float)(z_lo + 32 * J - 1), -rdfz, c0);
+                if (rdfz <= 1.0f && rdfz > 0.5f && t_lo > 1.0f - SINO_FRONT && t_hi < (float)(d.nv + SINO_BACK - 3))
+                    fast = ADJ_FAST;
+            }
+            const unsigned mask = __ballot_sync(0xffffffffu, ok);
+            if (ok) {
+                const int at = __popc(mask & ((1u << lane) - 1));
+                list[at] = q;
+                slot[at] = (al & 7) | fast;
+            }
+            __syncwarp();
+            const int n = __popc(mask);
+            for (int i = 0; i < n; ++i) {
+                const AdjEntry q = list[i];
+                const int sl = slot[i];
+                AdjAcc<J> s;
+                if (sl >= ADJ_FAST) row_sums<2, false, J>(q, 0, zc, d, s);
+                else {
+                    const float span = -2.0f * q.nrdfz.x;   // rows per footprint: ceil(2 / dfz)
+                    if (span <= 1.0f) row_sums<1, true, J>(q, 0, zc, d, s);
+                    else if (span <= 2.0f) row_sums<2, true, J>(q, 0, zc, d, s);
+                    else if (span <= 3.0f) row_sums<3, true, J>(q, 0, zc, d, s);
+                    else row_sums<0, true, J>(q, (int)fminf(ceilf(span), (float)(d.nv + 8)), zc, d, s);
+                }
+                switch (sl & 7) {
+                    case 7: acc[0].add(q.wa, s); break;   // -1: the line before the run
+                    case 0: acc[0].add(q.wb, s); acc[1].add(q.wa, s); break;
+                    case 1: acc[1].add(q.wb, s); acc[2].add(q.wa, s); break;
+                    case 2: acc[2].add(q.wb, s); acc[3].add(q.wa, s); break;
+                    default: acc[3].add(q.wb, s); break;
+                }
+            }
+            __syncwarp();
+            iu += slots;
+        }
     }
 }
 
-// One thread per run of ZB voxels along z; block 32 (x) x 4 (y).
-// e is the step-weighted sinogram e' = step * e.
+// Blocks per SM that the register limit asks for: as measured fastest for each J
+// (384^3 x 2, J = 12: 1.81 ms with 4, 1.99 with 5, 2.47 with no limit; J = 6: 2.00
+// with 5, 2.22 with none; 128^3 x 8, J = 4: 0.67 with 6, 0.73 with none).
+__host__ __device__ constexpr int adj_min_blocks(int J) { return J >= 8 ? 4 : J >= 5 ? 5 : J >= 3 ? 6 : 8; }
+
+// A block takes ADJ_T x ADJ_T voxel lines and 32 J voxels of each; lane = z, so
+// that a warp's loads run along the detector rows.  First warp w takes the lines
+// of x = x0 + w for the x-major rays, then, the sums handed over through shared
+// memory, those of y = y0 + w for the y-major rays: either way a column's sums
+// over its rows, most of the work, serve both lines beside its crossing, and no
+// sum is read back per ray.  Bound by instruction issue: about 14 instructions
+// per (column, voxel along z), and some 40 per column that J voxels per lane
+// share (packed pairs, the list, the choice of the two lines).  A thread per run
+// of voxels that added each row's two terms into shared memory visited every
+// crossing twice: A^T at 384^3 x 16, 512 x 384, 24 views 41.6 -> 14.3 ms (J = 12;
+// J = 4: 18.5), 128^3 x 8, 192 x 160, 32 views in a 90 degree wedge 1.59 -> 0.63
+// ms, 24^3 x 4, 32 x 32, 12 views 85 -> 30 us.  Tiles of 8 x 8 lines with J = 4
+// need fewer columns per line (0.79 against 0.88) but took 20 ms.
+// e is the step-weighted sinogram e' = step * e in lines of rows.
 //   ADJ_PLAIN:   out = A^T e
 //   ADJ_CG_INIT: r = A^T e + (v - z)/sigma^2, p = r, partial sum r.r
 //   ADJ_CG_Q:    q = A^T e + p/sigma^2, partial sum p.q
-// (at most 64 registers: eight blocks per SM, no spills)
-template <int MODE, int ZB>
-__global__ void __launch_bounds__(128, 8) joseph_adj_kernel(
+template <int MODE, int J>
+__global__ void __launch_bounds__(32 * ADJ_T, adj_min_blocks(J)) joseph_adj_kernel(
     const float4* __restrict__ col, const float2* __restrict__ trig, const int* __restrict__ vflag,
     const float* __restrict__ e, float* __restrict__ out, const float* __restrict__ a1,
     const float* __restrict__ a2, float* __restrict__ out2, double* __restrict__ partial,
-    float inv_s2, ProjDims d) {
-    __shared__ float acc[ZB][128];
-    const int tid = threadIdx.y * 32 + threadIdx.x;
-    const int ix = blockIdx.x * 32 + threadIdx.x;
-    const int iy = blockIdx.y * 4 + threadIdx.y;
-    const int nzb = (d.nz + ZB - 1) / ZB;
-    const int zb = blockIdx.z % nzb;
-    const int t = blockIdx.z / nzb;
-    const int iz_lo = zb * ZB;
-    const bool inside = ix < d.nx && iy < d.ny;
+    float inv_s2, ProjDims d, int slots) {
+    extern __shared__ float adj_tile[];   // [y][x][adj_line(J)]
+    __shared__ AdjEntry list[ADJ_T][ADJ_ENTRIES];
+    __shared__ int slot[ADJ_T][ADJ_ENTRIES];
+    const int lane = threadIdx.x, w = threadIdx.y;
+    const int nzb = (d.nz + 32 * J - 1) / (32 * J);
+    const int zb = blockIdx.z % nzb, t = blockIdx.z / nzb;
+    const int x0 = blockIdx.x * ADJ_T, y0 = blockIdx.y * ADJ_T, z0 = zb * 32 * J + lane;
+    AdjAcc<J> acc[ADJ_T], zc;
+    {
+        float a[J];
 #pragma unroll
-    for (int k = 0; k < ZB; ++k) acc[k][tid] = 0.0f;
-    if (inside) {
-        for (int j = 0; j < d.views; ++j) {
-            const int g = t * d.views + j;
-            const float2 cs = __ldg(trig + g);
-            const int fl = __ldg(vflag + g);
-            if (fl & 1) gather_runs<true, ZB>(col, e, g, ix, iy, iz_lo, cs.x, cs.y, d, acc, tid);
-            if (fl & 2) gather_runs<false, ZB>(col, e, g, ix, iy, iz_lo, cs.x, cs.y, d, acc, tid);
-        }
+        for (int j = 0; j < J; ++j) a[j] = d.cz - (float)(z0 + 32 * j);
+        zc.set(a);
     }
+#pragma unroll
+    for (int i = 0; i < ADJ_T; ++i) acc[i].zero();
+    if (x0 + w < d.nx)
+        gather_run<true, J>(col, trig, vflag, e, t, x0 + w, y0, zb * 32 * J, zc, d, slots, list[w], slot[w], acc);
+#pragma unroll
+    for (int i = 0; i < ADJ_T; ++i) {
+        float v[J];
+        acc[i].get(v);
+#pragma unroll
+        for (int j = 0; j < J; ++j) adj_tile[(i * ADJ_T + w) * adj_line(J) + 32 * j + lane] = v[j];
+    }
+    __syncthreads();
+    float* tile = adj_tile + w * ADJ_T * adj_line(J);   // the lines of y = y0 + w
+#pragma unroll
+    for (int i = 0; i < ADJ_T; ++i) {
+        float v[J];
+#pragma unroll
+        for (int j = 0; j < J; ++j) v[j] = tile[i * adj_line(J) + 32 * j + lane];
+        acc[i].set(v);
+    }
+    const int iy = y0 + w;
     double dot = 0.0;
-    for (int k = 0; k < ZB; ++k) {
-        const int iz = iz_lo + k;
-        if (!inside || iz >= d.nz) break;
-        const size_t i = (((size_t)t * d.nz + iz) * d.ny + iy) * d.nx + ix;
-        const float s = acc[k][tid];
-        if (MODE == ADJ_PLAIN) {
-            out[i] = s;
-        } else if (MODE == ADJ_CG_INIT) {   // a1 = v, a2 = z
-            const float r = s + (a1[i] - a2[i]) * inv_s2;
-            out[i] = r;
-            out2[i] = r;
-            dot += (double)r * (double)r;
-        } else {                            // a1 = p
-            const float p = a1[i];
-            const float q = s + p * inv_s2;
-            out[i] = q;
-            dot += (double)p * (double)q;
+    if (iy < d.ny) {
+        gather_run<false, J>(col, trig, vflag, e, t, iy, x0, zb * 32 * J, zc, d, slots, list[w], slot[w], acc);
+        // the volume is contiguous along x: ADJ_T lanes write the x of one z
+#pragma unroll
+        for (int i = 0; i < ADJ_T; ++i) {
+            float v[J];
+            acc[i].get(v);
+#pragma unroll
+            for (int j = 0; j < J; ++j) tile[i * adj_line(J) + 32 * j + lane] = v[j];
+        }
+        __syncwarp();
+        const int ix = x0 + lane % ADJ_T;
+#pragma unroll 4
+        for (int k = lane / ADJ_T; k < 32 * J; k += 32 / ADJ_T) {
+            const int iz = zb * 32 * J + k;
+            if (ix >= d.nx || iz >= d.nz) break;
+            const size_t i = (((size_t)t * d.nz + iz) * d.ny + iy) * d.nx + ix;
+            const float s = tile[(lane % ADJ_T) * adj_line(J) + k];
+            if (MODE == ADJ_PLAIN) {
+                out[i] = s;
+            } else if (MODE == ADJ_CG_INIT) {   // a1 = v, a2 = z
+                const float r = s + (a1[i] - a2[i]) * inv_s2;
+                out[i] = r;
+                out2[i] = r;
+                dot += (double)r * (double)r;
+            } else {                            // a1 = p
+                const float p = a1[i];
+                const float q = s + p * inv_s2;
+                out[i] = q;
+                dot += (double)p * (double)q;
+            }
         }
     }
     if (MODE != ADJ_PLAIN) {
         const double sum = block_sum_f64(dot);
-        if (tid == 0) {
+        if (lane == 0 && w == 0) {
             const int bpf = gridDim.x * gridDim.y * nzb;   // blocks per frame
             const int b = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * zb);
             partial[(size_t)t * bpf + b] = sum;
@@ -543,17 +732,23 @@ __global__ void __launch_bounds__(128, 8) joseph_adj_kernel(
     }
 }
 
-// e' = step * e for every ray (input of the gather for a plain A^T).
+// e' = step * e for every ray, into lines of rows (the gather's input), through
+// 32 x 32 tiles of one view.
 __global__ void step_weight_kernel(const float4* __restrict__ col, const float* __restrict__ e,
                                    float* __restrict__ out, ProjDims d) {
-    const int iu = blockIdx.x * 32 + threadIdx.x;
-    const int iv = blockIdx.y * 4 + threadIdx.y;
-    const int g = blockIdx.z;
-    if (iu >= d.nu || iv >= d.nv) return;
-    const ColParams c = load_col(col, (size_t)g * d.nu + iu);
-    const RayZ rz = ray_z(c, det_v(iv, d), d.cz);
-    const size_t ray = ((size_t)g * d.nv + iv) * d.nu + iu;
-    out[ray] = rz.step * e[ray];
+    __shared__ float tile[32][33];
+    const int g = blockIdx.x, u0 = blockIdx.y * 32, v0 = blockIdx.z * 32;
+    const int iu = u0 + threadIdx.x;
+    if (iu < d.nu) {
+        const ColParams c = load_col(col, (size_t)g * d.nu + iu);
+        for (int k = threadIdx.y; k < 32 && v0 + k < d.nv; k += blockDim.y)
+            tile[k][threadIdx.x] = ray_z(c, det_v(v0 + k, d), d.cz).step * e[((size_t)g * d.nv + v0 + k) * d.nu + iu];
+    }
+    __syncthreads();
+    const int iv = v0 + threadIdx.x;
+    if (iv >= d.nv) return;
+    for (int k = threadIdx.y; k < 32 && u0 + k < d.nu; k += blockDim.y)
+        out[((size_t)g * d.nu + u0 + k) * sino_pitch(d.nv) + SINO_FRONT + iv] = tile[threadIdx.x][k];
 }
 
 // ------------------------------------------------------------------ CG scalars
@@ -961,7 +1156,7 @@ struct msf_projector {
     float* d_zero = nullptr;   // one line of zeros
     float* d_sw = nullptr;     // step-weighted sinogram for msf_backproject
     int fwd_bx = 32, fwd_by = 4;   // forward launch shape (fwd_cols_of: detector columns per block)
-    int adj_zb = 16;               // gather z-run length
+    int adj_zb = 64;               // gather z-run (adj_j: voxels per lane)
     uint64_t tuning_gen = 0;       // advanced whenever the launch shapes change
     size_t bytes = 0;
 };
@@ -969,6 +1164,7 @@ struct msf_projector {
 struct msf_dataprox {
     msf_projector* p = nullptr;
     float *d_r = nullptr, *d_p = nullptr, *d_p2 = nullptr, *d_q = nullptr, *d_s = nullptr;
+    float* d_rows = nullptr;   // step-weighted sinogram in lines of rows
     double *d_partial = nullptr, *d_rr = nullptr, *d_alpha = nullptr, *d_beta = nullptr;
     int* d_status = nullptr;
     int parts_adj = 0, parts_upd = 0, parts_max = 0;
@@ -983,6 +1179,9 @@ namespace msf {
 
 static size_t frame_size(const msf_vol& v) { return (size_t)v.nx * v.ny * v.nz; }
 static size_t vol_size(const msf_vol& v) { return frame_size(v) * v.nt; }
+static size_t rows_size(const msf_projector* p) {   // a sinogram in lines of rows
+    return (size_t)p->vol.nt * p->geom.views * p->geom.nu * sino_pitch(p->geom.nv);
+}
 static size_t sino_size(const msf_projector* p) {
     return (size_t)p->geom.nu * p->geom.nv * p->geom.views * p->vol.nt;
 }
@@ -997,7 +1196,7 @@ static msf_status launch_lines(msf_projector* p, const float* in, cudaStream_t s
     return MSF_OK;
 }
 
-template <int MODE, bool PAR>
+template <int MODE, bool PAR, bool ROWS>
 static void launch_fwd_kernel(msf_projector* p, const float* vz, float* out, const float* lam, const float* meas,
                               int kpx, int kpy, cudaStream_t st) {
     const ProjDims& d = p->dims;
@@ -1009,7 +1208,7 @@ static void launch_fwd_kernel(msf_projector* p, const float* vz, float* out, con
     const size_t smem = (size_t)32 * R * (ncol + 1) * sizeof(float);
 #define MSF_FWD_CASE(N)                                                                                            \
     case N:                                                                                                        \
-        joseph_fwd_kernel<MODE, N, PAR><<<grid, block, smem, st>>>(vz, p->d_zero, p->d_col, out, lam, meas, d,     \
+        joseph_fwd_kernel<MODE, N, PAR, ROWS><<<grid, block, smem, st>>>(vz, p->d_zero, p->d_col, out, lam, meas, d,     \
                                                                     kpx, kpy);                                     \
         break;
     switch (R) {
@@ -1022,24 +1221,22 @@ static void launch_fwd_kernel(msf_projector* p, const float* vz, float* out, con
 #undef MSF_FWD_CASE
 }
 
-// A of the volume whose lines are vz.
-static msf_status launch_fwd_lines(msf_projector* p, int mode, const float* vz, float* out, const float* lam,
-                                   const float* meas, cudaStream_t st) {
+// A of the volume whose lines are vz (MODE), written as a sinogram or, ROWS, as
+// lines of rows.
+template <int MODE, bool ROWS>
+static msf_status launch_fwd_lines(msf_projector* p, const float* vz, float* out, const float* lam, const float* meas,
+                                   cudaStream_t st) {
     MSF_PROF("joseph_fwd", st);
-    if (mode == FWD_PLAIN)
-        launch_fwd_kernel<FWD_PLAIN, false>(p, vz, out, lam, meas, 0, 0, st);
-    else if (mode == FWD_LAMBDA)
-        launch_fwd_kernel<FWD_LAMBDA, false>(p, vz, out, lam, meas, 0, 0, st);
-    else
-        launch_fwd_kernel<FWD_RESIDUAL, false>(p, vz, out, lam, meas, 0, 0, st);
+    launch_fwd_kernel<MODE, false, ROWS>(p, vz, out, lam, meas, 0, 0, st);
     MSF_LAUNCH_CHECK();
     return MSF_OK;
 }
 
-static msf_status launch_fwd(msf_projector* p, int mode, const float* x, float* out,
-                             const float* lam, const float* meas, cudaStream_t st) {
+template <int MODE, bool ROWS>
+static msf_status launch_fwd(msf_projector* p, const float* x, float* out, const float* lam, const float* meas,
+                             cudaStream_t st) {
     MSF_TRY(launch_lines(p, x, st));
-    return launch_fwd_lines(p, mode, p->d_vz, out, lam, meas, st);
+    return launch_fwd_lines<MODE, ROWS>(p, p->d_vz, out, lam, meas, st);
 }
 
 // A x for an x that is zero outside the voxels with x = kpx and y = kpy (mod 2)
@@ -1047,13 +1244,32 @@ static msf_status launch_fwd(msf_projector* p, int mode, const float* x, float* 
 static msf_status launch_fwd_parity(msf_projector* p, const float* x, float* out, int kpx, int kpy, cudaStream_t st) {
     MSF_TRY(launch_lines(p, x, st));
     MSF_PROF("joseph_fwd", st);
-    launch_fwd_kernel<FWD_PLAIN, true>(p, p->d_vz, out, nullptr, nullptr, kpx, kpy, st);
+    launch_fwd_kernel<FWD_PLAIN, true, false>(p, p->d_vz, out, nullptr, nullptr, kpx, kpy, st);
     MSF_LAUNCH_CHECK();
     return MSF_OK;
 }
 
-static int adj_nzb(const ProjDims& d, int zb) { return (d.nz + zb - 1) / zb; }
-static dim3 adj_grid(const ProjDims& d, int zb) { return dim3((d.nx + 31) / 32, (d.ny + 3) / 4, adj_nzb(d, zb) * d.nt); }
+// Voxels per lane (J) of an adjoint launch: the plan's z-run allows at most 2 (8),
+// 4 (16), 6 (32) or 12 (64); a line's sets of 32 voxels are split evenly over as
+// few blocks as that allows (J above 6 is rounded up to an even number).
+static int adj_j(const ProjDims& d, int zrun) {
+    const int cap = zrun == 8 ? 2 : zrun == 16 ? 4 : zrun == 32 ? 6 : 12;
+    const int sets = (d.nz + 31) / 32, blocks = (sets + cap - 1) / cap;
+    const int J = (sets + blocks - 1) / blocks;
+    return J <= 6 ? J : (J + 1) & ~1;
+}
+// Columns that a run of ADJ_T lines has on the axis, and one more.
+static int adj_slots(const ProjDims& d) {
+    const double n = ceil((ADJ_T + 1) * (double)d.vox * d.dsd / d.dso / d.du) + 1.0;
+    return n < 2.0 ? 2 : n > 32.0 ? 32 : (int)n;
+}
+static int adj_nzb(const ProjDims& d, int zrun) {
+    const int run = 32 * adj_j(d, zrun);
+    return (d.nz + run - 1) / run;
+}
+static dim3 adj_grid(const ProjDims& d, int zrun) {
+    return dim3((d.nx + ADJ_T - 1) / ADJ_T, (d.ny + ADJ_T - 1) / ADJ_T, adj_nzb(d, zrun) * d.nt);
+}
 // partial sums per frame of an adjoint launch
 static int adj_parts(const msf_projector* p) {
     const dim3 g = adj_grid(p->dims, p->adj_zb);
@@ -1064,15 +1280,26 @@ template <int MODE>
 static void launch_adj_zb(msf_projector* p, const float* e, float* out, const float* a1, const float* a2,
                           float* out2, double* partial, float inv_s2, cudaStream_t st) {
     const ProjDims& d = p->dims;
-    const dim3 block(32, 4), grid = adj_grid(d, p->adj_zb);
-    if (p->adj_zb == 8)
-        joseph_adj_kernel<MODE, 8><<<grid, block, 0, st>>>(p->d_col, p->d_trig, p->d_vflag, e, out, a1, a2, out2, partial, inv_s2, d);
-    else if (p->adj_zb == 32)
-        joseph_adj_kernel<MODE, 32><<<grid, block, 0, st>>>(p->d_col, p->d_trig, p->d_vflag, e, out, a1, a2, out2, partial, inv_s2, d);
-    else if (p->adj_zb == 64)
-        joseph_adj_kernel<MODE, 64><<<grid, block, 0, st>>>(p->d_col, p->d_trig, p->d_vflag, e, out, a1, a2, out2, partial, inv_s2, d);
-    else
-        joseph_adj_kernel<MODE, 16><<<grid, block, 0, st>>>(p->d_col, p->d_trig, p->d_vflag, e, out, a1, a2, out2, partial, inv_s2, d);
+    const int J = adj_j(d, p->adj_zb), slots = adj_slots(d);
+    const dim3 block(32, ADJ_T), grid = adj_grid(d, p->adj_zb);
+    const size_t smem = (size_t)ADJ_T * ADJ_T * adj_line(J) * sizeof(float);
+#define MSF_ADJ_CASE(N)                                                                                             \
+    case N:                                                                                                         \
+        joseph_adj_kernel<MODE, N><<<grid, block, smem, st>>>(p->d_col, p->d_trig, p->d_vflag, e, out, a1, a2, out2, \
+                                                               partial, inv_s2, d, slots);                          \
+        break;
+    switch (J) {
+        MSF_ADJ_CASE(1)
+        MSF_ADJ_CASE(2)
+        MSF_ADJ_CASE(3)
+        MSF_ADJ_CASE(4)
+        MSF_ADJ_CASE(5)
+        MSF_ADJ_CASE(6)
+        MSF_ADJ_CASE(8)
+        MSF_ADJ_CASE(10)
+        MSF_ADJ_CASE(12)
+    }
+#undef MSF_ADJ_CASE
 }
 
 static msf_status launch_adj(msf_projector* p, int mode, const float* e, float* out,
@@ -1144,12 +1371,12 @@ extern "C" msf_status msf_projector_create(const msf_geom* geom, const msf_vol* 
         cudaMalloc(&p->d_trig, G * sizeof(float2)) != cudaSuccess ||
         cudaMalloc(&p->d_vflag, G * sizeof(int)) != cudaSuccess ||
         cudaMalloc(&p->d_vz, vz_bytes) != cudaSuccess || cudaMalloc(&p->d_zero, line_bytes) != cudaSuccess ||
-        cudaMalloc(&p->d_sw, sino_size(p) * sizeof(float)) != cudaSuccess) {
+        cudaMalloc(&p->d_sw, rows_size(p) * sizeof(float)) != cudaSuccess) {
         cudaGetLastError();
         return cleanup(fail(MSF_ERR_NOMEM, "msf_projector_create: out of device memory"));
     }
     p->bytes = G * sizeof(double) + col_bytes + G * (sizeof(float2) + sizeof(int)) + vz_bytes + line_bytes +
-               sino_size(p) * sizeof(float);
+               rows_size(p) * sizeof(float);
     std::vector<float2> trig(G);
     for (int g = 0; g < G; ++g) trig[g] = make_float2((float)cos(p->angles[g]), (float)sin(p->angles[g]));
     int* d_bad = nullptr;
@@ -1159,6 +1386,7 @@ extern "C" msf_status msf_projector_create(const msf_geom* geom, const msf_vol* 
     if (e == cudaSuccess) e = cudaMemset(p->d_vflag, 0, G * sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(p->d_vz, 0, vz_bytes);
     if (e == cudaSuccess) e = cudaMemset(p->d_zero, 0, line_bytes);
+    if (e == cudaSuccess) e = cudaMemset(p->d_sw, 0, rows_size(p) * sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc(&d_bad, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(d_bad, 0, sizeof(int));
     if (e == cudaSuccess) {
@@ -1191,7 +1419,7 @@ extern "C" size_t msf_projector_bytes(const msf_projector* p) { return p ? p->by
 
 extern "C" msf_status msf_project(msf_projector* p, const float* d_x, float* d_y, void* stream) {
     MSF_REQUIRE(p && d_x && d_y, "msf_project: NULL argument");
-    return launch_fwd(p, FWD_PLAIN, d_x, d_y, nullptr, nullptr, as_stream(stream));
+    return launch_fwd<FWD_PLAIN, false>(p, d_x, d_y, nullptr, nullptr, as_stream(stream));
 }
 
 extern "C" msf_status msf_backproject(msf_projector* p, const float* d_y, float* d_x, void* stream) {
@@ -1200,7 +1428,7 @@ extern "C" msf_status msf_backproject(msf_projector* p, const float* d_y, float*
     {
         const ProjDims& d = p->dims;
         MSF_PROF("step_weight", st);
-        step_weight_kernel<<<dim3((d.nu + 31) / 32, (d.nv + 3) / 4, d.nt * d.views), dim3(32, 4), 0, st>>>(
+        step_weight_kernel<<<dim3(d.nt * d.views, (d.nu + 31) / 32, (d.nv + 31) / 32), dim3(32, 8), 0, st>>>(
             p->d_col, d_y, p->d_sw, d);
         MSF_LAUNCH_CHECK();
     }
@@ -1223,7 +1451,7 @@ extern "C" msf_status msf_dataprox_create(msf_projector* p, msf_dataprox** out) 
         d->parts_icd = ((par_count(v.nx, 0) + 31) / 32) * ((par_count(v.ny, 0) + 3) / 4) *
                        ((par_count(v.nz, 0) + ICD_ZB - 1) / ICD_ZB);
     }
-    if (cudaMalloc(&d->d_s2, ns * 4) != cudaSuccess ||
+    if (cudaMalloc(&d->d_s2, ns * 4) != cudaSuccess || cudaMalloc(&d->d_rows, rows_size(p) * 4) != cudaSuccess ||
         cudaMalloc(&d->d_ipart, (size_t)nt * d->parts_icd * 2 * 8) != cudaSuccess ||
         cudaMalloc(&d->d_spart, (size_t)nt * ICD_SINO_BLOCKS * 8) != cudaSuccess ||
         cudaMalloc(&d->d_r, nv * 4) != cudaSuccess || cudaMalloc(&d->d_p, nv * 4) != cudaSuccess ||
@@ -1236,7 +1464,8 @@ extern "C" msf_status msf_dataprox_create(msf_projector* p, msf_dataprox** out) 
         msf_dataprox_destroy(d);
         return fail(MSF_ERR_NOMEM, "msf_dataprox_create: out of device memory");
     }
-    if (cudaMemset(d->d_status, 0, sizeof(int)) != cudaSuccess) {
+    if (cudaMemset(d->d_status, 0, sizeof(int)) != cudaSuccess ||
+        cudaMemset(d->d_rows, 0, rows_size(p) * 4) != cudaSuccess) {
         msf_dataprox_destroy(d);
         return fail(MSF_ERR_CUDA, "msf_dataprox_create: memset failed");
     }
@@ -1249,7 +1478,7 @@ extern "C" void msf_dataprox_destroy(msf_dataprox* d) {
     cudaFree(d->d_r); cudaFree(d->d_p); cudaFree(d->d_p2); cudaFree(d->d_q); cudaFree(d->d_s);
     cudaFree(d->d_partial); cudaFree(d->d_rr); cudaFree(d->d_alpha); cudaFree(d->d_beta);
     cudaFree(d->d_status);
-    cudaFree(d->d_s2); cudaFree(d->d_ipart); cudaFree(d->d_spart);
+    cudaFree(d->d_s2); cudaFree(d->d_rows); cudaFree(d->d_ipart); cudaFree(d->d_spart);
     delete d;
 }
 
@@ -1265,8 +1494,8 @@ extern "C" msf_status msf_prox_data(msf_dataprox* dp, const float* d_y, const fl
     const int nt = p->vol.nt;
     const size_t fs = frame_size(p->vol);
     // r = A^T Lambda (y - A z) + (v - z)/sigma^2 ; p = r ; rr = r.r
-    MSF_TRY(launch_fwd(p, FWD_RESIDUAL, d_x, dp->d_s, d_lambda, d_y, st));
-    MSF_TRY(launch_adj(p, ADJ_CG_INIT, dp->d_s, dp->d_r, d_v, d_x, dp->d_p, dp->d_partial, inv_s2, st));
+    MSF_TRY((launch_fwd<FWD_RESIDUAL, true>(p, d_x, dp->d_rows, d_lambda, d_y, st)));
+    MSF_TRY(launch_adj(p, ADJ_CG_INIT, dp->d_rows, dp->d_r, d_v, d_x, dp->d_p, dp->d_partial, inv_s2, st));
     {
         MSF_PROF("cg_finalize", st);
         cg_finalize_kernel<FIN_RR0><<<nt, 256, 0, st>>>(dp->d_partial, adj_parts(p), dp->d_rr, nullptr, dp->d_status);
@@ -1288,9 +1517,9 @@ extern "C" msf_status msf_prox_data(msf_dataprox* dp, const float* d_y, const fl
             pc = pn;
         }
         // s = Lambda A p
-        MSF_TRY(launch_fwd_lines(p, FWD_LAMBDA, p->d_vz, dp->d_s, d_lambda, nullptr, st));
+        MSF_TRY((launch_fwd_lines<FWD_LAMBDA, true>(p, p->d_vz, dp->d_rows, d_lambda, nullptr, st)));
         // q = A^T s + p/sigma^2 ; alpha = rr / p.q
-        MSF_TRY(launch_adj(p, ADJ_CG_Q, dp->d_s, dp->d_q, pc, nullptr, nullptr, dp->d_partial, inv_s2, st));
+        MSF_TRY(launch_adj(p, ADJ_CG_Q, dp->d_rows, dp->d_q, pc, nullptr, nullptr, dp->d_partial, inv_s2, st));
         {
             MSF_PROF("cg_finalize", st);
             cg_finalize_kernel<FIN_ALPHA><<<nt, 256, 0, st>>>(dp->d_partial, adj_parts(p), dp->d_rr, dp->d_alpha, dp->d_status);
@@ -1323,7 +1552,7 @@ extern "C" msf_status msf_prox_data_icd(msf_dataprox* dp, const float* d_y, cons
     const int nt = v.nt;
     const float inv_s2 = (float)(1.0 / (sigma * sigma));
     // e' = step Lambda (y - A z)
-    MSF_TRY(launch_fwd(p, FWD_RESIDUAL, d_x, dp->d_s, d_lambda, d_y, st));
+    MSF_TRY((launch_fwd<FWD_RESIDUAL, false>(p, d_x, dp->d_s, d_lambda, d_y, st)));
     {   // theta2 = (A^T Lambda A)_ss + 1/sigma^2
         MSF_PROF("icd_step2", st);
         icd_step2_kernel<<<dim3((d.nu + 31) / 32, (d.nv + 3) / 4, d.nt * d.views), dim3(32, 4), 0, st>>>(
@@ -1619,14 +1848,14 @@ extern "C" msf_status msf_projector_autotune(msf_projector* p, void* stream, int
         cudaEventElapsedTime(&ms, e0, e1);
         return ms;
     };
-    MSF_TRY_CUDA(cudaMemsetAsync(p->d_sw, 0, ns * sizeof(float), st));
+    MSF_TRY_CUDA(cudaMemsetAsync(p->d_sw, 0, rows_size(p) * sizeof(float), st));
     const int shapes[3][2] = {{32, 4}, {64, 2}, {16, 8}};
     float best = 1e30f;
     int bi = 0;
     for (int i = 0; i < 3; ++i) {
         p->fwd_bx = shapes[i][0];
         p->fwd_by = shapes[i][1];
-        const float ms = time_it([&] { launch_fwd_kernel<FWD_PLAIN, false>(p, p->d_vz, tmp, nullptr, nullptr, 0, 0, st); });
+        const float ms = time_it([&] { launch_fwd_kernel<FWD_PLAIN, false, false>(p, p->d_vz, tmp, nullptr, nullptr, 0, 0, st); });
         if (ms < best) { best = ms; bi = i; }
     }
     p->fwd_bx = shapes[bi][0];

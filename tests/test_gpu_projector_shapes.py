@@ -64,3 +64,64 @@ def test_forward_equals_the_direct_kernel(M, shape, bad):
             assert torch.equal(torch.nan_to_num(y, 7.0), torch.nan_to_num(ref, 7.0)), (cols, rows)
     finally:
         L.msf_projector_destroy(h)
+
+
+def _oracle_At(y, geom, vol, ang):
+    """A^T in FP64: the oracle's scatter over the plan's own shape."""
+    import oracle
+    out = np.zeros((vol.nt, vol.nz, vol.ny, vol.nx))
+    for t in range(vol.nt):
+        a = np.ascontiguousarray(ang[t * geom.views:(t + 1) * geom.views])
+        oracle._L().or_project(oracle._p(out[t]), oracle._p(np.ascontiguousarray(y[t])), vol.nx, vol.ny, vol.nz, 1.0, geom.nu,
+                               geom.nv, geom.du, geom.dv, geom.dso, geom.dsd, oracle._p(a), geom.views, 1)
+    return out
+
+
+# detectors of fine rows (up to 16 rows per voxel), of coarse rows (several voxels per row) and of fine columns
+ADJ_SHAPES = SHAPES + [(12, 9, 33, 1, 20, 400, 3, 0.4), (15, 18, 96, 1, 25, 6, 4, 1.0), (13, 11, 40, 2, 250, 37, 3, 0.8)]
+
+
+@pytest.mark.parametrize("shape", ADJ_SHAPES, ids=lambda s: "x".join(map(str, s)))
+def test_adjoint_matches_oracle_at_ragged_sizes(M, shape):
+    import torch
+    geom, vol, ang = _geometry(M, *shape)
+    y = np.random.default_rng(6).standard_normal((vol.nt, geom.views, geom.nv, geom.nu)).astype(np.float32)
+    ref = _oracle_At(y.astype(np.float64), geom, vol, ang)
+    yg = torch.from_numpy(y).cuda()
+    L = M.lib()
+    h = ctypes.c_void_p()
+    assert L.msf_projector_create(ctypes.byref(geom), ctypes.byref(vol), ctypes.byref(h)) == 0, L.msf_last_error()
+    try:
+        first = None
+        for zrun in (8, 16, 32, 64):
+            assert L.msf_projector_set_tuning(h, 32, 4, zrun) == 0
+            x = torch.full((vol.nt, vol.nz, vol.ny, vol.nx), -1.0, device="cuda")
+            assert L.msf_backproject(h, yg.data_ptr(), x.data_ptr(), None) == 0
+            torch.cuda.synchronize()
+            got = x.cpu().numpy().astype(np.float64)
+            assert np.linalg.norm(got - ref) <= 1e-5 * np.linalg.norm(ref), zrun   # the projector's tolerance
+            first = x if first is None else first
+            assert torch.equal(x, first), zrun
+    finally:
+        L.msf_projector_destroy(h)
+
+
+def test_nonfinite_reading_reaches_its_own_footprint_only(M):
+    import torch
+    geom, vol, ang = _geometry(M, 20, 21, 30, 1, 24, 27, 4)
+    y = np.zeros((1, geom.views, geom.nv, geom.nu), np.float32)
+    y[0, 1, 13, 11] = 1.0
+    ref = _oracle_At(y.astype(np.float64), geom, vol, ang)
+    y[0, 1, 13, 11] = np.inf
+    L = M.lib()
+    h = ctypes.c_void_p()
+    assert L.msf_projector_create(ctypes.byref(geom), ctypes.byref(vol), ctypes.byref(h)) == 0, L.msf_last_error()
+    try:
+        x = torch.zeros((1, vol.nz, vol.ny, vol.nx), device="cuda")
+        assert L.msf_backproject(h, torch.from_numpy(y).cuda().data_ptr(), x.data_ptr(), None) == 0
+        torch.cuda.synchronize()
+        hit = ~np.isfinite(x.cpu().numpy())
+    finally:
+        L.msf_projector_destroy(h)
+    w = ref / ref.max()
+    assert hit[w > 1e-3].all() and not hit[w < -1e-9].any() and not (hit & (w == 0)).any()
