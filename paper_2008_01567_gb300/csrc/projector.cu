@@ -116,35 +116,72 @@ __global__ void column_table_kernel(const double* __restrict__ angles, float4* _
 constexpr int VZ_FRONT = 4;
 __host__ __device__ __forceinline__ int vz_pitch(int nz) { return (nz + VZ_FRONT + 2 + 7) & ~7; }
 
-// Copies [nt][nz][ny][nx] -> z-contiguous lines, through 32 x 32 shared tiles
-// of one (t, y) plane.  Bound by HBM (8 bytes per voxel).
-// FUSED: v = r + beta_t p (the CG direction update) with p = in; v is also
-// written to pnext.
-template <bool FUSED>
-__global__ void lines_kernel(const float* __restrict__ in, float* __restrict__ vz, const float* __restrict__ r,
-                             float* __restrict__ pnext, const double* __restrict__ beta, int nx, int ny, int nz) {
-    __shared__ float tile[32][33];
-    const int t = blockIdx.x / ny, y = blockIdx.x % ny;
-    const int x0 = blockIdx.y * 32, z0 = blockIdx.z * 32;
+// Transposes between a volume [nt][nz][ny][nx] and its lines, through 64 x 64
+// shared tiles of one (t, y) plane: 256-byte pieces on both sides, 16 loads per
+// thread in flight.  Bound by HBM.
+enum LinesMode { LINES_COPY = 0, LINES_PAIR = 1 };
+constexpr int LT = 64;
+
+// LINES_COPY: vz = lines of in.  LINES_PAIR: also vd = lines of v - in.
+template <int MODE>
+__global__ void __launch_bounds__(256) lines_kernel(const float* __restrict__ in, float* __restrict__ vz,
+                                                    const float* __restrict__ v, float* __restrict__ vd, int nx, int ny,
+                                                    int nz) {
+    __shared__ float tile[LT][LT + 1];
+    const int xt = (nx + LT - 1) / LT, ty = blockIdx.x / xt, t = ty / ny, y = ty % ny;
+    const int x0 = blockIdx.x % xt * LT, z0 = blockIdx.y * LT;
     const int nzp = vz_pitch(nz);
-    float bt = 0.0f;
-    if (FUSED) bt = (float)beta[t];
-    for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-        const int x = x0 + threadIdx.x, z = z0 + k;
+    const int lo = threadIdx.x % LT, hi = threadIdx.x / LT;
+    float keep[MODE == LINES_PAIR ? LT / 4 : 1];
+#pragma unroll
+    for (int k = 0; k < LT / 4; ++k) {
+        const int x = x0 + lo, z = z0 + 4 * k + hi;
+        const bool ok = x < nx && z < nz;
+        const size_t i = (((size_t)t * nz + z) * ny + y) * nx + x;
+        const float a = ok ? in[i] : 0.0f;
+        if (MODE == LINES_PAIR) keep[k] = ok ? __fsub_rn(v[i], a) : 0.0f;
+        tile[4 * k + hi][lo] = a;
+    }
+#pragma unroll
+    for (int pass = 0; pass < (MODE == LINES_PAIR ? 2 : 1); ++pass) {
+        float* out = pass ? vd : vz;
+        if (pass) {
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < LT / 4; ++k) tile[4 * k + hi][lo] = keep[MODE == LINES_PAIR ? k : 0];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < LT / 4; ++k) {
+            const int x = x0 + 4 * k + hi, z = z0 + lo;
+            if (x < nx && z < nz) out[(((size_t)t * ny + y) * nx + x) * nzp + VZ_FRONT + z] = tile[lo][4 * k + hi];
+        }
+    }
+}
+
+// x[nt][nz][ny][nx] = z + alpha_t p, z and p as lines (the last CG step).
+__global__ void __launch_bounds__(256) volume_kernel(const float* __restrict__ vz, const float* __restrict__ p,
+                                                     const double* __restrict__ alpha, float* __restrict__ out, int nx,
+                                                     int ny, int nz) {
+    __shared__ float tile[LT][LT + 1];
+    const int xt = (nx + LT - 1) / LT, ty = blockIdx.x / xt, t = ty / ny, y = ty % ny;
+    const int x0 = blockIdx.x % xt * LT, z0 = blockIdx.y * LT;
+    const int nzp = vz_pitch(nz);
+    const int lo = threadIdx.x % LT, hi = threadIdx.x / LT;
+    const float a = (float)alpha[t];
+#pragma unroll
+    for (int k = 0; k < LT / 4; ++k) {
+        const int x = x0 + 4 * k + hi, z = z0 + lo;
         if (x < nx && z < nz) {
-            const size_t i = (((size_t)t * nz + z) * ny + y) * nx + x;
-            float v = in[i];
-            if (FUSED) {
-                v = __fmaf_rn(bt, v, r[i]);
-                pnext[i] = v;
-            }
-            tile[k][threadIdx.x] = v;
+            const size_t i = (((size_t)t * ny + y) * nx + x) * nzp + VZ_FRONT + z;
+            tile[lo][4 * k + hi] = __fmaf_rn(a, p[i], vz[i]);
         }
     }
     __syncthreads();
-    for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-        const int x = x0 + k, z = z0 + threadIdx.x;
-        if (x < nx && z < nz) vz[(((size_t)t * ny + y) * nx + x) * nzp + VZ_FRONT + z] = tile[threadIdx.x][k];
+#pragma unroll
+    for (int k = 0; k < LT / 4; ++k) {
+        const int x = x0 + lo, z = z0 + 4 * k + hi;
+        if (x < nx && z < nz) out[(((size_t)t * nz + z) * ny + y) * nx + x] = tile[4 * k + hi][lo];
     }
 }
 
@@ -398,6 +435,56 @@ __global__ void __launch_bounds__(256, R == 5 ? 1 : 3) joseph_fwd_kernel(
 
 enum AdjMode { ADJ_PLAIN = 0, ADJ_CG_INIT = 1, ADJ_CG_Q = 2 };
 
+// ------------------------------------------------------------------ CG scalars
+//
+// A kernel whose blocks each hold a partial sum of a frame hands them to the
+// frame's last block, which adds them in a fixed order and forms the scalar:
+//   FIN_RR0:   rr = sum
+//   FIN_ALPHA: alpha = rr / sum (0 when sum == 0)
+//   FIN_BETA:  beta = sum / rr (0 when rr == 0); rr = sum
+// Any non-finite sum raises the status flag.  (A kernel of its own per scalar
+// cost a launch, 11 per five CG steps.)
+enum FinMode { FIN_RR0 = 0, FIN_ALPHA = 1, FIN_BETA = 2 };
+
+struct CgScalars {
+    double* partial;      // [nt][blocks of a frame]
+    double *rr, *coef;    // [nt]
+    int* status;
+    unsigned* count;      // [nt], zero between kernels: blocks of the frame that have stored their sum
+};
+
+// sum: this block's partial, in thread 0; b of nparts: its place in frame t.
+template <int FIN>
+__device__ __forceinline__ void frame_finalize(double sum, int t, int b, int nparts, const CgScalars& c) {
+    __shared__ bool last;
+    const int tid = threadIdx.x + blockDim.x * threadIdx.y, nthreads = blockDim.x * blockDim.y;
+    double* part = c.partial + (size_t)t * nparts;
+    if (tid == 0) {
+        part[b] = sum;
+        __threadfence();
+        last = atomicAdd(c.count + t, 1u) == (unsigned)nparts - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    double s = 0.0;
+    for (int i = tid; i < nparts; i += nthreads) s += __ldcg(part + i);
+    s = block_sum_f64(s);
+    if (tid == 0) {
+        if (!isfinite(s)) atomicExch(c.status, (int)MSF_ERR_NUMERIC);
+        if (FIN == FIN_RR0) {
+            c.rr[t] = s;
+        } else if (FIN == FIN_ALPHA) {
+            c.coef[t] = (s != 0.0) ? c.rr[t] / s : 0.0;
+        } else {
+            c.coef[t] = (c.rr[t] != 0.0) ? s / c.rr[t] : 0.0;
+            c.rr[t] = s;
+        }
+        c.count[t] = 0;
+    }
+}
+
+
 constexpr int ADJ_T = 4;           // a block's tile: ADJ_T x ADJ_T voxel lines in (x, y), one warp per ADJ_T
 constexpr int ADJ_ENTRIES = 32;    // columns of a warp's list
 // floats of one line in a block's tile: its 32 J voxels, and 8 that put the
@@ -645,14 +732,14 @@ __host__ __device__ constexpr int adj_min_blocks(int J) { return J >= 8 ? 4 : J 
 // need fewer columns per line (0.79 against 0.88) but took 20 ms.
 // e is the step-weighted sinogram e' = step * e in lines of rows.
 //   ADJ_PLAIN:   out = A^T e
-//   ADJ_CG_INIT: r = A^T e + (v - z)/sigma^2, p = r, partial sum r.r
-//   ADJ_CG_Q:    q = A^T e + p/sigma^2, partial sum p.q
+//   ADJ_CG_INIT: r = A^T e + (v - z)/sigma^2, p = r, rr = r.r (a1 = v - z)
+//   ADJ_CG_Q:    q = A^T e + p/sigma^2, alpha = rr / p.q      (a1 = p)
+// (the CG's vectors as lines, the volume of ADJ_PLAIN as [nt][nz][ny][nx])
 template <int MODE, int J>
 __global__ void __launch_bounds__(32 * ADJ_T, adj_min_blocks(J)) joseph_adj_kernel(
     const float4* __restrict__ col, const float2* __restrict__ trig, const int* __restrict__ vflag,
-    const float* __restrict__ e, float* __restrict__ out, const float* __restrict__ a1,
-    const float* __restrict__ a2, float* __restrict__ out2, double* __restrict__ partial,
-    float inv_s2, ProjDims d, int slots) {
+    const float* __restrict__ e, float* __restrict__ out, const float* __restrict__ a1, float* __restrict__ out2,
+    CgScalars cg, float inv_s2, ProjDims d, int slots) {
     extern __shared__ float adj_tile[];   // [y][x][adj_line(J)]
     __shared__ AdjEntry list[ADJ_T][ADJ_ENTRIES];
     __shared__ int slot[ADJ_T][ADJ_ENTRIES];
@@ -691,44 +778,47 @@ __global__ void __launch_bounds__(32 * ADJ_T, adj_min_blocks(J)) joseph_adj_kern
     double dot = 0.0;
     if (iy < d.ny) {
         gather_run<false, J>(col, trig, vflag, e, t, iy, x0, zb * 32 * J, zc, d, slots, list[w], slot[w], acc);
-        // the volume is contiguous along x: ADJ_T lanes write the x of one z
+        if (MODE == ADJ_PLAIN) {
+            // the volume is contiguous along x: ADJ_T lanes write the x of one z
 #pragma unroll
-        for (int i = 0; i < ADJ_T; ++i) {
-            float v[J];
-            acc[i].get(v);
+            for (int i = 0; i < ADJ_T; ++i) {
+                float v[J];
+                acc[i].get(v);
 #pragma unroll
-            for (int j = 0; j < J; ++j) tile[i * adj_line(J) + 32 * j + lane] = v[j];
-        }
-        __syncwarp();
-        const int ix = x0 + lane % ADJ_T;
+                for (int j = 0; j < J; ++j) tile[i * adj_line(J) + 32 * j + lane] = v[j];
+            }
+            __syncwarp();
+            const int ix = x0 + lane % ADJ_T;
 #pragma unroll 4
-        for (int k = lane / ADJ_T; k < 32 * J; k += 32 / ADJ_T) {
-            const int iz = zb * 32 * J + k;
-            if (ix >= d.nx || iz >= d.nz) break;
-            const size_t i = (((size_t)t * d.nz + iz) * d.ny + iy) * d.nx + ix;
-            const float s = tile[(lane % ADJ_T) * adj_line(J) + k];
-            if (MODE == ADJ_PLAIN) {
-                out[i] = s;
-            } else if (MODE == ADJ_CG_INIT) {   // a1 = v, a2 = z
-                const float r = s + (a1[i] - a2[i]) * inv_s2;
-                out[i] = r;
-                out2[i] = r;
-                dot += (double)r * (double)r;
-            } else {                            // a1 = p
-                const float p = a1[i];
-                const float q = s + p * inv_s2;
-                out[i] = q;
-                dot += (double)p * (double)q;
+            for (int k = lane / ADJ_T; k < 32 * J; k += 32 / ADJ_T) {
+                const int iz = zb * 32 * J + k;
+                if (ix >= d.nx || iz >= d.nz) break;
+                out[(((size_t)t * d.nz + iz) * d.ny + iy) * d.nx + ix] = tile[(lane % ADJ_T) * adj_line(J) + k];
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < ADJ_T; ++i) {
+                if (x0 + i >= d.nx) break;
+                const size_t line = (((size_t)t * d.ny + iy) * d.nx + x0 + i) * vz_pitch(d.nz) + VZ_FRONT;
+                float v[J];
+                acc[i].get(v);
+#pragma unroll
+                for (int j = 0; j < J; ++j) {
+                    if (z0 + 32 * j >= d.nz) break;
+                    const size_t k = line + z0 + 32 * j;
+                    const float a = a1[k], r = __fmaf_rn(a, inv_s2, v[j]);
+                    out[k] = r;
+                    if (MODE == ADJ_CG_INIT) out2[k] = r;
+                    dot += (double)(MODE == ADJ_CG_INIT ? r : a) * (double)r;
+                }
             }
         }
     }
     if (MODE != ADJ_PLAIN) {
         const double sum = block_sum_f64(dot);
-        if (lane == 0 && w == 0) {
-            const int bpf = gridDim.x * gridDim.y * nzb;   // blocks per frame
-            const int b = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * zb);
-            partial[(size_t)t * bpf + b] = sum;
-        }
+        const int bpf = gridDim.x * gridDim.y * nzb;   // blocks per frame
+        const int b = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * zb);
+        frame_finalize<MODE == ADJ_CG_INIT ? FIN_RR0 : FIN_ALPHA>(sum, t, b, bpf, cg);
     }
 }
 
@@ -751,62 +841,77 @@ __global__ void step_weight_kernel(const float4* __restrict__ col, const float* 
         out[((size_t)g * d.nu + u0 + k) * sino_pitch(d.nv) + SINO_FRONT + iv] = tile[threadIdx.x][k];
 }
 
-// ------------------------------------------------------------------ CG scalars
+// ------------------------------------------------------------------ CG vectors
 
-enum FinMode { FIN_RR0 = 0, FIN_ALPHA = 1, FIN_BETA = 2 };
-
-// One block per frame: sums that frame's block partials in a fixed order.
-//   FIN_RR0:   rr = sum
-//   FIN_ALPHA: alpha = rr / sum (0 when sum == 0)
-//   FIN_BETA:  beta = sum / rr (0 when rr == 0); rr = sum
-// Any non-finite sum raises the status flag.
-template <int MODE>
-__global__ void cg_finalize_kernel(const double* __restrict__ partial, int nparts,
-                                   double* __restrict__ rr, double* __restrict__ coef,
-                                   int* __restrict__ status) {
-    const int t = blockIdx.x;
-    double s = 0.0;
-    for (int i = threadIdx.x; i < nparts; i += blockDim.x) s += partial[(size_t)t * nparts + i];
-    s = block_sum_f64(s);
-    if (threadIdx.x == 0) {
-        if (!isfinite(s)) atomicExch(status, (int)MSF_ERR_NUMERIC);
-        if (MODE == FIN_RR0) {
-            rr[t] = s;
-        } else if (MODE == FIN_ALPHA) {
-            coef[t] = (s != 0.0) ? rr[t] / s : 0.0;
-        } else {
-            coef[t] = (rr[t] != 0.0) ? s / rr[t] : 0.0;
-            rr[t] = s;
-        }
-    }
+// The vectors are lines; a warp takes one line (several short ones), its lanes
+// units of four voxels.  The margins of the lines stay untouched.
+template <typename F>
+__device__ __forceinline__ void for_units(size_t lines, int nz, F&& f) {
+    const int n4 = (nz + 3) / 4, nzp = vz_pitch(nz);
+    int gw = 32;   // lanes per line
+    while (gw > 1 && gw / 2 >= n4) gw /= 2;
+    const int lane = threadIdx.x & 31, per = 32 / gw, warps = blockDim.x >> 5;
+    const size_t first = ((size_t)blockIdx.x * warps + (threadIdx.x >> 5)) * per + lane / gw;
+    for (size_t l = first; l < lines; l += (size_t)gridDim.x * warps * per)
+        for (int u = lane % gw; u < n4; u += gw) f(l * nzp + VZ_FRONT + 4 * u, min(4, nz - 4 * u));
 }
 
-// z += alpha p; r -= alpha q; partial r.r  (grid: blocks_per_frame x nt).
-// Each thread adds the squares of runs of 8 of its elements in FP32 before its
-// FP64 sum (FP64 arithmetic is a small fraction of the FP32 rate on this GPU);
-// the order of every addition is fixed.
-__global__ void cg_update_kernel(float* __restrict__ z, float* __restrict__ r,
-                                 const float* __restrict__ p, const float* __restrict__ q,
-                                 const double* __restrict__ alpha, double* __restrict__ partial,
-                                 size_t fs) {
-    const int t = blockIdx.y;
-    const float a = (float)alpha[t];
-    const size_t off = (size_t)t * fs;
-    const size_t stride = (size_t)gridDim.x * blockDim.x;
-    double dot = 0.0;
-    size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    while (i < fs) {
-        float run = 0.0f;
-        for (int k = 0; k < 8 && i < fs; ++k, i += stride) {
-            z[off + i] = __fmaf_rn(a, p[off + i], z[off + i]);
-            const float rn = __fmaf_rn(-a, q[off + i], r[off + i]);
-            r[off + i] = rn;
-            run = __fmaf_rn(rn, rn, run);
-        }
-        dot += (double)run;
+__device__ __forceinline__ float4 load4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+// the first n of four values
+__device__ __forceinline__ void store4(float* p, float4 v, int n) {
+    if (n == 4) {
+        *reinterpret_cast<float4*>(p) = v;
+    } else {
+        p[0] = v.x;
+        if (n > 1) p[1] = v.y;
+        if (n > 2) p[2] = v.z;
     }
-    const double s = block_sum_f64(dot);
-    if (threadIdx.x == 0) partial[(size_t)t * gridDim.x + blockIdx.x] = s;
+}
+__device__ __forceinline__ float4 fma4(float a, float4 x, float4 y) {
+    return make_float4(__fmaf_rn(a, x.x, y.x), __fmaf_rn(a, x.y, y.y), __fmaf_rn(a, x.z, y.z), __fmaf_rn(a, x.w, y.w));
+}
+
+// r -= alpha q; beta = r.r / rr  (grid: blocks of a frame x nt).  Each thread
+// adds the squares of runs of 8 of its elements in FP32 before its FP64 sum
+// (FP64 arithmetic is a small fraction of the FP32 rate on this GPU); the order
+// of every addition is fixed.  Bound by HBM (12 bytes per voxel).
+__global__ void __launch_bounds__(256) cg_residual_kernel(float* __restrict__ r, const float* __restrict__ q,
+                                                          const double* __restrict__ alpha, CgScalars cg, size_t lines,
+                                                          int nz) {
+    const int t = blockIdx.y;
+    const float a = -(float)alpha[t];
+    const size_t off = (size_t)t * lines * vz_pitch(nz);
+    double dot = 0.0;
+    float run = 0.0f;
+    int k = 0;
+    for_units(lines, nz, [&](size_t i, int n) {
+        const float4 v = fma4(a, load4(q + off + i), load4(r + off + i));
+        store4(r + off + i, v, n);
+        run = __fmaf_rn(v.x, v.x, run);
+        if (n > 1) run = __fmaf_rn(v.y, v.y, run);
+        if (n > 2) run = __fmaf_rn(v.z, v.z, run);
+        if (n > 3) run = __fmaf_rn(v.w, v.w, run);
+        if (++k & 1) return;
+        dot += (double)run;
+        run = 0.0f;
+    });
+    const double s = block_sum_f64(dot + (double)run);
+    frame_finalize<FIN_BETA>(s, t, blockIdx.x, gridDim.x, cg);
+}
+
+// z += alpha p; p = r + beta p.  Bound by HBM (20 bytes per voxel).
+__global__ void __launch_bounds__(256) cg_direction_kernel(float* __restrict__ z, float* __restrict__ p,
+                                                           const float* __restrict__ r,
+                                                           const double* __restrict__ alpha,
+                                                           const double* __restrict__ beta, size_t lines, int nz) {
+    const int t = blockIdx.y;
+    const float a = (float)alpha[t], b = (float)beta[t];
+    const size_t off = (size_t)t * lines * vz_pitch(nz);
+    for_units(lines, nz, [&](size_t i, int n) {
+        const float4 pv = load4(p + off + i);
+        store4(z + off + i, fma4(a, pv, load4(z + off + i)), n);
+        store4(p + off + i, fma4(b, pv, load4(r + off + i)), n);
+    });
 }
 
 // ------------------------------------------------------------------ grouped ICD data agent
@@ -1163,11 +1268,15 @@ struct msf_projector {
 
 struct msf_dataprox {
     msf_projector* p = nullptr;
-    float *d_r = nullptr, *d_p = nullptr, *d_p2 = nullptr, *d_q = nullptr, *d_s = nullptr;
+    // CG: residual, direction and A^T Lambda A p + p / sigma^2, as lines (d_q
+    // first holds v - z; z itself runs in the plan's d_vz)
+    float *d_r = nullptr, *d_p = nullptr, *d_q = nullptr;
+    float *d_dlt = nullptr, *d_t2 = nullptr, *d_s = nullptr;   // ICD: delta, theta2, sinogram
     float* d_rows = nullptr;   // step-weighted sinogram in lines of rows
     double *d_partial = nullptr, *d_rr = nullptr, *d_alpha = nullptr, *d_beta = nullptr;
     int* d_status = nullptr;
-    int parts_adj = 0, parts_upd = 0, parts_max = 0;
+    unsigned* d_count = nullptr;
+    int parts_upd = 0;
     // grouped ICD: a second sinogram (A delta, and step^2 Lambda for theta2),
     // the group gather's partial sums and the sinogram pass's partial sums
     float* d_s2 = nullptr;
@@ -1179,6 +1288,9 @@ namespace msf {
 
 static size_t frame_size(const msf_vol& v) { return (size_t)v.nx * v.ny * v.nz; }
 static size_t vol_size(const msf_vol& v) { return frame_size(v) * v.nt; }
+static size_t vz_size(const msf_vol& v) {   // a volume as lines
+    return (size_t)v.nt * v.ny * v.nx * vz_pitch(v.nz);
+}
 static size_t rows_size(const msf_projector* p) {   // a sinogram in lines of rows
     return (size_t)p->vol.nt * p->geom.views * p->geom.nu * sino_pitch(p->geom.nv);
 }
@@ -1186,12 +1298,12 @@ static size_t sino_size(const msf_projector* p) {
     return (size_t)p->geom.nu * p->geom.nv * p->geom.views * p->vol.nt;
 }
 
-static dim3 lines_grid(const msf_vol& v) { return dim3(v.ny * v.nt, (v.nx + 31) / 32, (v.nz + 31) / 32); }
+static dim3 lines_grid(const msf_vol& v) { return dim3((v.nx + LT - 1) / LT * v.ny * v.nt, (v.nz + LT - 1) / LT); }
 
 static msf_status launch_lines(msf_projector* p, const float* in, cudaStream_t st) {
     const msf_vol& v = p->vol;
     MSF_PROF("transpose", st);
-    lines_kernel<false><<<lines_grid(v), dim3(32, 8), 0, st>>>(in, p->d_vz, nullptr, nullptr, nullptr, v.nx, v.ny, v.nz);
+    lines_kernel<LINES_COPY><<<lines_grid(v), 256, 0, st>>>(in, p->d_vz, nullptr, nullptr, v.nx, v.ny, v.nz);
     MSF_LAUNCH_CHECK();
     return MSF_OK;
 }
@@ -1270,23 +1382,17 @@ static int adj_nzb(const ProjDims& d, int zrun) {
 static dim3 adj_grid(const ProjDims& d, int zrun) {
     return dim3((d.nx + ADJ_T - 1) / ADJ_T, (d.ny + ADJ_T - 1) / ADJ_T, adj_nzb(d, zrun) * d.nt);
 }
-// partial sums per frame of an adjoint launch
-static int adj_parts(const msf_projector* p) {
-    const dim3 g = adj_grid(p->dims, p->adj_zb);
-    return g.x * g.y * adj_nzb(p->dims, p->adj_zb);
-}
-
 template <int MODE>
-static void launch_adj_zb(msf_projector* p, const float* e, float* out, const float* a1, const float* a2,
-                          float* out2, double* partial, float inv_s2, cudaStream_t st) {
+static void launch_adj_zb(msf_projector* p, const float* e, float* out, const float* a1, float* out2,
+                          const CgScalars& cg, float inv_s2, cudaStream_t st) {
     const ProjDims& d = p->dims;
     const int J = adj_j(d, p->adj_zb), slots = adj_slots(d);
     const dim3 block(32, ADJ_T), grid = adj_grid(d, p->adj_zb);
     const size_t smem = (size_t)ADJ_T * ADJ_T * adj_line(J) * sizeof(float);
 #define MSF_ADJ_CASE(N)                                                                                             \
     case N:                                                                                                         \
-        joseph_adj_kernel<MODE, N><<<grid, block, smem, st>>>(p->d_col, p->d_trig, p->d_vflag, e, out, a1, a2, out2, \
-                                                               partial, inv_s2, d, slots);                          \
+        joseph_adj_kernel<MODE, N><<<grid, block, smem, st>>>(p->d_col, p->d_trig, p->d_vflag, e, out, a1, out2, cg, \
+                                                               inv_s2, d, slots);                                   \
         break;
     switch (J) {
         MSF_ADJ_CASE(1)
@@ -1302,16 +1408,11 @@ static void launch_adj_zb(msf_projector* p, const float* e, float* out, const fl
 #undef MSF_ADJ_CASE
 }
 
-static msf_status launch_adj(msf_projector* p, int mode, const float* e, float* out,
-                             const float* a1, const float* a2, float* out2, double* partial,
-                             float inv_s2, cudaStream_t st) {
+template <int MODE>
+static msf_status launch_adj(msf_projector* p, const float* e, float* out, const float* a1, float* out2,
+                             const CgScalars& cg, float inv_s2, cudaStream_t st) {
     MSF_PROF("joseph_adj", st);
-    if (mode == ADJ_PLAIN)
-        launch_adj_zb<ADJ_PLAIN>(p, e, out, a1, a2, out2, partial, inv_s2, st);
-    else if (mode == ADJ_CG_INIT)
-        launch_adj_zb<ADJ_CG_INIT>(p, e, out, a1, a2, out2, partial, inv_s2, st);
-    else
-        launch_adj_zb<ADJ_CG_Q>(p, e, out, a1, a2, out2, partial, inv_s2, st);
+    launch_adj_zb<MODE>(p, e, out, a1, out2, cg, inv_s2, st);
     MSF_LAUNCH_CHECK();
     return MSF_OK;
 }
@@ -1365,7 +1466,7 @@ extern "C" msf_status msf_projector_create(const msf_geom* geom, const msf_vol* 
     auto cleanup = [&](msf_status st) { msf_projector_destroy(p); return st; };
     const size_t col_bytes = (size_t)G * geom->nu * 2 * sizeof(float4);
     const size_t line_bytes = vz_pitch(vol->nz) * sizeof(float);
-    const size_t vz_bytes = (size_t)vol->nt * vol->ny * vol->nx * line_bytes;
+    const size_t vz_bytes = vz_size(*vol) * sizeof(float);
     if (cudaMalloc(&p->d_angles, G * sizeof(double)) != cudaSuccess ||
         cudaMalloc(&p->d_col, col_bytes) != cudaSuccess ||
         cudaMalloc(&p->d_trig, G * sizeof(float2)) != cudaSuccess ||
@@ -1432,7 +1533,7 @@ extern "C" msf_status msf_backproject(msf_projector* p, const float* d_y, float*
             p->d_col, d_y, p->d_sw, d);
         MSF_LAUNCH_CHECK();
     }
-    return launch_adj(p, ADJ_PLAIN, p->d_sw, d_x, nullptr, nullptr, nullptr, nullptr, 0.0f, st);
+    return launch_adj<ADJ_PLAIN>(p, p->d_sw, d_x, nullptr, nullptr, CgScalars{}, 0.0f, st);
 }
 
 extern "C" msf_status msf_dataprox_create(msf_projector* p, msf_dataprox** out) {
@@ -1441,10 +1542,13 @@ extern "C" msf_status msf_dataprox_create(msf_projector* p, msf_dataprox** out) 
     msf_dataprox* d = new msf_dataprox();
     d->p = p;
     const size_t nv = vol_size(p->vol), ns = sino_size(p);
+    const size_t nl = vz_size(p->vol);
     const dim3 ga = adj_grid(p->dims, 8);             // the largest block count of any z-run
-    d->parts_adj = ga.x * ga.y * adj_nzb(p->dims, 8);
-    d->parts_upd = 512;
-    d->parts_max = d->parts_adj > d->parts_upd ? d->parts_adj : d->parts_upd;
+    const int parts_adj = ga.x * ga.y * adj_nzb(p->dims, 8);
+    // blocks of a frame of the vector kernels: eight warps of one line or more each
+    const size_t lines = (size_t)p->vol.nx * p->vol.ny;
+    d->parts_upd = lines < 8 * 512 ? (int)((lines + 7) / 8) : 512;
+    const int parts_max = parts_adj > d->parts_upd ? parts_adj : d->parts_upd;
     const int nt = p->vol.nt;
     {   // the largest group grid (parity 0 along every axis)
         const msf_vol& v = p->vol;
@@ -1454,10 +1558,11 @@ extern "C" msf_status msf_dataprox_create(msf_projector* p, msf_dataprox** out) 
     if (cudaMalloc(&d->d_s2, ns * 4) != cudaSuccess || cudaMalloc(&d->d_rows, rows_size(p) * 4) != cudaSuccess ||
         cudaMalloc(&d->d_ipart, (size_t)nt * d->parts_icd * 2 * 8) != cudaSuccess ||
         cudaMalloc(&d->d_spart, (size_t)nt * ICD_SINO_BLOCKS * 8) != cudaSuccess ||
-        cudaMalloc(&d->d_r, nv * 4) != cudaSuccess || cudaMalloc(&d->d_p, nv * 4) != cudaSuccess ||
-        cudaMalloc(&d->d_p2, nv * 4) != cudaSuccess ||
-        cudaMalloc(&d->d_q, nv * 4) != cudaSuccess || cudaMalloc(&d->d_s, ns * 4) != cudaSuccess ||
-        cudaMalloc(&d->d_partial, (size_t)nt * d->parts_max * 8) != cudaSuccess ||
+        cudaMalloc(&d->d_r, nl * 4) != cudaSuccess || cudaMalloc(&d->d_p, nl * 4) != cudaSuccess ||
+        cudaMalloc(&d->d_q, nl * 4) != cudaSuccess || cudaMalloc(&d->d_dlt, nv * 4) != cudaSuccess ||
+        cudaMalloc(&d->d_t2, nv * 4) != cudaSuccess || cudaMalloc(&d->d_s, ns * 4) != cudaSuccess ||
+        cudaMalloc(&d->d_count, nt * sizeof(unsigned)) != cudaSuccess ||
+        cudaMalloc(&d->d_partial, (size_t)nt * parts_max * 8) != cudaSuccess ||
         cudaMalloc(&d->d_rr, nt * 8) != cudaSuccess || cudaMalloc(&d->d_alpha, nt * 8) != cudaSuccess ||
         cudaMalloc(&d->d_beta, nt * 8) != cudaSuccess || cudaMalloc(&d->d_status, sizeof(int)) != cudaSuccess) {
         cudaGetLastError();
@@ -1465,7 +1570,9 @@ extern "C" msf_status msf_dataprox_create(msf_projector* p, msf_dataprox** out) 
         return fail(MSF_ERR_NOMEM, "msf_dataprox_create: out of device memory");
     }
     if (cudaMemset(d->d_status, 0, sizeof(int)) != cudaSuccess ||
-        cudaMemset(d->d_rows, 0, rows_size(p) * 4) != cudaSuccess) {
+        cudaMemset(d->d_count, 0, nt * sizeof(unsigned)) != cudaSuccess ||
+        cudaMemset(d->d_p, 0, nl * 4) != cudaSuccess || cudaMemset(d->d_r, 0, nl * 4) != cudaSuccess ||
+        cudaMemset(d->d_q, 0, nl * 4) != cudaSuccess || cudaMemset(d->d_rows, 0, rows_size(p) * 4) != cudaSuccess) {
         msf_dataprox_destroy(d);
         return fail(MSF_ERR_CUDA, "msf_dataprox_create: memset failed");
     }
@@ -1475,7 +1582,8 @@ extern "C" msf_status msf_dataprox_create(msf_projector* p, msf_dataprox** out) 
 
 extern "C" void msf_dataprox_destroy(msf_dataprox* d) {
     if (!d) return;
-    cudaFree(d->d_r); cudaFree(d->d_p); cudaFree(d->d_p2); cudaFree(d->d_q); cudaFree(d->d_s);
+    cudaFree(d->d_r); cudaFree(d->d_p); cudaFree(d->d_q); cudaFree(d->d_dlt); cudaFree(d->d_t2); cudaFree(d->d_s);
+    cudaFree(d->d_count);
     cudaFree(d->d_partial); cudaFree(d->d_rr); cudaFree(d->d_alpha); cudaFree(d->d_beta);
     cudaFree(d->d_status);
     cudaFree(d->d_s2); cudaFree(d->d_rows); cudaFree(d->d_ipart); cudaFree(d->d_spart);
@@ -1491,51 +1599,40 @@ extern "C" msf_status msf_prox_data(msf_dataprox* dp, const float* d_y, const fl
     msf_projector* p = dp->p;
     cudaStream_t st = as_stream(stream);
     const float inv_s2 = (float)(1.0 / (sigma * sigma));
-    const int nt = p->vol.nt;
-    const size_t fs = frame_size(p->vol);
-    // r = A^T Lambda (y - A z) + (v - z)/sigma^2 ; p = r ; rr = r.r
-    MSF_TRY((launch_fwd<FWD_RESIDUAL, true>(p, d_x, dp->d_rows, d_lambda, d_y, st)));
-    MSF_TRY(launch_adj(p, ADJ_CG_INIT, dp->d_rows, dp->d_r, d_v, d_x, dp->d_p, dp->d_partial, inv_s2, st));
-    {
-        MSF_PROF("cg_finalize", st);
-        cg_finalize_kernel<FIN_RR0><<<nt, 256, 0, st>>>(dp->d_partial, adj_parts(p), dp->d_rr, nullptr, dp->d_status);
+    const msf_vol& v = p->vol;
+    const size_t lines = (size_t)v.nx * v.ny;
+    const dim3 ugrid(dp->parts_upd, v.nt);
+    const CgScalars ca{dp->d_partial, dp->d_rr, dp->d_alpha, dp->d_status, dp->d_count};
+    const CgScalars cb{dp->d_partial, dp->d_rr, dp->d_beta, dp->d_status, dp->d_count};
+    float* z = p->d_vz;
+    {   // z and v - z as lines
+        MSF_PROF("transpose", st);
+        lines_kernel<LINES_PAIR><<<lines_grid(v), 256, 0, st>>>(d_x, z, d_v, dp->d_q, v.nx, v.ny, v.nz);
         MSF_LAUNCH_CHECK();
     }
-    const msf_vol& v = p->vol;
-    // the direction p alternates between two buffers
-    float* pc = dp->d_p;
+    // r = A^T Lambda (y - A z) + (v - z)/sigma^2 ; p = r ; rr = r.r
+    MSF_TRY((launch_fwd_lines<FWD_RESIDUAL, true>(p, z, dp->d_rows, d_lambda, d_y, st)));
+    MSF_TRY(launch_adj<ADJ_CG_INIT>(p, dp->d_rows, dp->d_r, dp->d_q, dp->d_p, ca, inv_s2, st));
     for (int it = 0; it < n_cg; ++it) {
-        // lines of p for the forward (fused with p = r + beta p after the first pass)
-        if (it == 0) {
-            MSF_TRY(launch_lines(p, pc, st));
-        } else {
-            float* pn = pc == dp->d_p ? dp->d_p2 : dp->d_p;
-            MSF_PROF("transpose_pupdate", st);
-            lines_kernel<true><<<lines_grid(v), dim3(32, 8), 0, st>>>(pc, p->d_vz, dp->d_r, pn, dp->d_beta, v.nx, v.ny,
-                                                                      v.nz);
-            MSF_LAUNCH_CHECK();
-            pc = pn;
-        }
-        // s = Lambda A p
-        MSF_TRY((launch_fwd_lines<FWD_LAMBDA, true>(p, p->d_vz, dp->d_rows, d_lambda, nullptr, st)));
-        // q = A^T s + p/sigma^2 ; alpha = rr / p.q
-        MSF_TRY(launch_adj(p, ADJ_CG_Q, dp->d_rows, dp->d_q, pc, nullptr, nullptr, dp->d_partial, inv_s2, st));
-        {
-            MSF_PROF("cg_finalize", st);
-            cg_finalize_kernel<FIN_ALPHA><<<nt, 256, 0, st>>>(dp->d_partial, adj_parts(p), dp->d_rr, dp->d_alpha, dp->d_status);
+        // s = Lambda A p ; q = A^T s + p/sigma^2 ; alpha = rr / p.q
+        MSF_TRY((launch_fwd_lines<FWD_LAMBDA, true>(p, dp->d_p, dp->d_rows, d_lambda, nullptr, st)));
+        MSF_TRY(launch_adj<ADJ_CG_Q>(p, dp->d_rows, dp->d_q, dp->d_p, nullptr, ca, inv_s2, st));
+        if (it + 1 == n_cg) break;
+        {   // r -= alpha q ; beta = r.r / rr
+            MSF_PROF("cg_residual", st);
+            cg_residual_kernel<<<ugrid, 256, 0, st>>>(dp->d_r, dp->d_q, dp->d_alpha, cb, lines, v.nz);
             MSF_LAUNCH_CHECK();
         }
-        {   // z += alpha p ; r -= alpha q ; beta = r.r / rr
-            MSF_PROF("cg_update", st);
-            cg_update_kernel<<<dim3(dp->parts_upd, nt), 256, 0, st>>>(d_x, dp->d_r, pc, dp->d_q, dp->d_alpha, dp->d_partial, fs);
-            MSF_LAUNCH_CHECK();
-        }
-        {
-            MSF_PROF("cg_finalize", st);
-            cg_finalize_kernel<FIN_BETA><<<nt, 256, 0, st>>>(dp->d_partial, dp->parts_upd, dp->d_rr, dp->d_beta, dp->d_status);
+        {   // z += alpha p ; p = r + beta p
+            MSF_PROF("cg_direction", st);
+            cg_direction_kernel<<<ugrid, 256, 0, st>>>(z, dp->d_p, dp->d_r, dp->d_alpha, dp->d_beta, lines, v.nz);
             MSF_LAUNCH_CHECK();
         }
     }
+    // the last step's z + alpha p, back in volume order (its r has no reader)
+    MSF_PROF("volume", st);
+    volume_kernel<<<lines_grid(v), 256, 0, st>>>(z, dp->d_p, dp->d_alpha, d_x, v.nx, v.ny, v.nz);
+    MSF_LAUNCH_CHECK();
     return MSF_OK;
 }
 
@@ -1562,11 +1659,11 @@ extern "C" msf_status msf_prox_data_icd(msf_dataprox* dp, const float* d_y, cons
     {
         MSF_PROF("icd_theta2", st);
         const dim3 grid((d.nx + 31) / 32, (d.ny + 3) / 4, ((d.nz + 15) / 16) * d.nt);
-        icd_theta2_kernel<16><<<grid, dim3(32, 4), 0, st>>>(p->d_col, p->d_trig, p->d_vflag, dp->d_s2, dp->d_q,
+        icd_theta2_kernel<16><<<grid, dim3(32, 4), 0, st>>>(p->d_col, p->d_trig, p->d_vflag, dp->d_s2, dp->d_t2,
                                                             inv_s2, d);
         MSF_LAUNCH_CHECK();
     }
-    MSF_TRY_CUDA(cudaMemsetAsync(dp->d_p, 0, vol_size(v) * sizeof(float), st));
+    MSF_TRY_CUDA(cudaMemsetAsync(dp->d_dlt, 0, vol_size(v) * sizeof(float), st));
     for (int sw = 0; sw < n_sweeps; ++sw) {
         for (int grp = 0; grp < 8; ++grp) {
             IcdGroup G;
@@ -1579,12 +1676,12 @@ extern "C" msf_status msf_prox_data_icd(msf_dataprox* dp, const float* d_y, cons
             {
                 MSF_PROF("icd_group", st);
                 icd_group_kernel<ICD_ZB><<<grid, dim3(32, 4), 0, st>>>(p->d_col, p->d_trig, p->d_vflag, dp->d_s,
-                                                                      d_x, d_v, dp->d_q, dp->d_p, dp->d_ipart,
+                                                                      d_x, d_v, dp->d_t2, dp->d_dlt, dp->d_ipart,
                                                                       inv_s2, G, d);
                 MSF_LAUNCH_CHECK();
             }
             // A delta: delta is zero outside the group (icd_update clears it)
-            MSF_TRY(launch_fwd_parity(p, dp->d_p, dp->d_s2, G.px, G.py, st));
+            MSF_TRY(launch_fwd_parity(p, dp->d_dlt, dp->d_s2, G.px, G.py, st));
             {
                 MSF_PROF("icd_sino", st);
                 icd_sino_kernel<0><<<dim3(ICD_SINO_BLOCKS, nt), 256, 0, st>>>(p->d_col, dp->d_s2, d_lambda, dp->d_s,
@@ -1599,7 +1696,7 @@ extern "C" msf_status msf_prox_data_icd(msf_dataprox* dp, const float* d_y, cons
             }
             {
                 MSF_PROF("icd_update", st);
-                icd_update_kernel<<<152 * 4, 256, 0, st>>>(d_x, dp->d_p, dp->d_alpha, G, d);
+                icd_update_kernel<<<152 * 4, 256, 0, st>>>(d_x, dp->d_dlt, dp->d_alpha, G, d);
                 MSF_LAUNCH_CHECK();
             }
             {
@@ -1875,7 +1972,7 @@ extern "C" msf_status msf_projector_autotune(msf_projector* p, void* stream, int
     int bz = 1;
     for (int i = 0; i < (deep64 ? 4 : 3); ++i) {
         p->adj_zb = zbs[i];
-        const float ms = time_it([&] { launch_adj_zb<ADJ_PLAIN>(p, p->d_sw, tmp, nullptr, nullptr, nullptr, nullptr, 0.0f, st); });
+        const float ms = time_it([&] { launch_adj_zb<ADJ_PLAIN>(p, p->d_sw, tmp, nullptr, nullptr, CgScalars{}, 0.0f, st); });
         if (ms < best) { best = ms; bz = i; }
     }
     p->adj_zb = zbs[bz];
