@@ -20,21 +20,89 @@ struct MrfDims {
     float inv_s2;                // 1/sigma^2
     float inv_tsx;               // 1/(T sigma_x)
     float pq;                    // p - q
-    float q_over_p;
-    float inv_2sx2;              // 1/(2 sigma_x^2)  (p = 2)
-    float bf, be, bc, bt;        // face, edge, corner, temporal weights
+    // surrogate coefficients of the face, edge, corner and temporal neighbours,
+    // 2 b a(D) = w (k1 + k2 w) with w = 1 / (1 + r): 2 b (q/p) / (2 sigma_x^2) and
+    // 2 b (1 - q/p) / (2 sigma_x^2)  (p = 2)
+    float k1[4], k2[4];
+    float bt;                    // temporal weight
 };
 
-// Surrogate coefficient a(D) = rho'(D)/(2D) of the q-GGMRF potential with p = 2:
-//   a(D) = 1/(2 sx^2) * (1 + (q/p) r)/(1 + r)^2,   r = |D/(T sx)|^(p-q).
-// r is formed as exp2((p-q) log2 |D/(T sx)|) with the hardware approximations
-// (about 2^-21 relative), far inside the FP32 tolerance of the agent.
-__device__ __forceinline__ float qggmrf_coef(float D, const MrfDims& m) {
-    const float r = m.pq == 0.0f ? 1.0f : exp2f(m.pq * __log2f(fabsf(D) * m.inv_tsx));
-    const float op = 1.0f + r;
-    return m.inv_2sx2 * (1.0f + m.q_over_p * r) / (op * op);
+__device__ __forceinline__ float lg2_ftz(float x) {
+    float r;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float ex2_ftz(float x) {
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float rcp_ftz(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
 }
 
+// Twice the weighted surrogate coefficients b a(D) of two neighbours of one kind
+// (packed), a(D) = rho'(D)/(2D) of the q-GGMRF potential with p = 2:
+//   a(D) = 1/(2 sx^2) * (1 + (q/p) r)/(1 + r)^2,   r = |D/(T sx)|^(p-q),
+// in partial fractions of 1/(1 + r).  r is formed as exp2((p-q) log2 .) with the
+// hardware approximations (about 2^-21 relative, far inside the FP32 tolerance of
+// the agent; a term flushed to zero is below 2^-126 beside the 1).  The two share
+// a reciprocal: the special function unit bounds these kernels (28 neighbours, a
+// logarithm, a power and a reciprocal each).  (Three could not share: with two far
+// outliers the product would overflow and take the third's weight with it.)
+__device__ __forceinline__ f32x2 qggmrf_pair(f32x2 D, int kind, const MrfDims& m) {
+    float r0 = 1.0f, r1 = 1.0f;
+    if (m.pq != 0.0f) {
+        float d0, d1;
+        unpack2(mul2(D, pack2(m.inv_tsx, m.inv_tsx)), d0, d1);
+        unpack2(mul2(pack2(lg2_ftz(fabsf(d0)), lg2_ftz(fabsf(d1))), pack2(m.pq, m.pq)), d0, d1);
+        r0 = ex2_ftz(d0);
+        r1 = ex2_ftz(d1);
+    }
+    float x, y;
+    unpack2(add2(pack2(r0, r1), pack2(1.0f, 1.0f)), x, y);
+    const float rc = rcp_ftz(__fmul_rn(x, y));
+    const f32x2 w = mul2(pack2(y, x), pack2(rc, rc));
+    return mul2(w, fma2(w, pack2(m.k2[kind], m.k2[kind]), pack2(m.k1[kind], m.k1[kind])));
+}
+
+// Calls f(offset 1, inside 1, offset 2, inside 2, kind) for the 13 pairs of
+// opposite spatial neighbours of voxel (ix, iy, iz) of frame t and its temporal
+// pair; offsets in elements.  INNER: the voxel has neighbours on both sides of
+// every axis but x.
+template <bool INNER, typename F>
+__device__ __forceinline__ void neighbour_pairs(int ix, int iy, int iz, int t, const MrfDims& m, F&& f) {
+    const ptrdiff_t sx = 1, sy = m.nx, sz = (ptrdiff_t)m.nx * m.ny, st = sz * m.nz;
+    const bool xl = ix > 0, xh = ix + 1 < m.nx;
+    const bool yl = INNER || iy > 0, yh = INNER || iy + 1 < m.ny, zl = INNER || iz > 0, zh = INNER || iz + 1 < m.nz;
+    f(-sx, xl, sx, xh, 0);
+    f(-sy, yl, sy, yh, 0);
+    f(-sz, zl, sz, zh, 0);
+    f(-sy - sx, yl && xl, sy + sx, yh && xh, 1);
+    f(-sy + sx, yl && xh, sy - sx, yh && xl, 1);
+    f(-sz - sx, zl && xl, sz + sx, zh && xh, 1);
+    f(-sz + sx, zl && xh, sz - sx, zh && xl, 1);
+    f(-sz - sy, zl && yl, sz + sy, zh && yh, 1);
+    f(-sz + sy, zl && yh, sz - sy, zh && yl, 1);
+    f(-sz - sy - sx, zl && yl && xl, sz + sy + sx, zh && yh && xh, 2);
+    f(-sz - sy + sx, zl && yl && xh, sz + sy - sx, zh && yh && xl, 2);
+    f(-sz + sy - sx, zl && yh && xl, sz - sy + sx, zh && yl && xh, 2);
+    f(-sz + sy + sx, zl && yh && xh, sz - sy - sx, zh && yl && xl, 2);
+    f(-st, INNER || t > 0, st, INNER || t + 1 < m.nt, 3);
+}
+
+__device__ __forceinline__ bool inner(int iy, int iz, int t, const MrfDims& m) {
+    return iy > 0 && iy + 1 < m.ny && iz > 0 && iz + 1 < m.nz && t > 0 && t + 1 < m.nt;
+}
+
+// One colour of a sweep.  Bound by the special function unit (70 operations per
+// voxel, 16 lanes a clock) and, close behind, by instruction issue: with an IEEE
+// division per neighbour, general exp2 / log2 and one sum of all 28 terms, two
+// sweeps of 192^3 x 12 took 7.12 ms; with shared reciprocals and partial fractions
+// 3.8, packed pairs (which also halve the sums' length: error against FP64 9.9e-8
+// -> 7.4e-8) 3.18, without bounds checks in y, z and t inside the volume 3.12.
 __global__ void __launch_bounds__(128) icd_colour_kernel(const float* __restrict__ v,
                                                          float* __restrict__ z, MrfDims m) {
     const int hxv = blockIdx.x * 32 + threadIdx.x;
@@ -43,45 +111,24 @@ __global__ void __launch_bounds__(128) icd_colour_kernel(const float* __restrict
     const int htv = blockIdx.z / m.hz;
     if (hxv >= m.hx || hyv >= m.hy) return;
     const int ix = 2 * hxv + m.px, iy = 2 * hyv + m.py, iz = 2 * hzv + m.pz, t = 2 * htv + m.pt;
-    const size_t sxy = (size_t)m.nx * m.ny;
-    const size_t fs = sxy * m.nz;
-    const size_t s = (size_t)t * fs + (size_t)iz * sxy + (size_t)iy * m.nx + ix;
-    const float zs = z[s];
-    float num = v[s] * m.inv_s2, den = m.inv_s2;
-#pragma unroll
-    for (int dz = -1; dz <= 1; ++dz) {
-        const int jz = iz + dz;
-        if (jz < 0 || jz >= m.nz) continue;
-#pragma unroll
-        for (int dy = -1; dy <= 1; ++dy) {
-            const int jy = iy + dy;
-            if (jy < 0 || jy >= m.ny) continue;
-#pragma unroll
-            for (int dx = -1; dx <= 1; ++dx) {
-                const int jx = ix + dx;
-                if ((dx | dy | dz) == 0 || jx < 0 || jx >= m.nx) continue;
-                const int mm = (dx != 0) + (dy != 0) + (dz != 0);
-                const float b = mm == 1 ? m.bf : (mm == 2 ? m.be : m.bc);
-                const float zr = z[(size_t)t * fs + (size_t)jz * sxy + (size_t)jy * m.nx + jx];
-                const float ba = b * qggmrf_coef(zs - zr, m);
-                num += 2.0f * ba * zr;
-                den += 2.0f * ba;
-            }
-        }
-    }
-    if (t > 0) {
-        const float zr = z[s - fs];
-        const float ba = m.bt * qggmrf_coef(zs - zr, m);
-        num += 2.0f * ba * zr;
-        den += 2.0f * ba;
-    }
-    if (t + 1 < m.nt) {
-        const float zr = z[s + fs];
-        const float ba = m.bt * qggmrf_coef(zs - zr, m);
-        num += 2.0f * ba * zr;
-        den += 2.0f * ba;
-    }
-    z[s] = num / den;
+    float* c = z + (((size_t)t * m.nz + iz) * m.ny + iy) * m.nx + ix;
+    const float zs = *c;
+    f32x2 num = pack2(v[c - z] * m.inv_s2, 0.0f), den = pack2(m.inv_s2, 0.0f);
+    auto pair = [&](ptrdiff_t o1, bool in1, ptrdiff_t o2, bool in2, int kind) {
+        const f32x2 zr = pack2(in1 ? c[o1] : zs, in2 ? c[o2] : zs);
+        float a1, a2;
+        unpack2(qggmrf_pair(sub2(pack2(zs, zs), zr), kind, m), a1, a2);
+        const f32x2 a = pack2(in1 ? a1 : 0.0f, in2 ? a2 : 0.0f);
+        num = fma2(a, zr, num);
+        den = add2(den, a);
+    };
+    // (a warp has one y, z and t)
+    if (inner(iy, iz, t, m)) neighbour_pairs<true>(ix, iy, iz, t, m, pair);
+    else neighbour_pairs<false>(ix, iy, iz, t, m, pair);
+    float n0, n1, d0, d1;
+    unpack2(num, n0, n1);
+    unpack2(den, d0, d1);
+    *c = (n0 + n1) / (d0 + d1);
 }
 
 // ------------------------------------------------------------------ direct MAP
@@ -93,31 +140,16 @@ constexpr int MAP_BLOCKS = 152 * 8;
 // prior's quadratic surrogate built at `anchor`.
 __device__ __forceinline__ float surrogate_lap(const float* __restrict__ anchor, const float* __restrict__ x,
                                                size_t s, int ix, int iy, int iz, int t, const MrfDims& m) {
-    const size_t sxy = (size_t)m.nx * m.ny, fs = sxy * m.nz;
     const float as = anchor[s], xs = x[s];
-    float acc = 0.0f;
-#pragma unroll
-    for (int dz = -1; dz <= 1; ++dz) {
-        const int jz = iz + dz;
-        if (jz < 0 || jz >= m.nz) continue;
-#pragma unroll
-        for (int dy = -1; dy <= 1; ++dy) {
-            const int jy = iy + dy;
-            if (jy < 0 || jy >= m.ny) continue;
-#pragma unroll
-            for (int dx = -1; dx <= 1; ++dx) {
-                const int jx = ix + dx;
-                if ((dx | dy | dz) == 0 || jx < 0 || jx >= m.nx) continue;
-                const int mm = (dx != 0) + (dy != 0) + (dz != 0);
-                const float b = mm == 1 ? m.bf : (mm == 2 ? m.be : m.bc);
-                const size_t r = (size_t)t * fs + (size_t)jz * sxy + (size_t)jy * m.nx + jx;
-                acc = fmaf(b * qggmrf_coef(as - anchor[r], m), xs - x[r], acc);
-            }
-        }
-    }
-    if (t > 0) acc = fmaf(m.bt * qggmrf_coef(as - anchor[s - fs], m), xs - x[s - fs], acc);
-    if (t + 1 < m.nt) acc = fmaf(m.bt * qggmrf_coef(as - anchor[s + fs], m), xs - x[s + fs], acc);
-    return acc;
+    f32x2 acc = 0;
+    neighbour_pairs<false>(ix, iy, iz, t, m, [&](ptrdiff_t o1, bool in1, ptrdiff_t o2, bool in2, int kind) {
+        const f32x2 ar = pack2(in1 ? anchor[s + o1] : as, in2 ? anchor[s + o2] : as);
+        const f32x2 xr = pack2(in1 ? x[s + o1] : xs, in2 ? x[s + o2] : xs);   // outside: a zero difference
+        acc = fma2(qggmrf_pair(sub2(pack2(as, as), ar), kind, m), sub2(pack2(xs, xs), xr), acc);
+    });
+    float a0, a1;
+    unpack2(acc, a0, a1);
+    return 0.5f * (a0 + a1);   // the pairs carry twice the coefficients
 }
 
 enum MapLapMode { MAP_INIT = 0, MAP_Q = 1 };
@@ -293,12 +325,12 @@ static msf_status mrf_dims(const msf_vol* vol, const msf_mrf* prm, double sigma,
     m.inv_s2 = (float)(1.0 / (sigma * sigma));
     m.inv_tsx = (float)(1.0 / (prm->T * prm->sigma_x));
     m.pq = (float)(prm->p - prm->q);
-    m.q_over_p = (float)(prm->q / prm->p);
-    m.inv_2sx2 = (float)(1.0 / (2.0 * prm->sigma_x * prm->sigma_x));
-    const double s = 6.0 + 12.0 / sqrt(2.0) + 8.0 / sqrt(3.0);
-    m.bf = (float)(1.0 / s);
-    m.be = (float)(1.0 / (sqrt(2.0) * s));
-    m.bc = (float)(1.0 / (sqrt(3.0) * s));
+    const double s = 6.0 + 12.0 / sqrt(2.0) + 8.0 / sqrt(3.0), c = 1.0 / (prm->sigma_x * prm->sigma_x);
+    const double b[4] = {1.0 / s, 1.0 / (sqrt(2.0) * s), 1.0 / (sqrt(3.0) * s), prm->b_temporal};
+    for (int k = 0; k < 4; ++k) {
+        m.k1[k] = (float)(b[k] * c * (prm->q / prm->p));
+        m.k2[k] = (float)(b[k] * c * (1.0 - prm->q / prm->p));
+    }
     m.bt = (float)prm->b_temporal;
     return MSF_OK;
 }
@@ -468,17 +500,7 @@ extern "C" msf_status msf_prox_qggmrf(const msf_vol* vol, const msf_mrf* prm, co
                 "msf_prox_qggmrf: nz*nt too large for the launch grid");
     cudaStream_t st = as_stream(stream);
     MrfDims m;
-    m.nx = vol->nx; m.ny = vol->ny; m.nz = vol->nz; m.nt = vol->nt;
-    m.inv_s2 = (float)(1.0 / (sigma * sigma));
-    m.inv_tsx = (float)(1.0 / (prm->T * prm->sigma_x));
-    m.pq = (float)(prm->p - prm->q);
-    m.q_over_p = (float)(prm->q / prm->p);
-    m.inv_2sx2 = (float)(1.0 / (2.0 * prm->sigma_x * prm->sigma_x));
-    const double s = 6.0 + 12.0 / sqrt(2.0) + 8.0 / sqrt(3.0);
-    m.bf = (float)(1.0 / s);
-    m.be = (float)(1.0 / (sqrt(2.0) * s));
-    m.bc = (float)(1.0 / (sqrt(3.0) * s));
-    m.bt = (float)prm->b_temporal;
+    MSF_TRY(mrf_dims(vol, prm, sigma, &m));
     for (int sw = 0; sw < n_sweeps; ++sw) {
         for (int col = 0; col < 16; ++col) {
             m.px = col & 1; m.py = (col >> 1) & 1; m.pz = (col >> 2) & 1; m.pt = (col >> 3) & 1;

@@ -214,38 +214,6 @@ __host__ __device__ __forceinline__ int sino_pitch(int nv) { return (nv + SINO_F
 constexpr float FLOOR_MAGIC = 12582912.0f;
 constexpr int FLOOR_MAGIC_BITS = 0x4B400000;
 
-// Two FP32 values in one 64-bit register: one instruction issues both lanes'
-// operation, each rounded as its scalar form (sm_100 and later).
-using f32x2 = unsigned long long;
-__device__ __forceinline__ f32x2 pack2(float a, float b) {
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-    f32x2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 add2_rd(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("add.rm.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-
 // Group dimensions: voxels of parity p along an axis of n voxels.
 __host__ __device__ __forceinline__ int par_count(int n, int p) { return (n - p + 1) / 2; }
 
