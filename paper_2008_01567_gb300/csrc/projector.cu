@@ -536,7 +536,8 @@ struct __align__(16) AdjEntry {
     float2 wb;           // 1 - wa: weight of the line before it
     const float* row0;   // the column's row 0, less FLOOR_MAGIC_BITS elements
 };
-constexpr int ADJ_FAST = 32;   // slot flag: two rows per footprint, none outside the line's margins
+// slot flags: two or three rows per footprint, no window outside the line's margins
+constexpr int ADJ_TWO = 32, ADJ_THREE = 16;
 
 __device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ f32x2 vfma(f32x2 a, f32x2 b, f32x2 c) { return fma2(a, b, c); }
@@ -567,10 +568,11 @@ __device__ __forceinline__ f32x2 vbc(float2 a, f32x2) { return pack2(a.x, a.y); 
 // the voxels V of a lane (one, or two packed).  f_z(iv) - z = (iv - cv) dfz +
 // (cz - z), both bracketed terms exact, so only dfz carries a rounding.  The
 // window starts at the first row with f_z > z - 1 and holds NR rows (NR = 0:
-// `rows`, any number); all but its last lie inside the voxel's footprint, and
-// the last is dropped where it does not, so that a non-finite reading reaches
-// the voxels of its own footprint only.  CLAMP: the window may lie outside the
-// detector.  SQ: squared weights.
+// `rows`, any number).  CLAMP: the window may lie outside the detector, and hold
+// more rows than a footprint (2 / dfz, rounded up); otherwise all rows but its
+// last lie inside the footprint.  A row outside it is dropped, so that a
+// non-finite reading reaches the voxels of its own footprint only.  SQ: squared
+// weights.
 template <int NR, bool CLAMP, bool SQ, typename V>
 __device__ __forceinline__ V row_sum(const AdjEntry& q, int rows, V zc, const ProjDims& d) {
     using L = Lanes<V>;
@@ -601,7 +603,7 @@ __device__ __forceinline__ V row_sum(const AdjEntry& q, int rows, V zc, const Pr
             if (SQ) w[k] = __fmul_rn(w[k], w[k]);
             if (NR) ev[k] = __ldg(q.row0 + row);
             else ev[k] = (unsigned)(row - FLOOR_MAGIC_BITS) < (unsigned)d.nv ? __ldg(q.row0 + row) : 0.0f;
-            if (i == n - 1 || !NR) ev[k] = w[k] > 0.0f ? ev[k] : 0.0f;
+            if (i == n - 1 || CLAMP) ev[k] = w[k] > 0.0f ? ev[k] : 0.0f;
         }
         s = vfma(L::pack(w), L::pack(ev), s);
         if (i + 1 < n) df = vadd(df, dfz);
@@ -658,24 +660,30 @@ __device__ __forceinline__ void row_sums(const AdjEntry& q, int rows, const AdjA
 // whose f_a, formed with the forward's own operations (bit for bit), touches the
 // run.  The warp then walks the list, its lanes taking voxels along z.  The order
 // of a voxel's terms (groups of views, columns in each) does not depend on J.
+// Part `part` of `parts` takes every parts-th group of views.
 template <bool XMAJ, int J, int STR, bool SQ>
 __device__ __forceinline__ void gather_run(const float4* __restrict__ col, const float2* __restrict__ trig,
                                            const int* __restrict__ vflag, const float* __restrict__ e, int t, int kpl,
-                                           int a_lo, int z_lo, const AdjAcc<J>& zc, const ProjDims& d, int slots,
-                                           AdjEntry* __restrict__ list, int* __restrict__ slot, AdjAcc<J>* acc) {
+                                           int a_lo, int z_lo, const AdjAcc<J>& zc, const ProjDims& d, int slots, int part,
+                                           int parts, AdjEntry* __restrict__ list, int* __restrict__ slot,
+                                           AdjAcc<J>* acc) {
     const int lane = threadIdx.x;
     const int na = XMAJ ? d.ny : d.nx, nvp = sino_pitch(d.nv);
     const int a_hi = min(a_lo + STR * (ADJ_T - 1) + 1, na);
     const float tk = __fsub_rn((float)kpl, XMAJ ? d.cx : d.cy);
     const float maj = tk * d.vox, lo = (a_lo - 1 - (XMAJ ? d.cy : d.cx)) * d.vox, hi = (a_hi - (XMAJ ? d.cy : d.cx)) * d.vox;
     const float margin = 0.01f + 4e-6f * d.nu;
-    const int vstep = 32 / slots, vi = lane / slots, ci = lane - vi * slots;
-    for (int v0 = 0; v0 < d.views; v0 += vstep) {
+    // views of a group: as many as the lanes take, but no fewer groups than parts
+    const int vstep = min(32 / slots, (d.views + parts - 1) / parts), vi = lane / slots, ci = lane - vi * slots;
+    for (int v0 = part * vstep; v0 < d.views; v0 += parts * vstep) {
         const int v = v0 + vi, g = t * d.views + v;
         int iu = d.nu, iu_hi = -1, flags = 0;
-        if (vi < vstep && v < d.views) flags = __ldg(vflag + g);
+        float2 cs = make_float2(0.0f, 0.0f);
+        if (vi < vstep && v < d.views) {
+            flags = __ldg(vflag + g);
+            cs = __ldg(trig + g);
+        }
         if (flags & (XMAJ ? 1 : 2)) {
-            const float2 cs = __ldg(trig + g);
             const float x1 = XMAJ ? maj : lo, y1 = XMAJ ? lo : maj, x2 = XMAJ ? maj : hi, y2 = XMAJ ? hi : maj;
             // an end beside the source projects anywhere: try every column
             const bool near = fminf(d.dso - x1 * cs.x - y1 * cs.y, d.dso - x2 * cs.x - y2 * cs.y) < 0.05f * d.dso;
@@ -710,12 +718,11 @@ __device__ __forceinline__ void gather_run(const float4* __restrict__ col, const
                 q.wa = make_float2(wa, wa);
                 q.wb = make_float2(wb, wb);
                 q.row0 = e + gcol * nvp + SINO_FRONT - FLOOR_MAGIC_BITS;
-                // two rows per footprint (1 <= dfz < 2) and every window of the
-                // run inside the line's margins
+                // every window of the run's voxels inside the line's margins
                 const float t_lo = __fmaf_rn(d.cz - (float)z_lo, -rdfz, c0);
-                const float t_hi = __fmaf_rn(d.cz - (float)(z_lo + STR * (32 * J - 1)), -rdfz, c0);
-                if (rdfz <= 1.0f && rdfz > 0.5f && t_lo > 1.0f - SINO_FRONT && t_hi < (float)(d.nv + SINO_BACK - 3))
-                    fast = ADJ_FAST;
+                const float t_hi = __fmaf_rn(d.cz - (float)min(z_lo + STR * (32 * J - 1), d.nz - 1), -rdfz, c0);
+                if (t_lo > 1.0f - SINO_FRONT && t_hi < (float)(d.nv + SINO_BACK - 4))
+                    fast = rdfz > 0.5f && rdfz <= 1.0f ? ADJ_TWO : rdfz > 1.0f && rdfz <= 1.5f ? ADJ_THREE : 0;
             }
             const unsigned mask = __ballot_sync(0xffffffffu, ok);
             if (ok) {
@@ -729,12 +736,13 @@ __device__ __forceinline__ void gather_run(const float4* __restrict__ col, const
                 const AdjEntry q = list[i];
                 const int sl = slot[i];
                 AdjAcc<J> s;
-                if (sl >= ADJ_FAST) row_sums<2, false, SQ, J>(q, 0, zc, d, s);
-                else {
+                if (sl >= ADJ_TWO) {
+                    row_sums<2, false, SQ, J>(q, 0, zc, d, s);
+                } else if (sl >= ADJ_THREE) {
+                    row_sums<3, false, SQ, J>(q, 0, zc, d, s);
+                } else {
                     const float span = -2.0f * q.nrdfz.x;   // rows per footprint: ceil(2 / dfz)
-                    if (span <= 1.0f) row_sums<1, true, SQ, J>(q, 0, zc, d, s);
-                    else if (span <= 2.0f) row_sums<2, true, SQ, J>(q, 0, zc, d, s);
-                    else if (span <= 3.0f) row_sums<3, true, SQ, J>(q, 0, zc, d, s);
+                    if (span <= 3.0f) row_sums<3, true, SQ, J>(q, 0, zc, d, s);
                     else row_sums<0, true, SQ, J>(q, (int)fminf(ceilf(span), (float)(d.nv + 8)), zc, d, s);
                 }
                 if (STR == 2) {
@@ -763,6 +771,75 @@ __device__ __forceinline__ void gather_run(const float4* __restrict__ col, const
 // with 5, 2.22 with none; 128^3 x 8, J = 4: 0.67 with 6, 0.73 with none).
 __host__ __device__ constexpr int adj_min_blocks(int J) { return J >= 8 ? 4 : J >= 5 ? 5 : J >= 3 ? 6 : 8; }
 
+// Both phases of a block on the lines x0 + STR i, y0 + STR w, voxels z_lo + STR (lane
+// + 32 j): leaves in acc[i] the sums of the lines of y = y0 + STR w (none if that
+// lies outside the volume).  VS sets of ADJ_T warps share the views (a small
+// volume has too few tiles to fill the GPU, and a warp's walk over the views sets
+// its time); the first set holds the result.
+template <int J, int VS>
+struct AdjShared {
+    AdjEntry list[ADJ_T * VS][ADJ_ENTRIES];
+    int slot[ADJ_T * VS][ADJ_ENTRIES];
+};
+
+template <int J, int VS, int STR, bool SQ>
+__device__ __forceinline__ void gather_tile(const float4* __restrict__ col, const float2* __restrict__ trig,
+                                            const int* __restrict__ vflag, const float* __restrict__ e, int t, int x0,
+                                            int y0, int z_lo, const ProjDims& d, int slots, float* adj_tile,
+                                            AdjShared<J, VS>& sh, AdjAcc<J>* acc) {
+    const int lane = threadIdx.x, wv = threadIdx.y, w = VS == 1 ? wv : wv % ADJ_T, part = VS == 1 ? 0 : wv / ADJ_T;
+    AdjAcc<J> zc;
+    {
+        float a[J];   // voxels past the volume repeat its last one
+#pragma unroll
+        for (int j = 0; j < J; ++j) a[j] = d.cz - (float)min(z_lo + STR * (lane + 32 * j), d.nz - 1);
+        zc.set(a);
+    }
+    float* all = adj_tile + part * ADJ_T * ADJ_T * adj_line(J);
+    float* tile = all + w * ADJ_T * adj_line(J);   // the lines of y = y0 + STR w
+    auto put = [&](float* line, int stride) {
+#pragma unroll
+        for (int i = 0; i < ADJ_T; ++i) {
+            float v[J];
+            acc[i].get(v);
+#pragma unroll
+            for (int j = 0; j < J; ++j) line[i * stride + 32 * j + lane] = v[j];
+        }
+    };
+#pragma unroll
+    for (int i = 0; i < ADJ_T; ++i) acc[i].zero();
+    if (x0 + STR * w < d.nx)
+        gather_run<true, J, STR, SQ>(col, trig, vflag, e, t, x0 + STR * w, y0, z_lo, zc, d, slots, part, VS, sh.list[wv],
+                                     sh.slot[wv], acc);
+    put(all + w * adj_line(J), ADJ_T * adj_line(J));
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < ADJ_T; ++i) {
+        float v[J];
+#pragma unroll
+        for (int j = 0; j < J; ++j) v[j] = tile[i * adj_line(J) + 32 * j + lane];
+        acc[i].set(v);
+    }
+    if (y0 + STR * w < d.ny)
+        gather_run<false, J, STR, SQ>(col, trig, vflag, e, t, y0 + STR * w, x0, z_lo, zc, d, slots, part, VS, sh.list[wv],
+                                      sh.slot[wv], acc);
+    if (VS > 1) {   // the parts' sums in order
+        if (part > 0) put(tile, adj_line(J));
+        __syncthreads();
+        if (part > 0) return;
+#pragma unroll
+        for (int i = 0; i < ADJ_T; ++i) {
+            float v[J];
+            acc[i].get(v);
+            for (int k = 1; k < VS; ++k)
+#pragma unroll
+                for (int j = 0; j < J; ++j)
+                    v[j] = __fadd_rn(v[j], tile[(k * ADJ_T * ADJ_T + i) * adj_line(J) + 32 * j + lane]);
+            acc[i].set(v);
+        }
+    }
+}
+
 // A block takes ADJ_T x ADJ_T voxel lines and 32 J voxels of each; lane = z, so
 // that a warp's loads run along the detector rows.  First warp w takes the lines
 // of x = x0 + w for the x-major rays, then, the sums handed over through shared
@@ -782,60 +859,13 @@ __host__ __device__ constexpr int adj_min_blocks(int J) { return J >= 8 ? 4 : J 
 //   ADJ_CG_Q:    q = A^T e + p/sigma^2, alpha = rr / p.q      (a1 = p)
 //   ADJ_THETA2:  (A.^2)^T e + 1/sigma^2 (the ICD agent's curvature)
 // (the CG's vectors as lines, the volume of ADJ_PLAIN as [nt][nz][ny][nx])
-struct AdjShared {
-    AdjEntry list[ADJ_T][ADJ_ENTRIES];
-    int slot[ADJ_T][ADJ_ENTRIES];
-};
-
-// Both phases of a block on the lines x0 + STR i, y0 + STR w, voxels z_lo + STR (lane
-// + 32 j): leaves in acc[i] the sums of the lines of y = y0 + STR w (none if that
-// lies outside the volume).
-template <int J, int STR, bool SQ>
-__device__ __forceinline__ void gather_tile(const float4* __restrict__ col, const float2* __restrict__ trig,
-                                            const int* __restrict__ vflag, const float* __restrict__ e, int t, int x0,
-                                            int y0, int z_lo, const ProjDims& d, int slots, float* adj_tile,
-                                            AdjShared& sh, AdjAcc<J>* acc) {
-    const int lane = threadIdx.x, w = threadIdx.y;
-    AdjAcc<J> zc;
-    {
-        float a[J];
-#pragma unroll
-        for (int j = 0; j < J; ++j) a[j] = d.cz - (float)(z_lo + STR * (lane + 32 * j));
-        zc.set(a);
-    }
-#pragma unroll
-    for (int i = 0; i < ADJ_T; ++i) acc[i].zero();
-    if (x0 + STR * w < d.nx)
-        gather_run<true, J, STR, SQ>(col, trig, vflag, e, t, x0 + STR * w, y0, z_lo, zc, d, slots, sh.list[w], sh.slot[w],
-                                     acc);
-#pragma unroll
-    for (int i = 0; i < ADJ_T; ++i) {
-        float v[J];
-        acc[i].get(v);
-#pragma unroll
-        for (int j = 0; j < J; ++j) adj_tile[(i * ADJ_T + w) * adj_line(J) + 32 * j + lane] = v[j];
-    }
-    __syncthreads();
-    const float* tile = adj_tile + w * ADJ_T * adj_line(J);   // the lines of y = y0 + STR w
-#pragma unroll
-    for (int i = 0; i < ADJ_T; ++i) {
-        float v[J];
-#pragma unroll
-        for (int j = 0; j < J; ++j) v[j] = tile[i * adj_line(J) + 32 * j + lane];
-        acc[i].set(v);
-    }
-    if (y0 + STR * w < d.ny)
-        gather_run<false, J, STR, SQ>(col, trig, vflag, e, t, y0 + STR * w, x0, z_lo, zc, d, slots, sh.list[w],
-                                      sh.slot[w], acc);
-}
-
-template <int MODE, int J>
-__global__ void __launch_bounds__(32 * ADJ_T, adj_min_blocks(J)) joseph_adj_kernel(
+template <int MODE, int J, int VS>
+__global__ void __launch_bounds__(32 * ADJ_T * VS, adj_min_blocks(J) >= VS ? adj_min_blocks(J) / VS : 1) joseph_adj_kernel(
     const float4* __restrict__ col, const float2* __restrict__ trig, const int* __restrict__ vflag,
     const float* __restrict__ e, float* __restrict__ out, const float* __restrict__ a1, float* __restrict__ out2,
     CgScalars cg, float inv_s2, ProjDims d, int slots) {
     extern __shared__ float adj_tile[];   // [y][x][adj_line(J)]
-    __shared__ AdjShared sh;
+    __shared__ AdjShared<J, VS> sh;
     const int lane = threadIdx.x, w = threadIdx.y;
     const int nzb = (d.nz + 32 * J - 1) / (32 * J);
     const int zb = blockIdx.z % nzb, t = blockIdx.z / nzb;
@@ -845,16 +875,16 @@ __global__ void __launch_bounds__(32 * ADJ_T, adj_min_blocks(J)) joseph_adj_kern
         // nothing else would hide its way from memory (19.5 -> 18.1 ms, A^T in the CG
         // at 384^3 x 16)
         const size_t first = (((size_t)t * d.ny + y0 + w) * d.nx + x0) * vz_pitch(d.nz) + VZ_FRONT + zb * 32 * J;
-        for (int k = lane; k < ADJ_T * J && y0 + w < d.ny; k += 32)
+        for (int k = lane; k < ADJ_T * J && w < ADJ_T && y0 + w < d.ny; k += 32)
             if (x0 + k / J < d.nx && zb * 32 * J + k % J * 32 < d.nz)
                 asm volatile("prefetch.global.L2 [%0];" ::"l"(a1 + first + (size_t)(k / J) * vz_pitch(d.nz) + k % J * 32));
     }
     AdjAcc<J> acc[ADJ_T];
-    gather_tile<J, 1, MODE == ADJ_THETA2>(col, trig, vflag, e, t, x0, y0, zb * 32 * J, d, slots, adj_tile, sh, acc);
+    gather_tile<J, VS, 1, MODE == ADJ_THETA2>(col, trig, vflag, e, t, x0, y0, zb * 32 * J, d, slots, adj_tile, sh, acc);
     float* tile = adj_tile + w * ADJ_T * adj_line(J);
     const int iy = y0 + w;
     double dot = 0.0;
-    if (iy < d.ny) {
+    if (w < ADJ_T && iy < d.ny) {
         if (MODE == ADJ_PLAIN) {
             // the volume is contiguous along x: ADJ_T lanes write the x of one z
 #pragma unroll
@@ -1024,23 +1054,23 @@ __global__ void __launch_bounds__(256) cg_direction_kernel(float* __restrict__ z
 // joseph_adj_kernel, in voxels of the group: 314 -> 89 us at 96^3 x 6, 160 x 128, 24
 // views; with delta projected straight from its lines, the line search's sum in
 // that projection and both updates in one launch, three sweeps 14.7 -> 5.8 ms.
-template <int J>
-__global__ void __launch_bounds__(32 * ADJ_T, adj_min_blocks(J)) icd_group_kernel(
+template <int J, int VS>
+__global__ void __launch_bounds__(32 * ADJ_T * VS, adj_min_blocks(J) >= VS ? adj_min_blocks(J) / VS : 1) icd_group_kernel(
     const float4* __restrict__ col, const float2* __restrict__ trig, const int* __restrict__ vflag,
     const float* __restrict__ e, const float* __restrict__ z, const float* __restrict__ v,
     const float* __restrict__ theta2, float* __restrict__ dlt, IcdSums S, float inv_s2, IcdGroup G, ProjDims d,
     int slots) {
     extern __shared__ float adj_tile[];
-    __shared__ AdjShared sh;
+    __shared__ AdjShared<J, VS> sh;
     const int lane = threadIdx.x, w = threadIdx.y;
     const int pairs = (d.nz + 1) / 2, nzb = (pairs + 32 * J - 1) / (32 * J);
     const int zb = blockIdx.z % nzb, t = blockIdx.z / nzb;
     const int x0 = G.px + 2 * ADJ_T * blockIdx.x, y0 = G.py + 2 * ADJ_T * blockIdx.y, m0 = zb * 32 * J;
     AdjAcc<J> acc[ADJ_T];
-    gather_tile<J, 2, false>(col, trig, vflag, e, t, x0, y0, G.pz + 2 * m0, d, slots, adj_tile, sh, acc);
+    gather_tile<J, VS, 2, false>(col, trig, vflag, e, t, x0, y0, G.pz + 2 * m0, d, slots, adj_tile, sh, acc);
     const int iy = y0 + 2 * w, nzp = vz_pitch(d.nz);
     double gd = 0.0, dd = 0.0;
-    if (iy < d.ny) {
+    if (w < ADJ_T && iy < d.ny) {
         const size_t first = (((size_t)t * d.ny + iy) * d.nx + x0) * nzp + VZ_FRONT;
 #pragma unroll
         for (int i = 0; i < ADJ_T; ++i) {
@@ -1314,6 +1344,15 @@ static int adj_j(int nz, int zrun) {
     const int J = (sets + blocks - 1) / blocks;
     return J <= 6 ? J : (J + 1) & ~1;
 }
+// Sets of warps that share a tile's views: by the lines of a frame alone (not by
+// the frames, the z-run or the GPU's load, since it groups a voxel's terms).  A^T
+// with its step weighting at 24^3 x 4, 32 x 32, 12 views: 37 us with one set, 30
+// with two, 26 with four; 40^3 x 4 (100 tiles): 45, 39, 43; 64^3 x 4 (256): 50, 61,
+// 69.  A tall volume fills the GPU along z.
+static int adj_parts_of_views(const ProjDims& d, int lines_x, int lines_y) {
+    const long long tiles = (long long)((lines_x + ADJ_T - 1) / ADJ_T) * ((lines_y + ADJ_T - 1) / ADJ_T);
+    return d.nz > 64 ? 1 : tiles <= 64 ? 4 : tiles <= 128 ? 2 : 1;
+}
 // Columns that a run of ADJ_T lines, str voxels apart, has on the axis, and one more.
 static int adj_slots(const ProjDims& d, int str) {
     const double n = ceil((str * (ADJ_T - 1) + 2) * (double)d.vox * d.dsd / d.dso / d.du) + 1.0;
@@ -1331,23 +1370,22 @@ static void launch_adj_zb(msf_projector* p, const float* e, float* out, const fl
                           const CgScalars& cg, float inv_s2, cudaStream_t st) {
     const ProjDims& d = p->dims;
     const int J = adj_j(d.nz, p->adj_zb), slots = adj_slots(d, 1);
-    const dim3 block(32, ADJ_T), grid = adj_grid(d, p->adj_zb);
+    const dim3 grid = adj_grid(d, p->adj_zb);
     const size_t smem = (size_t)ADJ_T * ADJ_T * adj_line(J) * sizeof(float);
-#define MSF_ADJ_CASE(N)                                                                                             \
-    case N:                                                                                                         \
-        joseph_adj_kernel<MODE, N><<<grid, block, smem, st>>>(p->d_col, p->d_trig, p->d_vflag, e, out, a1, out2, cg, \
-                                                               inv_s2, d, slots);                                   \
-        break;
+#define MSF_ADJ_CASE(N, P)                                                                                          \
+    joseph_adj_kernel<MODE, N, P><<<grid, dim3(32, ADJ_T * P), smem * P, st>>>(p->d_col, p->d_trig, p->d_vflag, e, \
+                                                                               out, a1, out2, cg, inv_s2, d, slots)
+    const int parts = adj_parts_of_views(d, d.nx, d.ny);
     switch (J) {
-        MSF_ADJ_CASE(1)
-        MSF_ADJ_CASE(2)
-        MSF_ADJ_CASE(3)
-        MSF_ADJ_CASE(4)
-        MSF_ADJ_CASE(5)
-        MSF_ADJ_CASE(6)
-        MSF_ADJ_CASE(8)
-        MSF_ADJ_CASE(10)
-        MSF_ADJ_CASE(12)
+        case 1: if (parts == 4) MSF_ADJ_CASE(1, 4); else if (parts == 2) MSF_ADJ_CASE(1, 2); else MSF_ADJ_CASE(1, 1); break;
+        case 2: if (parts == 4) MSF_ADJ_CASE(2, 4); else if (parts == 2) MSF_ADJ_CASE(2, 2); else MSF_ADJ_CASE(2, 1); break;
+        case 3: MSF_ADJ_CASE(3, 1); break;
+        case 4: MSF_ADJ_CASE(4, 1); break;
+        case 5: MSF_ADJ_CASE(5, 1); break;
+        case 6: MSF_ADJ_CASE(6, 1); break;
+        case 8: MSF_ADJ_CASE(8, 1); break;
+        case 10: MSF_ADJ_CASE(10, 1); break;
+        case 12: MSF_ADJ_CASE(12, 1); break;
     }
 #undef MSF_ADJ_CASE
 }
@@ -1371,25 +1409,24 @@ static msf_status launch_icd_group(msf_projector* p, const float* e, const float
                                    cudaStream_t st) {
     const ProjDims& d = p->dims;
     const int J = adj_j((d.nz + 1) / 2, p->adj_zb), slots = adj_slots(d, 2);
-    const dim3 block(32, ADJ_T), grid = icd_grid(d, G.gx, G.gy, p->adj_zb);
+    const dim3 grid = icd_grid(d, G.gx, G.gy, p->adj_zb);
     const size_t smem = (size_t)ADJ_T * ADJ_T * adj_line(J) * sizeof(float);
     S->gblocks = grid.x * grid.y * (grid.z / d.nt);
     MSF_PROF("icd_group", st);
-#define MSF_ICD_CASE(N)                                                                                              \
-    case N:                                                                                                          \
-        icd_group_kernel<N><<<grid, block, smem, st>>>(p->d_col, p->d_trig, p->d_vflag, e, z, v, theta2, dlt, *S,    \
-                                                       inv_s2, G, d, slots);                                         \
-        break;
+#define MSF_ICD_CASE(N, P)                                                                                          \
+    icd_group_kernel<N, P><<<grid, dim3(32, ADJ_T * P), smem * P, st>>>(p->d_col, p->d_trig, p->d_vflag, e, z, v,  \
+                                                                        theta2, dlt, *S, inv_s2, G, d, slots)
+    const int parts = adj_parts_of_views(d, par_count(d.nx, 0), par_count(d.ny, 0));
     switch (J) {
-        MSF_ICD_CASE(1)
-        MSF_ICD_CASE(2)
-        MSF_ICD_CASE(3)
-        MSF_ICD_CASE(4)
-        MSF_ICD_CASE(5)
-        MSF_ICD_CASE(6)
-        MSF_ICD_CASE(8)
-        MSF_ICD_CASE(10)
-        MSF_ICD_CASE(12)
+        case 1: if (parts == 4) MSF_ICD_CASE(1, 4); else if (parts == 2) MSF_ICD_CASE(1, 2); else MSF_ICD_CASE(1, 1); break;
+        case 2: MSF_ICD_CASE(2, 1); break;
+        case 3: MSF_ICD_CASE(3, 1); break;
+        case 4: MSF_ICD_CASE(4, 1); break;
+        case 5: MSF_ICD_CASE(5, 1); break;
+        case 6: MSF_ICD_CASE(6, 1); break;
+        case 8: MSF_ICD_CASE(8, 1); break;
+        case 10: MSF_ICD_CASE(10, 1); break;
+        case 12: MSF_ICD_CASE(12, 1); break;
     }
 #undef MSF_ICD_CASE
     MSF_LAUNCH_CHECK();
