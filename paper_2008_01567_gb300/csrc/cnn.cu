@@ -100,12 +100,21 @@ struct FoldArgs {
     long long w, b, gamma, beta, mean, var;   // offsets into params (-1: none)
 };
 
-// BatchNorm folding and BF16 packing of one layer:
+// All layers of the network: where a layer's packed weights start, and its arguments.
+struct FoldAll {
+    FoldArgs layer[LAYERS];
+    size_t off[LAYERS];
+};
+
+// BatchNorm folding and BF16 packing, one layer per blockIdx.y:
 //   w' = w * g/sqrt(var+eps),  b' = (b - mean) g/sqrt(var+eps) + beta.
 // Layer 1 is packed as a single K = 64 slice in the pack5 order; the last
-// layer's 1 output channel is padded to 16 rows.
-__global__ void fold_kernel(const float* __restrict__ params, __nv_bfloat16* __restrict__ wpack,
-                            float* __restrict__ bias, FoldArgs f) {
+// layer's 1 output channel is padded to 16 rows.  bias: [LAYERS][64].
+__global__ void fold_kernel(const float* __restrict__ params, __nv_bfloat16* __restrict__ wpack0,
+                            float* __restrict__ bias0, const __grid_constant__ FoldAll all) {
+    const FoldArgs& f = all.layer[blockIdx.y];
+    __nv_bfloat16* wpack = wpack0 + all.off[blockIdx.y];
+    float* bias = bias0 + blockIdx.y * CH;
     const int n_el = f.taps * f.rows * KPACK;
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n_el; e += gridDim.x * blockDim.x) {
         const int tap = e / (f.rows * KPACK);
@@ -134,6 +143,22 @@ __global__ void fold_kernel(const float* __restrict__ params, __nv_bfloat16* __r
         }
         bias[n] = bv;
     }
+}
+
+static FoldAll fold_args(const Offsets& o, const size_t* off, bool batchnorm) {
+    FoldAll a;
+    for (int l = 0; l < LAYERS; ++l) {
+        FoldArgs& f = a.layer[l];
+        f.layer = l; f.taps = taps_of(l); f.rows = rows_of(l); f.cin = cin_of(l); f.cout = cout_of(l);
+        f.w = (long long)o.w[l]; f.b = (long long)o.b[l];
+        const bool bn = batchnorm && l > 0 && l < LAYERS - 1;
+        f.gamma = bn ? (long long)o.gamma[l] : -1;
+        f.beta = bn ? (long long)o.beta[l] : -1;
+        f.mean = bn ? (long long)o.mean[l] : -1;
+        f.var = bn ? (long long)o.var[l] : -1;
+        a.off[l] = off[l];
+    }
+    return a;
 }
 
 // ---------------------------------------------------------------- geometry
@@ -1708,24 +1733,9 @@ struct msf_cnn {
 };
 
 static msf_status fold_all(msf_cnn* c, cudaStream_t st) {
-    for (int l = 0; l < LAYERS; ++l) {
-        FoldArgs f;
-        f.layer = l;
-        f.taps = taps_of(l);
-        f.rows = rows_of(l);
-        f.cin = cin_of(l);
-        f.cout = cout_of(l);
-        f.w = (long long)c->off.w[l];
-        f.b = (long long)c->off.b[l];
-        const bool bn = l > 0 && l < LAYERS - 1;
-        f.gamma = bn ? (long long)c->off.gamma[l] : -1;
-        f.beta = bn ? (long long)c->off.beta[l] : -1;
-        f.mean = bn ? (long long)c->off.mean[l] : -1;
-        f.var = bn ? (long long)c->off.var[l] : -1;
-        MSF_PROF("fold", st);
-        fold_kernel<<<64, 256, 0, st>>>(c->d_params, c->d_wpack + c->wpack_off[l], c->d_bias + l * CH, f);
-        MSF_LAUNCH_CHECK();
-    }
+    MSF_PROF("fold", st);
+    fold_kernel<<<dim3(64, LAYERS), 256, 0, st>>>(c->d_params, c->d_wpack, c->d_bias, fold_args(c->off, c->wpack_off, true));
+    MSF_LAUNCH_CHECK();
     c->folded = true;
     return MSF_OK;
 }
@@ -2214,9 +2224,9 @@ static size_t train_layout(int64_t P, TrainWS* w, uint8_t* base) {
 
 // [B][5][H][W] FP32 -> packed BF16 [B][H][W][64] (k = frame*9 + ky*3 + kx).
 __global__ void pack_batch_kernel(const float* __restrict__ x, uint4* __restrict__ out, int B, int H, int W) {
-    const size_t total = (size_t)B * H * W;
-    for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < total; p += (size_t)gridDim.x * blockDim.x) {
-        const int b = (int)(p % W), a = (int)((p / W) % H), img = (int)(p / ((size_t)H * W));
+    const unsigned total = (unsigned)B * H * W;   // at most 2^28
+    for (unsigned p = blockIdx.x * blockDim.x + threadIdx.x; p < total; p += gridDim.x * blockDim.x) {
+        const int b = (int)(p % (unsigned)W), a = (int)(p / (unsigned)W % (unsigned)H), img = (int)(p / ((unsigned)H * W));
         float v[FRAMES * 9];
 #pragma unroll
         for (int c = 0; c < FRAMES; ++c)
@@ -2234,15 +2244,18 @@ __global__ void pack_batch_kernel(const float* __restrict__ x, uint4* __restrict
             __nv_bfloat162 h = __floats2bfloat162_rn(2 * i < 45 ? v[2 * i] : 0.0f, 2 * i + 1 < 45 ? v[2 * i + 1] : 0.0f);
             w[i] = *reinterpret_cast<uint32_t*>(&h);
         }
-        uint4* dst = out + p * 8;
+        uint4* dst = out + (size_t)p * 8;
 #pragma unroll
         for (int c = 0; c < 8; ++c) dst[c] = make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
     }
 }
 
 // Input-gradient kernels of the hidden layers: W'[tap'][ci][co] = W[co][ci][2-ky][2-kx].
-__global__ void pack_dgrad_kernel(const float* __restrict__ params, __nv_bfloat16* __restrict__ wb, Offsets o) {
+// Also clears the zero bias of those convolutions.
+__global__ void pack_dgrad_kernel(const float* __restrict__ params, __nv_bfloat16* __restrict__ wb,
+                                  float* __restrict__ zeros, Offsets o) {
     const int n = 8 * 9 * CH * CH;
+    if (blockIdx.x == 0 && threadIdx.x < CH) zeros[threadIdx.x] = 0.0f;
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
         const int l = 1 + e / (9 * CH * CH);
         const int r = e % (9 * CH * CH);
@@ -2354,27 +2367,28 @@ __global__ void __launch_bounds__(256, 2) bn_bwd_reduce_kernel(const uint4* __re
     }
 }
 
-// Sum over the nblk per-block partials [nblk][2][64] of entry (k, c), by one
-// warp: lane l adds blocks l, l+32, ... in order, then a fixed shuffle tree
-// (the same order on every run); the result is in lane 0.
-__device__ __forceinline__ double warp_partial_sum(const double* __restrict__ part, int nblk, int k, int c, int ln) {
+// Sum over the nblk per-block partials [nblk][2][64] of entry (k, c), by one block
+// of FIN_THREADS threads (in thread 0): every load of a thread in flight at once,
+// and FP64 additions on as many SMs as there are outputs.  (By one warp per output,
+// 38 dependent loads and additions for 1216 partials, the sums took 10 us.)
+constexpr int FIN_THREADS = 128;
+__device__ __forceinline__ double block_partial_sum(const double* __restrict__ part, int nblk, int k, int c) {
     double s = 0.0;
-    for (int b = ln; b < nblk; b += 32) s += part[((size_t)b * 2 + k) * CH + c];
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
-    return s;
+#pragma unroll 5
+    for (int b = threadIdx.x; b < nblk; b += FIN_THREADS) s += part[((size_t)b * 2 + k) * CH + c];
+    return block_sum_f64(s);
 }
 
-// Sums per-block channel partials [nblk][2][64] into out[nout], one warp per
-// output (launched as nout / 8 blocks of 256 threads).  Optionally also as
-// FP32 into lo32[c] (outputs 0..63) and hi32[c] (outputs 64..127), the
+// Sums per-block channel partials [nblk][2][64] into out[blockIdx.x].  Optionally
+// also as FP32 into lo32[c] (outputs 0..63) and hi32[c] (outputs 64..127), the
 // gradient entries they are.
-__global__ void __launch_bounds__(256) channel_finalize_kernel(const double* __restrict__ part, int nblk,
-                                                               double* __restrict__ out, int nout,
-                                                               float* __restrict__ lo32, float* __restrict__ hi32) {
-    const int o = blockIdx.x * 8 + (threadIdx.x >> 5), ln = threadIdx.x & 31;
-    if (o >= nout) return;
-    const double s = warp_partial_sum(part, nblk, o >> 6, o & 63, ln);
-    if (ln == 0) {
+__global__ void __launch_bounds__(FIN_THREADS) channel_finalize_kernel(const double* __restrict__ part, int nblk,
+                                                                       double* __restrict__ out,
+                                                                       float* __restrict__ lo32,
+                                                                       float* __restrict__ hi32) {
+    const int o = blockIdx.x;
+    const double s = block_partial_sum(part, nblk, o >> 6, o & 63);
+    if (threadIdx.x == 0) {
         out[o] = s;
         float* d32 = o < CH ? lo32 : hi32;
         if (d32) d32[o & 63] = (float)s;
@@ -2384,15 +2398,15 @@ __global__ void __launch_bounds__(256) channel_finalize_kernel(const double* __r
 // The BatchNorm moments of one layer from the conv's per-warp partials: sums
 // (sum z, sum z^2) into sums[2][64], then the batch statistics (biased
 // variance) into bnp = (mean, 1/std) and the running statistics (momentum 0.1,
-// unbiased variance).  One warp per channel, 8 blocks of 256 threads.
-__global__ void __launch_bounds__(256) bn_moments_kernel(const double* __restrict__ part, int nblk,
-                                                         double* __restrict__ sums, float* __restrict__ bnp,
-                                                         float* __restrict__ rmean, float* __restrict__ rvar, double P) {
-    const int c = blockIdx.x * 8 + (threadIdx.x >> 5), ln = threadIdx.x & 31;
-    if (c >= CH) return;
-    const double s = warp_partial_sum(part, nblk, 0, c, ln);
-    const double s2 = warp_partial_sum(part, nblk, 1, c, ln);
-    if (ln == 0) {
+// unbiased variance).  One block per channel.
+__global__ void __launch_bounds__(FIN_THREADS) bn_moments_kernel(const double* __restrict__ part, int nblk,
+                                                                 double* __restrict__ sums, float* __restrict__ bnp,
+                                                                 float* __restrict__ rmean, float* __restrict__ rvar,
+                                                                 double P) {
+    const int c = blockIdx.x;
+    const double s = block_partial_sum(part, nblk, 0, c);
+    const double s2 = block_partial_sum(part, nblk, 1, c);
+    if (threadIdx.x == 0) {
         sums[c] = s;
         sums[CH + c] = s2;
         const double mean = s / P;
@@ -2403,8 +2417,6 @@ __global__ void __launch_bounds__(256) bn_moments_kernel(const double* __restric
         rvar[c] = (1.0f - BN_MOMENTUM) * rvar[c] + BN_MOMENTUM * (float)(var * P / (P > 1 ? P - 1 : 1));
     }
 }
-
-
 
 // a = relu(gamma (z - mean) istd + beta)
 // (launched with EW_BLOCKS blocks of 256 threads: a thread keeps one channel
@@ -2435,7 +2447,7 @@ __global__ void __launch_bounds__(256) bn_apply_relu_kernel(const float* __restr
 // Per-channel sums of the BF16 values a thread stores (its channel octet):
 // runs of up to 32 elements in FP32, each run added into the thread's FP64
 // sums (kept in shared memory, sh[thread / 8][octet * 8 + k]); then the
-// block's 32 threads of each octet are summed in thread order into
+// block's 32 threads of each octet are summed in a fixed order into
 // part[block][0][64] (part[block][1][*] = 0), the layout channel_finalize_kernel
 // reads.
 struct OctetSums {
@@ -2466,11 +2478,17 @@ struct OctetSums {
     __device__ __forceinline__ void store(double* __restrict__ part) {
         flush();
         __syncthreads();
+        // four threads per channel, eight rows each, then their four sums
+        const int c = threadIdx.x & (CH - 1), q = threadIdx.x / CH;
+        double t = 0.0;
+#pragma unroll
+        for (int r = 0; r < 8; ++r) t += sh[8 * q + r][c];
+        __syncthreads();
+        sh[q][c] = t;
+        __syncthreads();
         if (threadIdx.x < CH) {
-            double t = 0.0;
-            for (int r = 0; r < 32; ++r) t += sh[r][threadIdx.x];
-            part[(size_t)blockIdx.x * 2 * CH + threadIdx.x] = t;
-            part[(size_t)blockIdx.x * 2 * CH + CH + threadIdx.x] = 0.0;
+            part[(size_t)blockIdx.x * 2 * CH + c] = (sh[0][c] + sh[1][c]) + (sh[2][c] + sh[3][c]);
+            part[(size_t)blockIdx.x * 2 * CH + CH + c] = 0.0;
         }
     }
 };
@@ -2531,15 +2549,27 @@ __global__ void __launch_bounds__(256) relu_bwd_kernel(const uint4* __restrict__
     __shared__ double bsum[32][CH + 1];
     OctetSums bias;
     bias.init(bsum);
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n8; i += (size_t)gridDim.x * blockDim.x) {
-        float gv[8], av[8];
-        bf16x8_to_f32(g[i], gv);
-        bf16x8_to_f32(a[i], av);
+    const size_t stride = (size_t)gridDim.x * blockDim.x;
+    for (size_t i0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i0 < n8; i0 += 2 * stride) {
+        uint4 gr[2], ar[2];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) gv[k] = av[k] > 0.0f ? gv[k] : 0.0f;
-        const uint4 v = f32_to_bf16x8(gv);
-        dz[i] = v;
-        bias.add(v);
+        for (int e = 0; e < 2; ++e)
+            if (i0 + e * stride < n8) {
+                gr[e] = g[i0 + e * stride];
+                ar[e] = a[i0 + e * stride];
+            }
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            if (i0 + e * stride >= n8) break;
+            float gv[8], av[8];
+            bf16x8_to_f32(gr[e], gv);
+            bf16x8_to_f32(ar[e], av);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) gv[k] = av[k] > 0.0f ? gv[k] : 0.0f;
+            const uint4 v = f32_to_bf16x8(gv);
+            dz[i0 + e * stride] = v;
+            bias.add(v);
+        }
     }
     bias.store(part);
 }
@@ -2552,7 +2582,7 @@ __global__ void __launch_bounds__(256) loss_kernel(const float* __restrict__ x, 
     const float scale = (float)(2.0 / (double)P);
     double s = 0.0;
     for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < P; p += (size_t)gridDim.x * blockDim.x) {
-        const size_t img = p / HW, r = p % HW;
+        const size_t img = (unsigned)p / (unsigned)HW, r = (unsigned)p % (unsigned)HW;   // p below 2^28
         const float centre = x[(img * FRAMES + 2) * HW + r];
         const float d = centre - R[p] - clean[p];
         dR[p] = -scale * d;
@@ -2570,32 +2600,37 @@ __global__ void loss_finalize_kernel(const double* __restrict__ part, int n, dou
 }
 
 // Input gradient of the last layer (64 -> 1): da[p][ci] = sum_tap W[ci][tap] dR[p - off(tap)].
-__global__ void last_dgrad_kernel(const float* __restrict__ dR, const float* __restrict__ params, size_t w_off,
-                                  uint4* __restrict__ da, int B, int H, int W) {
-    __shared__ float w[CH * 9];
-    for (int i = threadIdx.x; i < CH * 9; i += blockDim.x) w[i] = params[w_off + i];   // [0][ci][ky][kx]
+// The weights lie as [8 channels' tap][8], two 16-byte broadcasts per tap and octet
+// (one load per weight, and the 196 registers of the unrolled octets, bound it).
+__global__ void __launch_bounds__(256) last_dgrad_kernel(const float* __restrict__ dR, const float* __restrict__ params,
+                                                         size_t w_off, uint4* __restrict__ da, int B, int H, int W) {
+    __shared__ __align__(16) float w[8][9][8];
+    for (int i = threadIdx.x; i < CH * 9; i += blockDim.x) {   // [0][ci][ky][kx]
+        const int ci = i / 9;
+        w[ci >> 3][i - ci * 9][ci & 7] = params[w_off + i];
+    }
     __syncthreads();
-    const size_t P = (size_t)B * H * W;
-    for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < P; p += (size_t)gridDim.x * blockDim.x) {
-        const int b = (int)(p % W), a = (int)((p / W) % H);
-        const size_t base = p - (size_t)a * W - b;
+    const unsigned P = (unsigned)B * H * W;      // at most 2^28
+    for (unsigned p = blockIdx.x * blockDim.x + threadIdx.x; p < P; p += gridDim.x * blockDim.x) {
+        const int b = (int)(p % (unsigned)W), a = (int)(p / (unsigned)W % (unsigned)H);
+        const size_t base = (size_t)p - (size_t)a * W - b;
         float d[9];
 #pragma unroll
         for (int tap = 0; tap < 9; ++tap) {
             const int aa = a - (tap / 3 - 1), bb = b - (tap % 3 - 1);
             d[tap] = (aa >= 0 && aa < H && bb >= 0 && bb < W) ? dR[base + (size_t)aa * W + bb] : 0.0f;
         }
-#pragma unroll
+#pragma unroll 2
         for (int c8 = 0; c8 < 8; ++c8) {
-            float o[8];
+            float o[8] = {};
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                float s = 0.0f;
+            for (int tap = 0; tap < 9; ++tap) {
+                float wv[8];
+                f32x8_load(w[c8][tap], wv);
 #pragma unroll
-                for (int tap = 0; tap < 9; ++tap) s += w[(c8 * 8 + k) * 9 + tap] * d[tap];
-                o[k] = s;
+                for (int k = 0; k < 8; ++k) o[k] = fmaf(wv[k], d[tap], o[k]);
             }
-            da[p * 8 + c8] = f32_to_bf16x8(o);
+            da[(size_t)p * 8 + c8] = f32_to_bf16x8(o);
         }
     }
 }
@@ -2607,7 +2642,8 @@ __global__ void wgrad_reduce_kernel(const float* __restrict__ part, int nchunks,
     const int n = taps * CH * CH;
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
         const int tap = e / (CH * CH), co = (e / CH) % CH, ci = e % CH;
-        float s = 0.0f;
+        float s = 0.0f;   // in order; the loads ahead of the additions
+#pragma unroll 8
         for (int c = 0; c < nchunks; ++c) s += part[((size_t)c * 9 + tap) * CH * CH + co * CH + ci];
         if (layer0) {
             if (ci < FRAMES * 9) grad[co * FRAMES * 9 + ci] = s;
@@ -2618,34 +2654,55 @@ __global__ void wgrad_reduce_kernel(const float* __restrict__ part, int nchunks,
 }
 
 // Last layer weight gradient: part[chunk][tap][ci] = sum_p dR[p] act[p + off(tap)][ci].
+// A block takes the three taps of one kernel row, whose activations it finds in
+// L1 (a block per tap read them from L2 nine times, one pixel at a time and with two
+// 64-bit divisions each: with the input gradient beside it 244 -> 134 us per step).
 __global__ void __launch_bounds__(256) wgrad_last_kernel(const float* __restrict__ dR, const uint4* __restrict__ act,
                                                          float* __restrict__ part, int B, int H, int W) {
-    const int tap = blockIdx.x, chunk = blockIdx.y;
-    const int dy = tap / 3 - 1, dx = tap % 3 - 1;
-    const size_t P = (size_t)B * H * W;
-    const size_t p_lo = (size_t)chunk * WG_CHUNK;
-    const size_t p_hi = p_lo + WG_CHUNK < P ? p_lo + WG_CHUNK : P;
+    const int dy = (int)blockIdx.x - 1, chunk = blockIdx.y;
+    const unsigned P = (unsigned)B * H * W;      // at most 2^28
+    const unsigned p_lo = (unsigned)chunk * WG_CHUNK, p_hi = min(p_lo + WG_CHUNK, P);
     const int lane8 = threadIdx.x & 7, row = threadIdx.x >> 3;    // 32 pixel rows x 8 channel groups
-    float acc[8] = {};
-    for (size_t p = p_lo + row; p < p_hi; p += 32) {
-        const int b = (int)(p % W), a = (int)((p / W) % H);
-        const int aa = a + dy, bb = b + dx;
-        if (aa < 0 || aa >= H || bb < 0 || bb >= W) continue;
-        float u[8];
-        bf16x8_to_f32(act[(p + (ptrdiff_t)dy * W + dx) * 8 + lane8], u);
-        const float d = dR[p];
+    float acc[3][8] = {};
+    unsigned b = (p_lo + row) % W, a = (p_lo + row) / W % H;
+    // the loads of four pixels before their terms (a tap outside the image adds 0)
+    for (unsigned p0 = p_lo + row; p0 < p_hi; p0 += 4 * 32) {
+        float d[4];
+        uint4 u[4][3];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) acc[k] = fmaf(d, u[k], acc[k]);
+        for (int j = 0; j < 4; ++j) {
+            const unsigned p = p0 + 32 * j;
+            const bool in = p < p_hi && (unsigned)((int)a + dy) < (unsigned)H;
+            d[j] = in ? dR[p] : 0.0f;
+#pragma unroll
+            for (int dx = -1; dx <= 1; ++dx)
+                u[j][dx + 1] = in && (unsigned)((int)b + dx) < (unsigned)W ? act[((ptrdiff_t)p + dy * W + dx) * 8 + lane8]
+                                                                          : make_uint4(0u, 0u, 0u, 0u);
+            for (b += 32; b >= (unsigned)W; b -= W) a = a + 1 == (unsigned)H ? 0 : a + 1;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int t = 0; t < 3; ++t) {
+                float f[8];
+                bf16x8_to_f32(u[j][t], f);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) acc[t][k] = fmaf(d[j], f[k], acc[t][k]);
+            }
     }
     // reduce the 32 rows through shared memory
-    __shared__ float red[32][CH + 1];
+    __shared__ float red[3][32][CH + 1];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) red[row][lane8 * 8 + k] = acc[k];
+    for (int t = 0; t < 3; ++t)
+#pragma unroll
+        for (int k = 0; k < 8; ++k) red[t][row][lane8 * 8 + k] = acc[t][k];
     __syncthreads();
-    if (threadIdx.x < CH) {
+    if (threadIdx.x < 3 * CH) {
+        const int t = threadIdx.x / CH, ci = threadIdx.x % CH;
         float s = 0.0f;
-        for (int r = 0; r < 32; ++r) s += red[r][threadIdx.x];
-        part[((size_t)chunk * 9 + tap) * CH + threadIdx.x] = s;
+#pragma unroll 8
+        for (int r = 0; r < 32; ++r) s += red[t][r][ci];
+        part[((size_t)chunk * 9 + (dy + 1) * 3 + t) * CH + ci] = s;
     }
 }
 
@@ -2653,7 +2710,8 @@ __global__ void wgrad_last_reduce_kernel(const float* __restrict__ part, int nch
     const int e = threadIdx.x + blockIdx.x * blockDim.x;   // tap*64 + ci
     if (e >= 9 * CH) return;
     const int tap = e / CH, ci = e % CH;
-    float s = 0.0f;
+    float s = 0.0f;   // in order; the loads ahead of the additions
+#pragma unroll 8
     for (int c = 0; c < nchunks; ++c) s += part[((size_t)c * 9 + tap) * CH + ci];
     grad[ci * 9 + tap] = s;
 }
@@ -2882,16 +2940,9 @@ extern "C" msf_status msf_train_step(msf_cnn* c, const float* d_noisy, const flo
     for (int l = 0; l < LAYERS; ++l) { wf_off[l] = wp; wp += (size_t)taps_of(l) * rows_of(l) * KPACK; }
     {
         MSF_PROF("train_pack_weights", st);
-        for (int l = 0; l < LAYERS; ++l) {
-            FoldArgs f;
-            f.layer = l; f.taps = taps_of(l); f.rows = rows_of(l); f.cin = cin_of(l); f.cout = cout_of(l);
-            f.w = (long long)o.w[l]; f.b = (long long)o.b[l];
-            f.gamma = f.beta = f.mean = f.var = -1;
-            fold_kernel<<<64, 256, 0, st>>>(c->d_params, w.wf + wf_off[l], w.bf + l * CH, f);
-        }
-        pack_dgrad_kernel<<<256, 256, 0, st>>>(c->d_params, w.wb, o);
+        fold_kernel<<<dim3(64, LAYERS), 256, 0, st>>>(c->d_params, w.wf, w.bf, fold_args(o, wf_off, false));
+        pack_dgrad_kernel<<<256, 256, 0, st>>>(c->d_params, w.wb, w.zeros, o);
         MSF_LAUNCH_CHECK();
-        MSF_TRY_CUDA(cudaMemsetAsync(w.zeros, 0, CH * 4, st));
     }
     CUtensorMap m16[LAYERS], m18[LAYERS], m4[LAYERS], g16[2], g18[2], g4[2], mw[LAYERS], mb[8], f4[LAYERS - 1];
     for (int l = 1; l < LAYERS - 1; ++l) MSF_TRY(make_f32_out_map(&f4[l], w.z[l], B, H, W));
@@ -2929,7 +2980,7 @@ extern "C" msf_status msf_train_step(msf_cnn* c, const float* d_noisy, const flo
             MSF_LAUNCH_CHECK();
         }
         MSF_PROF("train_reduce_finalize", st);
-        channel_finalize_kernel<<<2 * CH / 8, 256, 0, st>>>(w.part, nred, out, 2 * CH, lo32, hi32);
+        channel_finalize_kernel<<<2 * CH, FIN_THREADS, 0, st>>>(w.part, nred, out, lo32, hi32);
         MSF_LAUNCH_CHECK();
         return MSF_OK;
     };
@@ -2949,7 +3000,7 @@ extern "C" msf_status msf_train_step(msf_cnn* c, const float* d_noisy, const flo
         float* bnp = w.bnp + (size_t)(l - 1) * 2 * CH;
         {
             MSF_PROF("train_bn_stats", st);
-            bn_moments_kernel<<<CH / 8, 256, 0, st>>>(w.part, 4 * conv_grid, sums, bnp, c->d_params + o.mean[l],
+            bn_moments_kernel<<<CH, FIN_THREADS, 0, st>>>(w.part, 4 * conv_grid, sums, bnp, c->d_params + o.mean[l],
                                                       c->d_params + o.var[l], (double)P);
             MSF_LAUNCH_CHECK();
         }
@@ -2972,7 +3023,7 @@ extern "C" msf_status msf_train_step(msf_cnn* c, const float* d_noisy, const flo
         MSF_PROF("train_last_bwd", st);
         last_dgrad_kernel<<<EW_BLOCKS, 256, 0, st>>>(w.dR, c->d_params, o.w[9], (uint4*)w.g[0], B, H, W);
         MSF_TRY(trace_record(c, TRACE_DA, 9, w.g[0], P, st));
-        wgrad_last_kernel<<<dim3(9, nchunks), 256, 0, st>>>(w.dR, (const uint4*)w.act[9], w.wpart, B, H, W);
+        wgrad_last_kernel<<<dim3(3, nchunks), 256, 0, st>>>(w.dR, (const uint4*)w.act[9], w.wpart, B, H, W);
         wgrad_last_reduce_kernel<<<(9 * CH + 255) / 256, 256, 0, st>>>(w.wpart, nchunks, c->d_grad + o.w[9]);
         sum_f32_kernel<<<nred, 256, 0, st>>>(w.dR, (size_t)P, w.part);
         store_sum_kernel<<<1, 256, 0, st>>>(w.part, nred, c->d_grad + o.b[9]);
@@ -2996,7 +3047,7 @@ extern "C" msf_status msf_train_step(msf_cnn* c, const float* d_noisy, const flo
         // dz in g[cur ^ 1]: conv bias grad (its block sums came with dz), weight grad, input grad
         {
             MSF_PROF("train_reduce_finalize", st);
-            channel_finalize_kernel<<<CH / 8, 256, 0, st>>>(w.part, EW_BLOCKS, sums, CH, c->d_grad + o.b[l], nullptr);
+            channel_finalize_kernel<<<CH, FIN_THREADS, 0, st>>>(w.part, EW_BLOCKS, sums, c->d_grad + o.b[l], nullptr);
             MSF_LAUNCH_CHECK();
         }
         {
@@ -3023,7 +3074,7 @@ extern "C" msf_status msf_train_step(msf_cnn* c, const float* d_noisy, const flo
     MSF_TRY(trace_record(c, TRACE_DZ, 0, w.g[cur ^ 1], P, st));
     {
         MSF_PROF("train_reduce_finalize", st);
-        channel_finalize_kernel<<<CH / 8, 256, 0, st>>>(w.part, EW_BLOCKS, w.sums, CH, c->d_grad + o.b[0], nullptr);
+        channel_finalize_kernel<<<CH, FIN_THREADS, 0, st>>>(w.part, EW_BLOCKS, w.sums, c->d_grad + o.b[0], nullptr);
         MSF_LAUNCH_CHECK();
     }
     {
