@@ -20,8 +20,8 @@ struct msf_mace {
     msf_mace_desc desc;
     msf_dataprox* dp = nullptr;
     double* d_partial = nullptr;   // [2][nblocks]
-    double* d_sums = nullptr;      // [2]
-    double* h_sums = nullptr;      // pinned [2], written by the step's last copy
+    unsigned* d_count = nullptr;   // consensus blocks that have stored their partials
+    double* h_sums = nullptr;      // pinned [2], written by the step's last kernel
     int* h_status = nullptr;       // pinned copy of the data agent's numeric status word
     float* d_meas = nullptr;       // msf_mace_set_counts: counts, y, Lambda (3 sinograms)
     int nblocks = 0;
@@ -68,9 +68,20 @@ struct MaceCoef {
 // VEC = false); the per-voxel
 // terms are FP32 and each step's sum of four is added to FP64 thread sums,
 // so this HBM-bound pass does a few FP64 adds per four voxels.
+// A MACE step's last block also sums the partials (in a fixed order) and stores the
+// two sums and the data agent's status word in the handle's pinned host memory:
+// the step ends with this launch, without one for the sums and two copies.
+struct MaceResidual {
+    unsigned* count;      // zero between steps; NULL: the caller sums the partials
+    double* h_sums;       // pinned [2]
+    int* h_status;        // pinned
+    const int* status;
+};
+
 template <int K1, bool VEC>
 __global__ void __launch_bounds__(256) consensus_kernel(float* __restrict__ W, const float* __restrict__ X,
-                                                         size_t N, MaceCoef c, double* __restrict__ partial) {
+                                                         size_t N, MaceCoef c, double* __restrict__ partial,
+                                                         MaceResidual res) {
     double num = 0.0, den = 0.0;
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     auto voxel = [&](const float (&x)[K1], float (&w)[K1], float& dev, float& xb2) {
@@ -137,9 +148,31 @@ __global__ void __launch_bounds__(256) consensus_kernel(float* __restrict__ W, c
     }
     const double sn = block_sum_f64(num);
     const double sd = block_sum_f64(den);
+    __shared__ bool last;
     if (threadIdx.x == 0) {
         partial[blockIdx.x] = sn;
         partial[gridDim.x + blockIdx.x] = sd;
+        last = false;
+        if (res.count) {
+            __threadfence();
+            last = atomicAdd(res.count, 1u) == gridDim.x - 1;
+        }
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    double a = 0.0, b = 0.0;
+    for (int i = threadIdx.x; i < gridDim.x; i += blockDim.x) {
+        a += __ldcg(partial + i);
+        b += __ldcg(partial + gridDim.x + i);
+    }
+    a = block_sum_f64(a);
+    b = block_sum_f64(b);
+    if (threadIdx.x == 0) {
+        res.h_sums[0] = a;
+        res.h_sums[1] = b;
+        *res.h_status = *res.status;
+        *res.count = 0;
     }
 }
 
@@ -161,28 +194,27 @@ constexpr int CONSENSUS_BLOCKS = 152 * 8;
 static_assert(MSF_CONSENSUS_SUMS == 2 * CONSENSUS_BLOCKS && MSF_CONSENSUS_WORK == MSF_CONSENSUS_SUMS + 2,
               "msf_mace_consensus workspace layout");
 
-// The consensus pass over K1 stacked states of N voxels each, then the two
-// FP64 sums (into sums[0..1]) of the per-block partials.
+// Blocks of the consensus pass: four voxels per thread and step.
+static int consensus_blocks(size_t N) {
+    const size_t need = (N + 1023) / 1024;
+    return need < (size_t)CONSENSUS_BLOCKS ? (int)need : CONSENSUS_BLOCKS;
+}
+
+// The consensus pass over K1 stacked states of N voxels each.
 static msf_status launch_consensus(float* W, const float* X, int K1, size_t N, const MaceCoef& c, double* partial,
-                                   double* sums, cudaStream_t st) {
-    {
-        MSF_PROF("mace_consensus", st);
-        const bool vec = N % 4 == 0 && (uintptr_t)W % 16 == 0 && (uintptr_t)X % 16 == 0;
-        if (K1 == 2 && vec)
-            consensus_kernel<2, true><<<CONSENSUS_BLOCKS, 256, 0, st>>>(W, X, N, c, partial);
-        else if (K1 == 2)
-            consensus_kernel<2, false><<<CONSENSUS_BLOCKS, 256, 0, st>>>(W, X, N, c, partial);
-        else if (vec)
-            consensus_kernel<4, true><<<CONSENSUS_BLOCKS, 256, 0, st>>>(W, X, N, c, partial);
-        else
-            consensus_kernel<4, false><<<CONSENSUS_BLOCKS, 256, 0, st>>>(W, X, N, c, partial);
-        MSF_LAUNCH_CHECK();
-    }
-    {
-        MSF_PROF("mace_residual", st);
-        sum2_kernel<<<1, 1024, 0, st>>>(partial, CONSENSUS_BLOCKS, sums);
-        MSF_LAUNCH_CHECK();
-    }
+                                   const MaceResidual& res, cudaStream_t st) {
+    MSF_PROF("mace_consensus", st);
+    const bool vec = N % 4 == 0 && (uintptr_t)W % 16 == 0 && (uintptr_t)X % 16 == 0;
+    const int blocks = consensus_blocks(N);
+    if (K1 == 2 && vec)
+        consensus_kernel<2, true><<<blocks, 256, 0, st>>>(W, X, N, c, partial, res);
+    else if (K1 == 2)
+        consensus_kernel<2, false><<<blocks, 256, 0, st>>>(W, X, N, c, partial, res);
+    else if (vec)
+        consensus_kernel<4, true><<<blocks, 256, 0, st>>>(W, X, N, c, partial, res);
+    else
+        consensus_kernel<4, false><<<blocks, 256, 0, st>>>(W, X, N, c, partial, res);
+    MSF_LAUNCH_CHECK();
     return MSF_OK;
 }
 
@@ -214,14 +246,12 @@ static msf_status enqueue_consensus(msf_mace* m, const msf_mace_params* prm, cud
     for (int i = 0; i < 4; ++i) c.mu[i] = i < K1 ? (float)prm->mu[i] : 0.0f;
     c.two_rho = (float)(2.0 * prm->rho);
     c.K1 = K1;
-    MSF_TRY(launch_consensus(d.d_W, d.d_X, K1, m->N, c, m->d_partial, m->d_sums, st));
-    MSF_TRY_CUDA(cudaMemcpyAsync(m->h_sums, m->d_sums, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
-    MSF_TRY_CUDA(cudaMemcpyAsync(m->h_status, dataprox_status(m->dp), sizeof(int), cudaMemcpyDeviceToHost, st));
-    return MSF_OK;
+    const MaceResidual res{m->d_count, m->h_sums, m->h_status, dataprox_status(m->dp)};
+    return launch_consensus(d.d_W, d.d_X, K1, m->N, c, m->d_partial, res, st);
 }
 
-// Enqueues one whole iteration on st, ending with the copy of the two FP64
-// residual sums into the handle's pinned buffer.
+// Enqueues one whole iteration on st, ending with the two FP64 residual sums in
+// the handle's pinned buffer.
 static msf_status enqueue_step(msf_mace* m, const msf_mace_params* prm, cudaStream_t st) {
     const msf_mace_desc& d = m->desc;
     const size_t N = m->N;
@@ -421,7 +451,8 @@ extern "C" msf_status msf_mace_create(const msf_mace_desc* desc, msf_mace** out)
     m->N = (size_t)v->nx * v->ny * v->nz * v->nt;
     m->nblocks = CONSENSUS_BLOCKS;
     if (cudaMalloc(&m->d_partial, 2 * m->nblocks * sizeof(double)) != cudaSuccess ||
-        cudaMalloc(&m->d_sums, 2 * sizeof(double)) != cudaSuccess ||
+        cudaMalloc(&m->d_count, sizeof(unsigned)) != cudaSuccess ||
+        cudaMemset(m->d_count, 0, sizeof(unsigned)) != cudaSuccess ||
         cudaMallocHost(&m->h_sums, 2 * sizeof(double)) != cudaSuccess ||
         cudaMallocHost(&m->h_status, sizeof(int)) != cudaSuccess ||
         cudaStreamCreateWithFlags(&m->cap, cudaStreamNonBlocking) != cudaSuccess ||
@@ -445,7 +476,7 @@ extern "C" void msf_mace_destroy(msf_mace* m) {
     if (m->ev_prior) cudaEventDestroy(m->ev_prior);
     msf_dataprox_destroy(m->dp);
     cudaFree(m->d_partial);
-    cudaFree(m->d_sums);
+    cudaFree(m->d_count);
     if (m->h_sums) cudaFreeHost(m->h_sums);
     if (m->h_status) cudaFreeHost(m->h_status);
     cudaFree(m->d_meas);
@@ -597,5 +628,10 @@ extern "C" msf_status msf_mace_consensus(float* d_W, const float* d_X, int K1, s
     for (int i = 0; i < 4; ++i) c.mu[i] = i < K1 ? (float)mu[i] : 0.0f;
     c.two_rho = (float)(2.0 * rho);
     c.K1 = K1;
-    return launch_consensus(d_W, d_X, K1, N, c, d_work, d_work + 2 * CONSENSUS_BLOCKS, as_stream(stream));
+    cudaStream_t st = as_stream(stream);
+    MSF_TRY(launch_consensus(d_W, d_X, K1, N, c, d_work, MaceResidual{}, st));
+    MSF_PROF("mace_residual", st);
+    sum2_kernel<<<1, 1024, 0, st>>>(d_work, consensus_blocks(N), d_work + 2 * CONSENSUS_BLOCKS);
+    MSF_LAUNCH_CHECK();
+    return MSF_OK;
 }

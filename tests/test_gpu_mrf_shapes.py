@@ -29,7 +29,9 @@ def _sweeps(M, v, z, sigma, q, sx, bt, n):
     return zg.cpu().numpy().astype(np.float64), oracle.prox_qggmrf(v, z, sigma, 2.0, q, 1.0, sx, bt, n)
 
 
-@pytest.mark.parametrize("shape", [(1, 1, 1, 1), (1, 2, 1, 2), (3, 3, 3, 3), (2, 5, 9, 67), (4, 3, 2, 64), (3, 7, 4, 65), (1, 4, 33, 130)],
+@pytest.mark.parametrize("shape", [(1, 1, 1, 1), (1, 2, 1, 2), (3, 3, 3, 3), (2, 5, 9, 67), (4, 3, 2, 64), (3, 7, 4, 65), (1, 4, 33, 130),
+                                   # the largest volume of one launch (4096 voxels per colour), and the next that takes sixteen
+                                   (2, 32, 32, 32), (2, 32, 32, 33), (3, 21, 34, 70)],
                          ids=lambda s: "x".join(map(str, s)))
 @pytest.mark.parametrize("q", [1.0, 1.2, 2.0])
 def test_sweeps_match_oracle_at_ragged_sizes(M, shape, q):
