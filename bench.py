@@ -227,9 +227,11 @@ def algorithmic(scan, K1):
         "joseph_fwd": ("hbm", 4.0 * (N + 2 * M)),
         # adjoint: sinogram in, volume out (+ p in for the CG operator)
         "joseph_adj": ("hbm", 4.0 * (M + 2 * N)),
-        "transpose": ("hbm", 8.0 * N),
-        "transpose_pupdate": ("hbm", 16.0 * N),
-        "cg_update": ("hbm", 4.0 * 6 * N),
+        # volume order <-> lines along z (two volumes each way)
+        "transpose": ("hbm", 16.0 * N),
+        "volume": ("hbm", 12.0 * N),
+        "cg_residual": ("hbm", 12.0 * N),
+        "cg_direction": ("hbm", 20.0 * N),
         # one colour of the ICD sweep: its voxels read/written, all neighbours read
         "qggmrf_icd": ("hbm", 4.0 * (N + 3 * N / 16)),
         "mace_consensus": ("hbm", 4.0 * 3 * K1 * N),
@@ -600,16 +602,17 @@ def quality_run(step, X0, x_true, iters, points=QUALITY_POINTS):
 
 SMS, FP32_LANES, L1_BYTES_PER_CLK = 152, 128, 128   # per SM: FP32 lanes, L1 / shared-memory bytes per clock
 
-# Per in-grid ray-plane crossing (counted from the kernels' inner loops):
-#   forward: two 8-byte loads of the z-paired copies (16 B through the L1 data
-#     pipe) and 11.5 FP32-pipe instructions (per ray: the z crossing (FMA),
-#     its floor and fraction, three lerps of a subtraction and an FMA, the
-#     accumulation; the a crossing's FMA, floor and fraction shared by 2 rays);
-#   adjoint: each crossing is gathered by the two voxel runs holding its a taps;
-#     per visit a 4-byte sinogram load and two shared-memory read-modify-writes
-#     of the accumulators (20 B), and 12 FP32-pipe instructions.
+# Per in-grid ray-plane crossing, whatever kernel forms it:
+#   forward: its four bilinear taps read (16 B through the L1 data pipe) and 11.5
+#     FP32 operations (the z crossing, its floor and fraction, three lerps of a
+#     subtraction and an FMA, the accumulation; the a crossing shared by two rays);
+#   adjoint: the same crossing and weights, the ray's value (4 B) and four
+#     multiply-adds into the taps (a read and a write of 4 B each).
+# The kernels share parts of this between rays (packed pairs of rows, sums kept in
+# registers and used by both lines beside a crossing), so a fraction of the larger
+# floor says how far they are from that plain count, not from a hard limit.
 PROJ_MODEL = {"joseph_fwd": {"bytes": 16.0, "instr": 11.5},
-              "joseph_adj": {"bytes": 40.0, "instr": 24.0}}
+              "joseph_adj": {"bytes": 36.0, "instr": 15.5}}
 
 
 def in_grid_crossings(scan) -> int:
