@@ -1791,6 +1791,11 @@ extern "C" msf_status msf_cnn_create(int64_t max_pixels, msf_cnn** out) {
         cudaMemcpy(c->d_frozen, frozen.data(), P, cudaMemcpyHostToDevice);
         cudaMemset(c->d_grad, 0, P * 4);
     }
+    const msf_status st = settle_default_stream();
+    if (st != MSF_OK) {
+        msf_cnn_destroy(c);
+        return st;
+    }
     *out = c;
     return MSF_OK;
 }

@@ -33,6 +33,11 @@ msf_status check_device() {
     return MSF_OK;
 }
 
+msf_status settle_default_stream() {
+    MSF_TRY_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
+    return MSF_OK;
+}
+
 // y = -ln(max(n,1)/I0) and Lambda = c exp(-y): Sec. II, the weight matrix
 // Lambda_n = diag{c exp(-y_n)} of the Gaussian approximation to Poisson noise.
 __global__ void weights_kernel(const float* __restrict__ counts, float* __restrict__ y,

@@ -35,6 +35,13 @@ int* dataprox_status(msf_dataprox* d);
 uint64_t cnn_generation(const msf_cnn* c);
 msf_status cnn_prepare(msf_cnn* c, cudaStream_t st);
 
+// Waits for the clears and copies that the calling function has issued on the
+// default stream.  cudaMemset returns before the device has done it, and a
+// non-blocking stream is not ordered after the default stream: a handle whose
+// create call did not wait could have its workspace cleared under the first call
+// on such a stream.
+msf_status settle_default_stream();
+
 }  // namespace msf
 
 #define MSF_TRY_CUDA(call)                                                                  \

@@ -461,6 +461,11 @@ extern "C" msf_status msf_mace_create(const msf_mace_desc* desc, msf_mace** out)
         msf_mace_destroy(m);
         return fail(MSF_ERR_NOMEM, "msf_mace_create: out of memory");
     }
+    st = settle_default_stream();
+    if (st != MSF_OK) {
+        msf_mace_destroy(m);
+        return st;
+    }
     *out = m;
     return MSF_OK;
 }

@@ -397,6 +397,11 @@ extern "C" msf_status msf_map_create(msf_projector* p, msf_map** out) {
         msf_map_destroy(m);
         return fail(MSF_ERR_NOMEM, "msf_map_create: out of device memory");
     }
+    const msf_status st = settle_default_stream();
+    if (st != MSF_OK) {
+        msf_map_destroy(m);
+        return st;
+    }
     *out = m;
     return MSF_OK;
 }

@@ -1590,6 +1590,11 @@ extern "C" msf_status msf_dataprox_create(msf_projector* p, msf_dataprox** out) 
         msf_dataprox_destroy(d);
         return fail(MSF_ERR_CUDA, "msf_dataprox_create: memset failed");
     }
+    const msf_status settled = settle_default_stream();
+    if (settled != MSF_OK) {
+        msf_dataprox_destroy(d);
+        return settled;
+    }
     *out = d;
     return MSF_OK;
 }
