@@ -179,7 +179,7 @@ msf_status msf_weights(const float* d_counts, float* d_y, float* d_lambda, size_
 typedef struct msf_dataprox msf_dataprox;
 
 /* Workspace for the data proximal maps (CG and ICD) on the projector's problem
- * size: three 4D volumes in lines along z, three sinograms in lines of rows and
+ * size: three 4D volumes in lines along z, two sinograms in lines of rows and
  * per-frame FP64 partial sums. */
 msf_status msf_dataprox_create(msf_projector* p, msf_dataprox** out);
 void msf_dataprox_destroy(msf_dataprox* d);

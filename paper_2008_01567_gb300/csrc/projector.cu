@@ -110,12 +110,14 @@ __global__ void column_table_kernel(const double* __restrict__ angles, float4* _
 // ------------------------------------------------------------------ z-contiguous copies
 
 // The forward reads a frame as lines of voxels along z: line (y, x) of frame t
-// starts at ((t*ny + y)*nx + x) * nzp, voxel z at element VZ_FRONT + z.  The
-// elements before and after the nz voxels are zeros that nothing writes (the
-// buffers are cleared when they are allocated), so that a tap outside the
-// volume in z reads 0 without a check.
+// starts at VZ_FRONT + ((t*ny + y)*nx + x) * nzp.  The elements between the lines
+// (two or more, shared by a line's end and the next one's start) and the VZ_FRONT
+// before the first are zeros that nothing writes (the buffers are cleared when they
+// are allocated), so that a tap outside the volume in z reads 0 without a check.
+// (With margins of each line's own a volume of one slice took 32 bytes per voxel,
+// now 16; lines start on 16 bytes either way.)
 constexpr int VZ_FRONT = 4;
-__host__ __device__ __forceinline__ int vz_pitch(int nz) { return (nz + VZ_FRONT + 2 + 7) & ~7; }
+__host__ __device__ __forceinline__ int vz_pitch(int nz) { return (nz + 2 + 3) & ~3; }
 
 // Transposes between a volume [nt][nz][ny][nx] and its lines, through 64 x 64
 // shared tiles of one (t, y) plane: 256-byte pieces on both sides, 16 loads per
@@ -202,11 +204,12 @@ enum FwdMode { FWD_PLAIN = 0, FWD_LAMBDA = 1, FWD_RESIDUAL = 2, FWD_ICD = 3 };
 constexpr int FWD_MAX_R = 5;
 
 // The step-weighted sinogram e' as the gather reads it: lines of detector rows,
-// row iv of (view g, column iu) at (g*nu + iu) * sino_pitch + SINO_FRONT + iv.
-// The margins are zeros that nothing writes: rows a voxel's window reaches
-// beyond the detector read 0.
-constexpr int SINO_FRONT = 4, SINO_BACK = 4;
-__host__ __device__ __forceinline__ int sino_pitch(int nv) { return (nv + SINO_FRONT + SINO_BACK + 7) & ~7; }
+// row iv of (view g, column iu) at SINO_FRONT + (g*nu + iu) * sino_pitch + iv.
+// The elements between the lines (SINO_FRONT or more, shared) and before the first
+// are zeros that nothing writes: rows a voxel's window reaches beyond the detector
+// read 0.
+constexpr int SINO_FRONT = 4;
+__host__ __device__ __forceinline__ int sino_pitch(int nv) { return (nv + SINO_FRONT + 3) & ~3; }
 
 // 2^23 + 2^22: adding it in round-down mode leaves floor(f) in the low mantissa
 // bits for |f| < 2^22, so the floor and its integer cost two additions instead
@@ -285,7 +288,7 @@ __device__ __forceinline__ void icd_alpha(double sum, int t, int b, int nparts, 
 //   FWD_PLAIN:    out = A x
 //   FWD_LAMBDA:   out = step * Lambda * (A x)
 //   FWD_RESIDUAL: out = step * Lambda * (meas - A x)
-//   FWD_ICD:      out = A x, and the line search's alpha (icd_alpha)
+//   FWD_ICD:      out = (step * Lambda) * (A x), and the line search's alpha (icd_alpha)
 // (the CG modes write the step-weighted sinogram e' = step * e that the gather
 // adjoint consumes; ROWS: as lines of detector rows, sino_pitch).  The sums go
 // through shared memory so that the sinogram is read and written in 16-byte
@@ -444,7 +447,10 @@ __global__ void __launch_bounds__(256, R == 5 ? 1 : 3) joseph_fwd_kernel(
         float res = val;
         if (MODE == FWD_LAMBDA) res = step * (lam[ray] * val);
         if (MODE == FWD_RESIDUAL) res = step * (lam[ray] * (meas[ray] - val));
-        if (MODE == FWD_ICD) sq += (double)lam[ray] * (double)val * (double)val;
+        if (MODE == FWD_ICD) {
+            sq += (double)lam[ray] * (double)val * (double)val;
+            res = __fmul_rn(__fmul_rn(step, lam[ray]), val);
+        }
         if (ROWS) *sum = res;
         else out[ray] = res;
     }
@@ -721,7 +727,7 @@ __device__ __forceinline__ void gather_run(const float4* __restrict__ col, const
                 // every window of the run's voxels inside the line's margins
                 const float t_lo = __fmaf_rn(d.cz - (float)z_lo, -rdfz, c0);
                 const float t_hi = __fmaf_rn(d.cz - (float)min(z_lo + STR * (32 * J - 1), d.nz - 1), -rdfz, c0);
-                if (t_lo > 1.0f - SINO_FRONT && t_hi < (float)(d.nv + SINO_BACK - 4))
+                if (t_lo > 1.0f - SINO_FRONT && t_hi < (float)d.nv)
                     fast = rdfz > 0.5f && rdfz <= 1.0f ? ADJ_TWO : rdfz > 1.0f && rdfz <= 1.5f ? ADJ_THREE : 0;
             }
             const unsigned mask = __ballot_sync(0xffffffffu, ok);
@@ -1102,11 +1108,11 @@ __global__ void __launch_bounds__(32 * ADJ_T * VS, adj_min_blocks(J) >= VS ? adj
     }
 }
 
-// After a group step: e' -= alpha_t step Lambda (A delta) over the sinogram's
+// After a group step: e' -= alpha_t ad, ad = step Lambda (A delta), over the sinogram's
 // lines of rows (the first half of a frame's blocks), z += alpha_t delta over the
 // group's lines (the second half).
-__global__ void __launch_bounds__(256) icd_update_kernel(float* __restrict__ e, const float* __restrict__ sl,
-                                                         const float* __restrict__ ad, float* __restrict__ z,
+__global__ void __launch_bounds__(256) icd_update_kernel(float* __restrict__ e, const float* __restrict__ ad,
+                                                         float* __restrict__ z,
                                                          const float* __restrict__ dlt,
                                                          const double* __restrict__ alpha, IcdGroup G, ProjDims d) {
     const int t = blockIdx.y, half = gridDim.x / 2;
@@ -1114,10 +1120,7 @@ __global__ void __launch_bounds__(256) icd_update_kernel(float* __restrict__ e, 
     if (blockIdx.x < half) {
         const size_t lines = (size_t)d.views * d.nu, off = (size_t)t * lines * sino_pitch(d.nv);
         for_units(lines, d.nv, sino_pitch(d.nv), blockIdx.x, half, [&](size_t l) { return l; }, [&](size_t i, int n) {
-            const float4 s = load4(sl + off + i), p = load4(ad + off + i), v = load4(e + off + i);
-            store4(e + off + i,
-                   make_float4(__fmaf_rn(-a, __fmul_rn(s.x, p.x), v.x), __fmaf_rn(-a, __fmul_rn(s.y, p.y), v.y),
-                               __fmaf_rn(-a, __fmul_rn(s.z, p.z), v.z), __fmaf_rn(-a, __fmul_rn(s.w, p.w), v.w)), n);
+            store4(e + off + i, fma4(-a, load4(ad + off + i), load4(e + off + i)), n);
         });
     } else {
         const size_t off = (size_t)t * d.ny * d.nx * vz_pitch(d.nz);
@@ -1127,30 +1130,25 @@ __global__ void __launch_bounds__(256) icd_update_kernel(float* __restrict__ e, 
     }
 }
 
-// sl = step Lambda and e2 = step^2 Lambda (the theta2 gather's input) as lines of
-// rows, through 32 x 32 tiles of one view.
+// e2 = step^2 Lambda (the theta2 gather's input) as lines of rows, through 32 x 32
+// tiles of one view.
 __global__ void icd_weights_kernel(const float4* __restrict__ col, const float* __restrict__ lam,
-                                   float* __restrict__ sl, float* __restrict__ e2, ProjDims d) {
-    __shared__ float tile[32][33], tile2[32][33];
+                                   float* __restrict__ e2, ProjDims d) {
+    __shared__ float tile[32][33];
     const int g = blockIdx.x, u0 = blockIdx.y * 32, v0 = blockIdx.z * 32;
     const int iu = u0 + threadIdx.x;
     if (iu < d.nu) {
         const ColParams c = load_col(col, (size_t)g * d.nu + iu);
         for (int k = threadIdx.y; k < 32 && v0 + k < d.nv; k += blockDim.y) {
             const float step = ray_z(c, det_v(v0 + k, d), d.cz).step;
-            const float l = lam[((size_t)g * d.nv + v0 + k) * d.nu + iu];
-            tile[k][threadIdx.x] = __fmul_rn(step, l);
-            tile2[k][threadIdx.x] = __fmul_rn(__fmul_rn(step, step), l);
+            tile[k][threadIdx.x] = __fmul_rn(__fmul_rn(step, step), lam[((size_t)g * d.nv + v0 + k) * d.nu + iu]);
         }
     }
     __syncthreads();
     const int iv = v0 + threadIdx.x;
     if (iv >= d.nv) return;
-    for (int k = threadIdx.y; k < 32 && u0 + k < d.nu; k += blockDim.y) {
-        const size_t i = ((size_t)g * d.nu + u0 + k) * sino_pitch(d.nv) + SINO_FRONT + iv;
-        sl[i] = tile[threadIdx.x][k];
-        e2[i] = tile2[threadIdx.x][k];
-    }
+    for (int k = threadIdx.y; k < 32 && u0 + k < d.nu; k += blockDim.y)
+        e2[((size_t)g * d.nu + u0 + k) * sino_pitch(d.nv) + SINO_FRONT + iv] = tile[threadIdx.x][k];
 }
 
 // ------------------------------------------------------------------ phantom (test data)
@@ -1255,9 +1253,9 @@ struct msf_dataprox {
     // CG: residual, direction and A^T Lambda A p + p / sigma^2, as lines (d_q
     // first holds v - z; z itself runs in the plan's d_vz)
     float *d_r = nullptr, *d_p = nullptr, *d_q = nullptr;
-    // step-weighted sinograms in lines of rows: e' ; ICD: A delta (first step^2
-    // Lambda), step Lambda.  (ICD keeps delta, theta2 and v in d_p, d_r and d_q.)
-    float *d_rows = nullptr, *d_rows2 = nullptr, *d_sl = nullptr;
+    // step-weighted sinograms in lines of rows: e' ; ICD: step Lambda (A delta) (first
+    // step^2 Lambda).  (ICD keeps delta, theta2 and v in d_p, d_r and d_q.)
+    float *d_rows = nullptr, *d_rows2 = nullptr;
     double *d_partial = nullptr, *d_rr = nullptr, *d_alpha = nullptr, *d_beta = nullptr;
     int* d_status = nullptr;
     unsigned* d_count = nullptr;
@@ -1270,10 +1268,10 @@ namespace msf {
 static size_t frame_size(const msf_vol& v) { return (size_t)v.nx * v.ny * v.nz; }
 static size_t vol_size(const msf_vol& v) { return frame_size(v) * v.nt; }
 static size_t vz_size(const msf_vol& v) {   // a volume as lines
-    return (size_t)v.nt * v.ny * v.nx * vz_pitch(v.nz);
+    return VZ_FRONT + (size_t)v.nt * v.ny * v.nx * vz_pitch(v.nz);
 }
 static size_t rows_size(const msf_projector* p) {   // a sinogram in lines of rows
-    return (size_t)p->vol.nt * p->geom.views * p->geom.nu * sino_pitch(p->geom.nv);
+    return SINO_FRONT + (size_t)p->vol.nt * p->geom.views * p->geom.nu * sino_pitch(p->geom.nv);
 }
 static size_t sino_size(const msf_projector* p) {
     return (size_t)p->geom.nu * p->geom.nv * p->geom.views * p->vol.nt;
@@ -1481,7 +1479,7 @@ extern "C" msf_status msf_projector_create(const msf_geom* geom, const msf_vol* 
 
     auto cleanup = [&](msf_status st) { msf_projector_destroy(p); return st; };
     const size_t col_bytes = (size_t)G * geom->nu * 2 * sizeof(float4);
-    const size_t line_bytes = vz_pitch(vol->nz) * sizeof(float);
+    const size_t line_bytes = (VZ_FRONT + vz_pitch(vol->nz)) * sizeof(float);
     const size_t vz_bytes = vz_size(*vol) * sizeof(float);
     if (cudaMalloc(&p->d_angles, G * sizeof(double)) != cudaSuccess ||
         cudaMalloc(&p->d_col, col_bytes) != cudaSuccess ||
@@ -1570,7 +1568,6 @@ extern "C" msf_status msf_dataprox_create(msf_projector* p, msf_dataprox** out) 
     const size_t parts_icd = (size_t)gi.x * gi.y * (gi.z / nt);
     const size_t parts_fwd = (size_t)((p->dims.nu + 1) / 2) * p->dims.views * fwd_chunks(p->dims);
     if (cudaMalloc(&d->d_rows, nr * 4) != cudaSuccess || cudaMalloc(&d->d_rows2, nr * 4) != cudaSuccess ||
-        cudaMalloc(&d->d_sl, nr * 4) != cudaSuccess ||
         cudaMalloc(&d->d_ipart, (size_t)nt * parts_icd * 2 * 8) != cudaSuccess ||
         cudaMalloc(&d->d_spart, (size_t)nt * parts_fwd * 8) != cudaSuccess ||
         cudaMalloc(&d->d_r, nl * 4) != cudaSuccess || cudaMalloc(&d->d_p, nl * 4) != cudaSuccess ||
@@ -1582,11 +1579,12 @@ extern "C" msf_status msf_dataprox_create(msf_projector* p, msf_dataprox** out) 
         msf_dataprox_destroy(d);
         return fail(MSF_ERR_NOMEM, "msf_dataprox_create: out of device memory");
     }
+    // the lines that a projection or a gather reads need their margins cleared; those of
+    // d_r and d_q are loaded in units of four values at most, and dropped
     if (cudaMemset(d->d_status, 0, sizeof(int)) != cudaSuccess ||
         cudaMemset(d->d_count, 0, nt * sizeof(unsigned)) != cudaSuccess ||
-        cudaMemset(d->d_p, 0, nl * 4) != cudaSuccess || cudaMemset(d->d_r, 0, nl * 4) != cudaSuccess ||
-        cudaMemset(d->d_q, 0, nl * 4) != cudaSuccess || cudaMemset(d->d_rows, 0, nr * 4) != cudaSuccess ||
-        cudaMemset(d->d_rows2, 0, nr * 4) != cudaSuccess || cudaMemset(d->d_sl, 0, nr * 4) != cudaSuccess) {
+        cudaMemset(d->d_p, 0, nl * 4) != cudaSuccess || cudaMemset(d->d_rows, 0, nr * 4) != cudaSuccess ||
+        cudaMemset(d->d_rows2, 0, nr * 4) != cudaSuccess) {
         msf_dataprox_destroy(d);
         return fail(MSF_ERR_CUDA, "msf_dataprox_create: memset failed");
     }
@@ -1605,7 +1603,7 @@ extern "C" void msf_dataprox_destroy(msf_dataprox* d) {
     cudaFree(d->d_count);
     cudaFree(d->d_partial); cudaFree(d->d_rr); cudaFree(d->d_alpha); cudaFree(d->d_beta);
     cudaFree(d->d_status);
-    cudaFree(d->d_rows); cudaFree(d->d_rows2); cudaFree(d->d_sl); cudaFree(d->d_ipart); cudaFree(d->d_spart);
+    cudaFree(d->d_rows); cudaFree(d->d_rows2); cudaFree(d->d_ipart); cudaFree(d->d_spart);
     delete d;
 }
 
@@ -1675,10 +1673,10 @@ extern "C" msf_status msf_prox_data_icd(msf_dataprox* dp, const float* d_y, cons
     }
     // e' = step Lambda (y - A z)
     MSF_TRY((launch_fwd_lines<FWD_RESIDUAL, true>(p, z, dp->d_rows, d_lambda, d_y, st)));
-    {   // step Lambda, and step^2 Lambda in the buffer that then takes A delta
+    {   // step^2 Lambda, in the buffer that then takes step Lambda (A delta)
         MSF_PROF("icd_weights", st);
         icd_weights_kernel<<<dim3(nt * d.views, (d.nu + 31) / 32, (d.nv + 31) / 32), dim3(32, 8), 0, st>>>(
-            p->d_col, d_lambda, dp->d_sl, dp->d_rows2, d);
+            p->d_col, d_lambda, dp->d_rows2, d);
         MSF_LAUNCH_CHECK();
     }
     // theta2 = (A^T Lambda A)_ss + 1/sigma^2
@@ -1691,7 +1689,7 @@ extern "C" msf_status msf_prox_data_icd(msf_dataprox* dp, const float* d_y, cons
             G.gx = par_count(v.nx, G.px); G.gy = par_count(v.ny, G.py); G.gz = par_count(v.nz, G.pz);
             if (G.gx == 0 || G.gy == 0 || G.gz == 0) continue;
             MSF_TRY(launch_icd_group(p, dp->d_rows, z, vl, theta2, dlt, &S, inv_s2, G, st));
-            {   // A delta and alpha
+            {   // step Lambda (A delta), and alpha
                 MSF_PROF("joseph_fwd", st);
                 launch_fwd_kernel<FWD_ICD, true, true>(p, dlt, dp->d_rows2, d_lambda, nullptr, G.px, G.py, S, st);
                 MSF_LAUNCH_CHECK();
@@ -1700,8 +1698,7 @@ extern "C" msf_status msf_prox_data_icd(msf_dataprox* dp, const float* d_y, cons
                 MSF_PROF("icd_update", st);
                 const size_t lines = std::max((size_t)d.views * d.nu, (size_t)G.gx * G.gy);
                 const int half = (int)std::min<size_t>(256, (lines + 7) / 8);
-                icd_update_kernel<<<dim3(2 * half, nt), 256, 0, st>>>(dp->d_rows, dp->d_sl, dp->d_rows2, z, dlt,
-                                                                      dp->d_alpha, G, d);
+                icd_update_kernel<<<dim3(2 * half, nt), 256, 0, st>>>(dp->d_rows, dp->d_rows2, z, dlt, dp->d_alpha, G, d);
                 MSF_LAUNCH_CHECK();
             }
         }
