@@ -101,20 +101,23 @@ typedef struct msf_projector msf_projector;
  * would lie inside the volume's circumscribed cylinder (dso and dsd-dso must
  * exceed its radius), or when a ray could be steeper than 45 deg to the
  * rotation plane (the z-major case, which this projector does not model).
- * Allocates the table, a copy of a 4D volume in lines along z (the forward's
- * input, 4 bytes per voxel and per element of the lines' margins) and a
- * step-weighted sinogram. */
+ * Allocates the table, the forward's input (a copy of a 4D volume in lines along
+ * z, 4 bytes per voxel and per element of the lines' margins; or, where the
+ * detector has too few rows or the volume too few slices to fill a warp with
+ * them, two z-paired copies in planes, 16 bytes per voxel) and a step-weighted
+ * sinogram. */
 msf_status msf_projector_create(const msf_geom* geom, const msf_vol* vol, msf_projector** out);
 void msf_projector_destroy(msf_projector* p);
 /* Device bytes held by the plan. */
 size_t msf_projector_bytes(const msf_projector* p);
 
 /* Autotuner: times the forward projector with its three launch shapes, named
- * 32x4, 64x2 and 16x8 (4, 8 or 2 detector columns per block, one warp each over
- * sets of 32 rows), and the gather adjoint with the z-runs 8, 16 and 32 (at most
- * 2, 4 or 6 voxels per lane of a block's lines, 32 lanes) and, when its grid is
- * still at least 24 waves of 8 blocks per SM deep, 64 (at most 12), on this
- * plan's geometry, and keeps the fastest of each for the plan.
+ * 32x4, 64x2 and 16x8 (in lines 4, 8 or 2 detector columns per block, one warp
+ * each over sets of 32 rows; in planes columns x pairs of rows), and the gather
+ * adjoint with the z-runs 8, 16 and 32 (in lines at most 2, 4 or 6 voxels per lane
+ * of a block's lines, 32 lanes; in planes voxels per thread) and, when its grid is
+ * still at least 24 waves of 8 blocks per SM deep, 64 (in lines at most 12), on
+ * this plan's geometry, and keeps the fastest of each for the plan.
  * Results do not depend on the choice (same per-ray arithmetic and the same
  * per-voxel summation order).  Synchronises; allocates a temporary buffer.
  * h_choice (optional, 3 ints) receives {block columns, block rows, z-run}. */
@@ -179,8 +182,8 @@ msf_status msf_weights(const float* d_counts, float* d_y, float* d_lambda, size_
 typedef struct msf_dataprox msf_dataprox;
 
 /* Workspace for the data proximal maps (CG and ICD) on the projector's problem
- * size: three 4D volumes in lines along z, two sinograms in lines of rows and
- * per-frame FP64 partial sums. */
+ * size: three 4D volumes in lines along z and two sinograms in lines of rows (in
+ * planes, four volumes and two sinograms), and per-frame FP64 partial sums. */
 msf_status msf_dataprox_create(msf_projector* p, msf_dataprox** out);
 void msf_dataprox_destroy(msf_dataprox* d);
 

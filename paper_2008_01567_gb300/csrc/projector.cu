@@ -16,54 +16,19 @@
 //     f_z(k) = (c_z + v*c1) + (k - c_maj) * (v*inv_dmaj)
 // in fractional voxel indices, and the chord per plane is
 //     step = sqrt(|d_xy|^2 + v^2) * voxel/|d_maj|.
+//
+// The kernels here take a warp's lanes along detector rows and along z, on volumes in
+// lines along z; thin detectors and volumes take those of projector_planes.cu
+// (choose_routes).
 #include <math.h>
 
 #include <algorithm>
 #include <mutex>
 #include <vector>
 
-#include "common.cuh"
+#include "projector.cuh"
 
 namespace msf {
-
-struct ColParams {
-    float fa_mid, ba, c1, inv_dmaj;   // minor-axis line, z factors
-    float dxy2, vox_over_adm, xmajor, pad;
-};
-
-struct ProjDims {
-    int nx, ny, nz, nt, nu, nv, views;
-    float cx, cy, cz, cu, cv;   // (n-1)/2 of each axis
-    float vox, du, dv;
-    float dso, dsd;
-};
-
-struct RayZ {
-    float fz_mid, bz, step;
-};
-
-// The one place where a ray's z constants are formed; forward and adjoint
-// both call it, with explicit round-to-nearest intrinsics so the compiler
-// cannot contract the two call sites differently.
-__device__ __forceinline__ RayZ ray_z(const ColParams& c, float v, float cz) {
-    RayZ r;
-    r.fz_mid = __fmaf_rn(v, c.c1, cz);
-    r.bz = __fmul_rn(v, c.inv_dmaj);
-    r.step = __fmul_rn(__fsqrt_rn(__fmaf_rn(v, v, c.dxy2)), c.vox_over_adm);
-    return r;
-}
-
-__device__ __forceinline__ float det_v(int iv, const ProjDims& d) {
-    return __fmul_rn(__fsub_rn((float)iv, d.cv), d.dv);
-}
-
-__device__ __forceinline__ ColParams load_col(const float4* __restrict__ col, size_t idx) {
-    float4 a = __ldg(col + 2 * idx), b = __ldg(col + 2 * idx + 1);
-    ColParams c;
-    c.fa_mid = a.x; c.ba = a.y; c.c1 = a.z; c.inv_dmaj = a.w;
-    c.dxy2 = b.x; c.vox_over_adm = b.y; c.xmajor = b.z; c.pad = b.w;
-    return c;
-}
 
 // ------------------------------------------------------------------ FP64 table
 
@@ -126,11 +91,12 @@ enum LinesMode { LINES_COPY = 0, LINES_PAIR = 1, LINES_BOTH = 2 };
 constexpr int LT = 64;
 
 // LINES_COPY: vz = lines of in.  LINES_PAIR: also vd = lines of v - in; LINES_BOTH:
-// also vd = lines of v.
+// also vd = lines of v.  margins: also clears those of vz (a plan that keeps pairs in
+// the same place).
 template <int MODE>
 __global__ void __launch_bounds__(256) lines_kernel(const float* __restrict__ in, float* __restrict__ vz,
                                                     const float* __restrict__ v, float* __restrict__ vd, int nx, int ny,
-                                                    int nz) {
+                                                    int nz, bool margins) {
     __shared__ float tile[LT][LT + 1];
     const int xt = (nx + LT - 1) / LT, ty = blockIdx.x / xt, t = ty / ny, y = ty % ny;
     const int x0 = blockIdx.x % xt * LT, z0 = blockIdx.y * LT;
@@ -161,6 +127,12 @@ __global__ void __launch_bounds__(256) lines_kernel(const float* __restrict__ in
             const int x = x0 + 4 * k + hi, z = z0 + lo;
             if (x < nx && z < nz) out[(((size_t)t * ny + y) * nx + x) * nzp + VZ_FRONT + z] = tile[lo][4 * k + hi];
         }
+    }
+    if (margins && blockIdx.y == 0) {
+        const int m = nzp - nz;
+        for (int i = threadIdx.x; i < LT * m && x0 + i / m < nx; i += blockDim.x)
+            vz[(((size_t)t * ny + y) * nx + x0 + i / m) * nzp + VZ_FRONT + nz + i % m] = 0.0f;
+        if (blockIdx.x == 0 && threadIdx.x < VZ_FRONT) vz[threadIdx.x] = 0.0f;
     }
 }
 
@@ -193,8 +165,6 @@ __global__ void __launch_bounds__(256) volume_kernel(const float* __restrict__ v
 
 // ------------------------------------------------------------------ forward
 
-enum FwdMode { FWD_PLAIN = 0, FWD_LAMBDA = 1, FWD_RESIDUAL = 2, FWD_ICD = 3 };
-
 // Row sets (32 detector rows each) of one warp.  Five sets share a plane's
 // in-plane arithmetic among the most rays (160 rows: 0.67 ms in one chunk of
 // five, 0.86 in two of three); up to four sets two planes are unrolled under a
@@ -216,57 +186,6 @@ __host__ __device__ __forceinline__ int sino_pitch(int nv) { return (nv + SINO_F
 // of two conversions.
 constexpr float FLOOR_MAGIC = 12582912.0f;
 constexpr int FLOOR_MAGIC_BITS = 0x4B400000;
-
-// Group dimensions: voxels of parity p along an axis of n voxels.
-__host__ __device__ __forceinline__ int par_count(int n, int p) { return (n - p + 1) / 2; }
-
-struct IcdGroup {
-    int px, py, pz;
-    int gx, gy, gz;   // group voxels along x, y, z
-};
-
-// Sums of a group step: per frame, theta1.delta and delta.delta of the gather's
-// blocks, Lambda (A delta)^2 of the forward's, and the line search's scalar
-//   alpha_t = -sum(theta1.delta) / (sum Lambda (A delta)^2 + sum(delta.delta)/sigma^2).
-struct IcdSums {
-    double *gpart, *spart;   // [nt][gblocks][2], [nt][blocks of a frame's forward]
-    int gblocks;
-    double* alpha;           // [nt]
-    double inv_s2;
-    int* status;
-    unsigned* count;         // [nt], zero between kernels
-};
-
-// The sum of a forward block's Lambda (A delta)^2 (in thread 0); the frame's last
-// block forms alpha_t from the partials of both kernels in a fixed order.
-__device__ __forceinline__ void icd_alpha(double sum, int t, int b, int nparts, const IcdSums& S) {
-    __shared__ bool last;
-    const int tid = threadIdx.x + blockDim.x * threadIdx.y, nthreads = blockDim.x * blockDim.y;
-    double* part = S.spart + (size_t)t * nparts;
-    if (tid == 0) {
-        part[b] = sum;
-        __threadfence();
-        last = atomicAdd(S.count + t, 1u) == (unsigned)nparts - 1;
-    }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    double gd = 0.0, dd = 0.0, sq = 0.0;
-    for (int i = tid; i < S.gblocks; i += nthreads) {
-        gd += S.gpart[2 * ((size_t)t * S.gblocks + i)];
-        dd += S.gpart[2 * ((size_t)t * S.gblocks + i) + 1];
-    }
-    for (int i = tid; i < nparts; i += nthreads) sq += __ldcg(part + i);
-    gd = block_sum_f64(gd);
-    dd = block_sum_f64(dd);
-    sq = block_sum_f64(sq);
-    if (tid == 0) {
-        const double den = sq + dd * S.inv_s2;
-        if (!isfinite(gd) || !isfinite(den)) atomicExch(S.status, (int)MSF_ERR_NUMERIC);
-        S.alpha[t] = (den > 0.0 && isfinite(den) && isfinite(gd)) ? -gd / den : 0.0;
-        S.count[t] = 0;
-    }
-}
 
 // A warp takes one detector column and R sets of 32 consecutive rows (lane =
 // row in a set); a block takes blockDim.y neighbouring columns.  All rays of a
@@ -468,71 +387,11 @@ __global__ void __launch_bounds__(256, R == 5 ? 1 : 3) joseph_fwd_kernel(
 
 // ------------------------------------------------------------------ adjoint (gather)
 
-enum AdjMode { ADJ_PLAIN = 0, ADJ_CG_INIT = 1, ADJ_CG_Q = 2, ADJ_THETA2 = 3 };
-
-// ------------------------------------------------------------------ CG scalars
-//
-// A kernel whose blocks each hold a partial sum of a frame hands them to the
-// frame's last block, which adds them in a fixed order and forms the scalar:
-//   FIN_RR0:   rr = sum
-//   FIN_ALPHA: alpha = rr / sum (0 when sum == 0)
-//   FIN_BETA:  beta = sum / rr (0 when rr == 0); rr = sum
-// Any non-finite sum raises the status flag.  (A kernel of its own per scalar
-// cost a launch, 11 per five CG steps.)
-enum FinMode { FIN_RR0 = 0, FIN_ALPHA = 1, FIN_BETA = 2 };
-
-struct CgScalars {
-    double* partial;      // [nt][blocks of a frame]
-    double *rr, *coef;    // [nt]
-    int* status;
-    unsigned* count;      // [nt], zero between kernels: blocks of the frame that have stored their sum
-};
-
-// sum: this block's partial, in thread 0; b of nparts: its place in frame t.
-template <int FIN>
-__device__ __forceinline__ void frame_finalize(double sum, int t, int b, int nparts, const CgScalars& c) {
-    __shared__ bool last;
-    const int tid = threadIdx.x + blockDim.x * threadIdx.y, nthreads = blockDim.x * blockDim.y;
-    double* part = c.partial + (size_t)t * nparts;
-    if (tid == 0) {
-        part[b] = sum;
-        __threadfence();
-        last = atomicAdd(c.count + t, 1u) == (unsigned)nparts - 1;
-    }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    double s = 0.0;
-    for (int i = tid; i < nparts; i += nthreads) s += __ldcg(part + i);
-    s = block_sum_f64(s);
-    if (tid == 0) {
-        if (!isfinite(s)) atomicExch(c.status, (int)MSF_ERR_NUMERIC);
-        if (FIN == FIN_RR0) {
-            c.rr[t] = s;
-        } else if (FIN == FIN_ALPHA) {
-            c.coef[t] = (s != 0.0) ? c.rr[t] / s : 0.0;
-        } else {
-            c.coef[t] = (c.rr[t] != 0.0) ? s / c.rr[t] : 0.0;
-            c.rr[t] = s;
-        }
-        c.count[t] = 0;
-    }
-}
-
-
 constexpr int ADJ_T = 4;           // a block's tile: ADJ_T x ADJ_T voxel lines in (x, y), one warp per ADJ_T
 constexpr int ADJ_ENTRIES = 32;    // columns of a warp's list
 // floats of one line in a block's tile: its 32 J voxels, and 8 that put the
 // lines read together on different banks
 __host__ __device__ constexpr int adj_line(int J) { return 32 * J + 8; }
-
-// Detector u coordinate (in pixels) of the point (x, y, .) for view (cs, sn);
-// only used to bound candidate columns, so a fast division is enough.
-__device__ __forceinline__ float u_pixel(float x, float y, float cs, float sn, const ProjDims& d) {
-    const float lat = -x * sn + y * cs;
-    const float depth = d.dso - x * cs - y * sn;
-    return __fdividef(d.dsd * lat, depth * d.du) + d.cu;
-}
 
 // One detector column that crosses a warp's run of voxel lines; what the packed
 // operations take is stored twice.
@@ -1230,59 +1089,23 @@ __global__ void phantom_project_kernel(const double* __restrict__ angles, float*
 
 // ====================================================================== handles
 
-struct msf_projector {
-    msf_geom geom;
-    msf_vol vol;
-    msf::ProjDims dims;
-    std::vector<double> angles;
-    double* d_angles = nullptr;
-    float4* d_col = nullptr;
-    float2* d_trig = nullptr;
-    int* d_vflag = nullptr;
-    float* d_vz = nullptr;     // z-contiguous lines of a volume (the forward's input)
-    float* d_zero = nullptr;   // one line of zeros
-    float* d_sw = nullptr;     // step-weighted sinogram for msf_backproject
-    int fwd_bx = 32, fwd_by = 4;   // forward launch shape (fwd_cols_of: detector columns per block)
-    int adj_zb = 64;               // gather z-run (adj_j: voxels per lane)
-    uint64_t tuning_gen = 0;       // advanced whenever the launch shapes change
-    size_t bytes = 0;
-};
-
-struct msf_dataprox {
-    msf_projector* p = nullptr;
-    // CG: residual, direction and A^T Lambda A p + p / sigma^2, as lines (d_q
-    // first holds v - z; z itself runs in the plan's d_vz)
-    float *d_r = nullptr, *d_p = nullptr, *d_q = nullptr;
-    // step-weighted sinograms in lines of rows: e' ; ICD: step Lambda (A delta) (first
-    // step^2 Lambda).  (ICD keeps delta, theta2 and v in d_p, d_r and d_q.)
-    float *d_rows = nullptr, *d_rows2 = nullptr;
-    double *d_partial = nullptr, *d_rr = nullptr, *d_alpha = nullptr, *d_beta = nullptr;
-    int* d_status = nullptr;
-    unsigned* d_count = nullptr;
-    int parts_upd = 0;
-    double *d_ipart = nullptr, *d_spart = nullptr;   // ICD: partial sums of the group gather and its forward
-};
-
 namespace msf {
 
-static size_t frame_size(const msf_vol& v) { return (size_t)v.nx * v.ny * v.nz; }
-static size_t vol_size(const msf_vol& v) { return frame_size(v) * v.nt; }
 static size_t vz_size(const msf_vol& v) {   // a volume as lines
     return VZ_FRONT + (size_t)v.nt * v.ny * v.nx * vz_pitch(v.nz);
 }
 static size_t rows_size(const msf_projector* p) {   // a sinogram in lines of rows
     return SINO_FRONT + (size_t)p->vol.nt * p->geom.views * p->geom.nu * sino_pitch(p->geom.nv);
 }
-static size_t sino_size(const msf_projector* p) {
-    return (size_t)p->geom.nu * p->geom.nv * p->geom.views * p->vol.nt;
-}
+// Whether the plan keeps lines and pairs in one place (some calls take either).
+static bool shared_input(const msf_projector* p) { return p->d_vz && p->d_px; }
 
 static dim3 lines_grid(const msf_vol& v) { return dim3((v.nx + LT - 1) / LT * v.ny * v.nt, (v.nz + LT - 1) / LT); }
 
 static msf_status launch_lines(msf_projector* p, const float* in, cudaStream_t st) {
     const msf_vol& v = p->vol;
     MSF_PROF("transpose", st);
-    lines_kernel<LINES_COPY><<<lines_grid(v), 256, 0, st>>>(in, p->d_vz, nullptr, nullptr, v.nx, v.ny, v.nz);
+    lines_kernel<LINES_COPY><<<lines_grid(v), 256, 0, st>>>(in, p->d_vz, nullptr, nullptr, v.nx, v.ny, v.nz, shared_input(p));
     MSF_LAUNCH_CHECK();
     return MSF_OK;
 }
@@ -1397,6 +1220,44 @@ static msf_status launch_adj(msf_projector* p, const float* e, float* out, const
     return MSF_OK;
 }
 
+// Which calls take the planes' kernels (projector_planes.cu), where a warp's 32 lanes are
+// detector columns or voxels along x, instead of rows or voxels along z.  The bounds below
+// were drawn through times of both on 480 shapes of 16^2 to 512^2 voxels, 1 to 200 slices,
+// 1 to 160 rows, 24 to 48 views and 2 to 12 frames (given here as planes' gain over lines).
+// Where lanes are spare, the work sets the time once there is enough of it (columns, or lines
+// of voxels, of all frames); before that a warp's walk does, and the lines' is the shorter.
+//   A: up to a set of 32 rows, from 8000 columns for one row (128^2 x 1, 85920 columns: 6.7
+//      times) to 34000 for 32 (128^2 x 8, 85920: 1.2; 64^2, 42720: 0.95); with two sets, the
+//      second of which is short up to 48 rows, by columns x planes (384^2, 51552 columns: 33 rows
+//      1.3 to 1.5, 48 rows 1.0 to 1.1; 48^2, 32160: 0.9).
+//   A^T and CG: up to 16 slices by the lines of voxels (A^T of 512^2 x 1 x 2: 3.7 to 7.3 times,
+//      256^2 x 8 x 4: 1.9, 96^2 x 16 x 12: 1.0, 128^2 x 8 x 4: 1.15, 96^2 x 8 x 4: 0.75), sooner the
+//      more rows a voxel has; above, where the rows are too few for the voxels beside a column
+//      (384^2 x 64, 40 rows: 1.1, 64 rows: 0.67), or where CG's slower A outweighs A^T (384^2 x 24,
+//      33 rows: CG 1.14, A^T 0.97).
+//   ICD: its three launches a step tell in favour of lines further (192^2 x 12, 16 rows: 0.42;
+//      256^2 x 16 x 4: 0.87; 384^2 x 16 x 4: 1.18); in a workspace for planes it needs lines of at
+//      most 1.5 times the volume, as from eight slices.
+static void choose_routes(msf_projector* p) {
+    const ProjDims& d = p->dims;
+    if (!planes_fit(d)) return;
+    const int nz = d.nz, nv = d.nv;
+    const double cols = (double)d.nt * d.views * d.nu, lines = (double)d.nt * d.nx * d.ny;
+    p->fwd_planes = nv <= 32 ? cols >= 8000.0 + (nz <= 2 ? 4.0 : 25.0) * nv * nv
+                             : nv <= 48 && cols * std::max(d.nx, d.ny) >= 2e6 + 3.3e5 * (nv - 33);
+    if (nz <= 16) {
+        p->adj_planes = lines >= (16000.0 + 4500.0 * nz) * (nv >= 8 * nz ? 0.6 : nv >= 2 * nz ? 0.72 : 1.0);
+    } else if (nz < 24) {
+        p->adj_planes = lines >= 200000.0;
+    } else {
+        const int few = std::max(28, nz / 2 + (nz <= 64 ? 10 : 0));
+        p->adj_planes = (nv < few && lines >= (nz <= 64 ? 200000.0 : 130000.0)) ||
+                        (3 * nv < 2 * few && lines >= (nz <= 64 ? 50000.0 : 12000.0)) ||
+                        (p->fwd_planes && lines >= 400000.0 && (nz < 32 || (nz <= 40 && nv < 40)));
+    }
+    p->icd_planes = p->adj_planes && (nz < 8 || nv < 8 || 2 * nv <= nz || lines >= 18000.0 * nz);
+}
+
 static dim3 icd_grid(const ProjDims& d, int gx, int gy, int zrun) {
     const int pairs = (d.nz + 1) / 2, run = 32 * adj_j(pairs, zrun);
     return dim3((gx + ADJ_T - 1) / ADJ_T, (gy + ADJ_T - 1) / ADJ_T, (pairs + run - 1) / run * d.nt);
@@ -1477,21 +1338,32 @@ extern "C" msf_status msf_projector_create(const msf_geom* geom, const msf_vol* 
     d.vox = (float)vol->voxel; d.du = (float)geom->du; d.dv = (float)geom->dv;
     d.dso = (float)geom->dso; d.dsd = (float)geom->dsd;
 
+    choose_routes(p);
+    const bool planes = p->fwd_planes || p->adj_planes, lines = !p->fwd_planes || !p->adj_planes || !p->icd_planes;
+    if (p->adj_planes) p->adj_zb = 16;
+
     auto cleanup = [&](msf_status st) { msf_projector_destroy(p); return st; };
     const size_t col_bytes = (size_t)G * geom->nu * 2 * sizeof(float4);
     const size_t line_bytes = (VZ_FRONT + vz_pitch(vol->nz)) * sizeof(float);
-    const size_t vz_bytes = vz_size(*vol) * sizeof(float);
+    const size_t pair_bytes = planes ? vol_size(*vol) * 2 * sizeof(float2) : 0;
+    const size_t vz_bytes = lines ? vz_size(*vol) * sizeof(float) : 0;
+    const size_t in_bytes = std::max(pair_bytes, (p->adj_planes && !p->icd_planes ? 2 : 1) * vz_bytes);   // ICD: z and v
+    const size_t sw_bytes = (p->adj_planes ? sino_size(p) : rows_size(p)) * sizeof(float);
     if (cudaMalloc(&p->d_angles, G * sizeof(double)) != cudaSuccess ||
         cudaMalloc(&p->d_col, col_bytes) != cudaSuccess ||
         cudaMalloc(&p->d_trig, G * sizeof(float2)) != cudaSuccess ||
         cudaMalloc(&p->d_vflag, G * sizeof(int)) != cudaSuccess ||
-        cudaMalloc(&p->d_vz, vz_bytes) != cudaSuccess || cudaMalloc(&p->d_zero, line_bytes) != cudaSuccess ||
-        cudaMalloc(&p->d_sw, rows_size(p) * sizeof(float)) != cudaSuccess) {
+        cudaMalloc(&p->d_in, in_bytes) != cudaSuccess || cudaMalloc(&p->d_zero, line_bytes) != cudaSuccess ||
+        cudaMalloc(&p->d_sw, sw_bytes) != cudaSuccess) {
         cudaGetLastError();
         return cleanup(fail(MSF_ERR_NOMEM, "msf_projector_create: out of device memory"));
     }
-    p->bytes = G * sizeof(double) + col_bytes + G * (sizeof(float2) + sizeof(int)) + vz_bytes + line_bytes +
-               rows_size(p) * sizeof(float);
+    if (lines) p->d_vz = static_cast<float*>(p->d_in);
+    if (planes) {
+        p->d_px = static_cast<float2*>(p->d_in);
+        p->d_py = p->d_px + vol_size(*vol);
+    }
+    p->bytes = G * sizeof(double) + col_bytes + G * (sizeof(float2) + sizeof(int)) + in_bytes + line_bytes + sw_bytes;
     std::vector<float2> trig(G);
     for (int g = 0; g < G; ++g) trig[g] = make_float2((float)cos(p->angles[g]), (float)sin(p->angles[g]));
     int* d_bad = nullptr;
@@ -1499,9 +1371,9 @@ extern "C" msf_status msf_projector_create(const msf_geom* geom, const msf_vol* 
     cudaError_t e = cudaMemcpy(p->d_angles, p->angles.data(), G * sizeof(double), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(p->d_trig, trig.data(), G * sizeof(float2), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(p->d_vflag, 0, G * sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(p->d_vz, 0, vz_bytes);
+    if (e == cudaSuccess && lines && !planes) e = cudaMemset(p->d_vz, 0, vz_bytes);   // the lines' margins
     if (e == cudaSuccess) e = cudaMemset(p->d_zero, 0, line_bytes);
-    if (e == cudaSuccess) e = cudaMemset(p->d_sw, 0, rows_size(p) * sizeof(float));
+    if (e == cudaSuccess) e = cudaMemset(p->d_sw, 0, sw_bytes);
     if (e == cudaSuccess) e = cudaMalloc(&d_bad, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(d_bad, 0, sizeof(int));
     if (e == cudaSuccess) {
@@ -1524,7 +1396,7 @@ extern "C" void msf_projector_destroy(msf_projector* p) {
     cudaFree(p->d_col);
     cudaFree(p->d_trig);
     cudaFree(p->d_vflag);
-    cudaFree(p->d_vz);
+    cudaFree(p->d_in);
     cudaFree(p->d_zero);
     cudaFree(p->d_sw);
     delete p;
@@ -1534,12 +1406,14 @@ extern "C" size_t msf_projector_bytes(const msf_projector* p) { return p ? p->by
 
 extern "C" msf_status msf_project(msf_projector* p, const float* d_x, float* d_y, void* stream) {
     MSF_REQUIRE(p && d_x && d_y, "msf_project: NULL argument");
+    if (p->fwd_planes) return planes_project(p, d_x, d_y, as_stream(stream));
     return launch_fwd<FWD_PLAIN, false>(p, d_x, d_y, nullptr, nullptr, as_stream(stream));
 }
 
 extern "C" msf_status msf_backproject(msf_projector* p, const float* d_y, float* d_x, void* stream) {
     MSF_REQUIRE(p && d_x && d_y, "msf_backproject: NULL argument");
     cudaStream_t st = as_stream(stream);
+    if (p->adj_planes) return planes_backproject(p, d_y, d_x, st);
     {
         const ProjDims& d = p->dims;
         MSF_PROF("step_weight", st);
@@ -1550,48 +1424,83 @@ extern "C" msf_status msf_backproject(msf_projector* p, const float* d_y, float*
     return launch_adj<ADJ_PLAIN>(p, p->d_sw, d_x, nullptr, nullptr, CgScalars{}, 0.0f, st);
 }
 
-extern "C" msf_status msf_dataprox_create(msf_projector* p, msf_dataprox** out) {
-    MSF_REQUIRE(p && out, "msf_dataprox_create: NULL argument");
-    *out = nullptr;
-    msf_dataprox* d = new msf_dataprox();
-    d->p = p;
+// Partial sums of the ICD agent in lines: the largest grids of any group (parity 0) and tuning.
+static size_t icd_ipart(const msf_projector* p) {
+    const dim3 g = icd_grid(p->dims, par_count(p->vol.nx, 0), par_count(p->vol.ny, 0), 8);
+    return (size_t)g.x * g.y * g.z * 2;
+}
+static size_t icd_spart(const msf_projector* p) {
+    return (size_t)((p->dims.nu + 1) / 2) * p->dims.views * fwd_chunks(p->dims) * p->vol.nt;
+}
+
+// The data agents' workspace in lines.
+static msf_status lines_alloc(msf_dataprox* d) {
+    const msf_projector* p = d->p;
     const size_t nl = vz_size(p->vol), nr = rows_size(p);
+    const int nt = p->vol.nt;
     const dim3 ga = adj_grid(p->dims, 8);             // the largest block count of any z-run
     const int parts_adj = ga.x * ga.y * adj_nzb(p->dims, 8);
     // blocks of a frame of the vector kernels: eight warps of one line or more each
     const size_t lines = (size_t)p->vol.nx * p->vol.ny;
     d->parts_upd = lines < 8 * 512 ? (int)((lines + 7) / 8) : 512;
     const int parts_max = parts_adj > d->parts_upd ? parts_adj : d->parts_upd;
-    const int nt = p->vol.nt;
-    // the largest grids of any group (parity 0) and tuning
-    const dim3 gi = icd_grid(p->dims, par_count(p->vol.nx, 0), par_count(p->vol.ny, 0), 8);
-    const size_t parts_icd = (size_t)gi.x * gi.y * (gi.z / nt);
-    const size_t parts_fwd = (size_t)((p->dims.nu + 1) / 2) * p->dims.views * fwd_chunks(p->dims);
     if (cudaMalloc(&d->d_rows, nr * 4) != cudaSuccess || cudaMalloc(&d->d_rows2, nr * 4) != cudaSuccess ||
-        cudaMalloc(&d->d_ipart, (size_t)nt * parts_icd * 2 * 8) != cudaSuccess ||
-        cudaMalloc(&d->d_spart, (size_t)nt * parts_fwd * 8) != cudaSuccess ||
-        cudaMalloc(&d->d_r, nl * 4) != cudaSuccess || cudaMalloc(&d->d_p, nl * 4) != cudaSuccess ||
-        cudaMalloc(&d->d_q, nl * 4) != cudaSuccess || cudaMalloc(&d->d_count, nt * sizeof(unsigned)) != cudaSuccess ||
-        cudaMalloc(&d->d_partial, (size_t)nt * parts_max * 8) != cudaSuccess ||
-        cudaMalloc(&d->d_rr, nt * 8) != cudaSuccess || cudaMalloc(&d->d_alpha, nt * 8) != cudaSuccess ||
-        cudaMalloc(&d->d_beta, nt * 8) != cudaSuccess || cudaMalloc(&d->d_status, sizeof(int)) != cudaSuccess) {
+        cudaMalloc(&d->d_ipart, icd_ipart(p) * 8) != cudaSuccess ||
+        cudaMalloc(&d->d_spart, icd_spart(p) * 8) != cudaSuccess || cudaMalloc(&d->d_r, nl * 4) != cudaSuccess ||
+        cudaMalloc(&d->d_p, nl * 4) != cudaSuccess || cudaMalloc(&d->d_q, nl * 4) != cudaSuccess ||
+        cudaMalloc(&d->d_partial, (size_t)nt * parts_max * 8) != cudaSuccess)
+        return MSF_ERR_NOMEM;
+    d->i_v = d->d_q;
+    d->i_theta2 = d->d_r;
+    d->i_delta = d->d_p;
+    return MSF_OK;
+}
+
+// The lines that a projection or a gather reads need their margins cleared; those of d_r
+// and d_q are loaded in units of four values at most, and dropped.
+static bool lines_clear(msf_dataprox* d) {
+    const size_t nl = vz_size(d->p->vol), nr = rows_size(d->p);
+    return cudaMemset(d->d_p, 0, nl * 4) == cudaSuccess && cudaMemset(d->d_rows, 0, nr * 4) == cudaSuccess &&
+           cudaMemset(d->d_rows2, 0, nr * 4) == cudaSuccess;
+}
+
+// The workspace of a plan whose CG takes planes, with the ICD agent's lines in it.
+static msf_status planes_alloc(msf_dataprox* d) {
+    const msf_projector* p = d->p;
+    if (p->icd_planes) return planes_dataprox_alloc(d, 0, 0, 0);
+    MSF_TRY(planes_dataprox_alloc(d, rows_size(p), icd_ipart(p), icd_spart(p)));
+    d->i_v = p->d_vz + vz_size(p->vol);
+    d->i_theta2 = d->d_r;
+    d->i_delta = d->d_r + vz_size(p->vol);
+    return MSF_OK;
+}
+
+extern "C" msf_status msf_dataprox_create(msf_projector* p, msf_dataprox** out) {
+    MSF_REQUIRE(p && out, "msf_dataprox_create: NULL argument");
+    *out = nullptr;
+    msf_dataprox* d = new msf_dataprox();
+    d->p = p;
+    const int nt = p->vol.nt;
+    msf_status st = p->adj_planes ? planes_alloc(d) : lines_alloc(d);
+    if (st == MSF_OK &&
+        (cudaMalloc(&d->d_count, nt * sizeof(unsigned)) != cudaSuccess || cudaMalloc(&d->d_rr, nt * 8) != cudaSuccess ||
+         cudaMalloc(&d->d_alpha, nt * 8) != cudaSuccess || cudaMalloc(&d->d_beta, nt * 8) != cudaSuccess ||
+         cudaMalloc(&d->d_status, sizeof(int)) != cudaSuccess))
+        st = MSF_ERR_NOMEM;
+    if (st != MSF_OK) {
         cudaGetLastError();
         msf_dataprox_destroy(d);
-        return fail(MSF_ERR_NOMEM, "msf_dataprox_create: out of device memory");
+        return fail(st, "msf_dataprox_create: out of device memory");
     }
-    // the lines that a projection or a gather reads need their margins cleared; those of
-    // d_r and d_q are loaded in units of four values at most, and dropped
-    if (cudaMemset(d->d_status, 0, sizeof(int)) != cudaSuccess ||
-        cudaMemset(d->d_count, 0, nt * sizeof(unsigned)) != cudaSuccess ||
-        cudaMemset(d->d_p, 0, nl * 4) != cudaSuccess || cudaMemset(d->d_rows, 0, nr * 4) != cudaSuccess ||
-        cudaMemset(d->d_rows2, 0, nr * 4) != cudaSuccess) {
+    if ((!p->adj_planes && !lines_clear(d)) || cudaMemset(d->d_status, 0, sizeof(int)) != cudaSuccess ||
+        cudaMemset(d->d_count, 0, nt * sizeof(unsigned)) != cudaSuccess) {
         msf_dataprox_destroy(d);
         return fail(MSF_ERR_CUDA, "msf_dataprox_create: memset failed");
     }
-    const msf_status settled = settle_default_stream();
-    if (settled != MSF_OK) {
+    st = settle_default_stream();
+    if (st != MSF_OK) {
         msf_dataprox_destroy(d);
-        return settled;
+        return st;
     }
     *out = d;
     return MSF_OK;
@@ -1599,7 +1508,11 @@ extern "C" msf_status msf_dataprox_create(msf_projector* p, msf_dataprox** out) 
 
 extern "C" void msf_dataprox_destroy(msf_dataprox* d) {
     if (!d) return;
-    cudaFree(d->d_r); cudaFree(d->d_p); cudaFree(d->d_q);
+    cudaFree(d->d_r);
+    if (!d->d_p2) {   // (planes: one allocation)
+        cudaFree(d->d_p);
+        cudaFree(d->d_q);
+    }
     cudaFree(d->d_count);
     cudaFree(d->d_partial); cudaFree(d->d_rr); cudaFree(d->d_alpha); cudaFree(d->d_beta);
     cudaFree(d->d_status);
@@ -1616,6 +1529,7 @@ extern "C" msf_status msf_prox_data(msf_dataprox* dp, const float* d_y, const fl
     msf_projector* p = dp->p;
     cudaStream_t st = as_stream(stream);
     const float inv_s2 = (float)(1.0 / (sigma * sigma));
+    if (p->adj_planes) return planes_prox_cg(dp, d_y, d_lambda, d_v, d_x, inv_s2, n_cg, st);
     const msf_vol& v = p->vol;
     const size_t lines = (size_t)v.nx * v.ny;
     const dim3 ugrid(dp->parts_upd, v.nt);
@@ -1624,7 +1538,7 @@ extern "C" msf_status msf_prox_data(msf_dataprox* dp, const float* d_y, const fl
     float* z = p->d_vz;
     {   // z and v - z as lines
         MSF_PROF("transpose", st);
-        lines_kernel<LINES_PAIR><<<lines_grid(v), 256, 0, st>>>(d_x, z, d_v, dp->d_q, v.nx, v.ny, v.nz);
+        lines_kernel<LINES_PAIR><<<lines_grid(v), 256, 0, st>>>(d_x, z, d_v, dp->d_q, v.nx, v.ny, v.nz, shared_input(p));
         MSF_LAUNCH_CHECK();
     }
     // r = A^T Lambda (y - A z) + (v - z)/sigma^2 ; p = r ; rr = r.r
@@ -1661,14 +1575,20 @@ extern "C" msf_status msf_prox_data_icd(msf_dataprox* dp, const float* d_y, cons
     if (n_sweeps == 0) return MSF_OK;
     msf_projector* p = dp->p;
     cudaStream_t st = as_stream(stream);
+    if (p->icd_planes) return planes_prox_icd(dp, d_y, d_lambda, d_v, d_x, sigma, n_sweeps, st);
     const ProjDims& d = p->dims;
     const msf_vol& v = p->vol;
     const int nt = v.nt;
     const float inv_s2 = (float)(1.0 / (sigma * sigma));
-    float *z = p->d_vz, *vl = dp->d_q, *theta2 = dp->d_r, *dlt = dp->d_p;
+    float *z = p->d_vz, *vl = dp->i_v, *theta2 = dp->i_theta2, *dlt = dp->i_delta;
+    if (p->adj_planes) {   // the margins, in a workspace that CG overwrites
+        MSF_TRY_CUDA(cudaMemsetAsync(dlt, 0, vz_size(v) * sizeof(float), st));
+        MSF_TRY_CUDA(cudaMemsetAsync(dp->d_rows, 0, rows_size(p) * sizeof(float), st));
+        MSF_TRY_CUDA(cudaMemsetAsync(dp->d_rows2, 0, rows_size(p) * sizeof(float), st));
+    }
     {   // z and v as lines
         MSF_PROF("transpose", st);
-        lines_kernel<LINES_BOTH><<<lines_grid(v), 256, 0, st>>>(d_x, z, d_v, vl, v.nx, v.ny, v.nz);
+        lines_kernel<LINES_BOTH><<<lines_grid(v), 256, 0, st>>>(d_x, z, d_v, vl, v.nx, v.ny, v.nz, shared_input(p));
         MSF_LAUNCH_CHECK();
     }
     // e' = step Lambda (y - A z)
@@ -1926,8 +1846,8 @@ extern "C" msf_status msf_projector_autotune(msf_projector* p, void* stream, int
     MSF_REQUIRE(p, "msf_projector_autotune: NULL plan");
     cudaStream_t st = as_stream(stream);
     const size_t nv = vol_size(p->vol), ns = sino_size(p);
-    // inputs: the plan's own scratch (transposed stack and step-weighted sinogram)
-    // are overwritten; outputs go to a temporary buffer allocated here
+    // inputs: the plan's own scratch, whose values the timing does not depend on (pairs and
+    // step-weighted sinogram are cleared); outputs go to a temporary buffer allocated here
     float* tmp = nullptr;
     MSF_TRY_CUDA(cudaMalloc(&tmp, (nv > ns ? nv : ns) * sizeof(float)));
     cudaEvent_t e0, e1;
@@ -1944,14 +1864,19 @@ extern "C" msf_status msf_projector_autotune(msf_projector* p, void* stream, int
         cudaEventElapsedTime(&ms, e0, e1);
         return ms;
     };
-    MSF_TRY_CUDA(cudaMemsetAsync(p->d_sw, 0, rows_size(p) * sizeof(float), st));
+    MSF_TRY_CUDA(cudaMemsetAsync(p->d_sw, 0, (p->adj_planes ? sino_size(p) : rows_size(p)) * sizeof(float), st));
+    if (p->d_px) MSF_TRY_CUDA(cudaMemsetAsync(p->d_px, 0, 2 * nv * sizeof(float2), st));
     const int shapes[3][2] = {{32, 4}, {64, 2}, {16, 8}};
     float best = 1e30f;
     int bi = 0;
     for (int i = 0; i < 3; ++i) {
         p->fwd_bx = shapes[i][0];
         p->fwd_by = shapes[i][1];
-        const float ms = time_it([&] { launch_fwd_kernel<FWD_PLAIN, false, false>(p, p->d_vz, tmp, nullptr, nullptr, 0, 0, IcdSums{}, st); });
+        const float ms = time_it([&] {   // A's kernel, and the agents' where they take the other layout
+            if (p->fwd_planes || p->adj_planes) planes_project_pairs(p, tmp, st);
+            if (!p->fwd_planes || !p->adj_planes)
+                launch_fwd_kernel<FWD_PLAIN, false, false>(p, p->d_vz, tmp, nullptr, nullptr, 0, 0, IcdSums{}, st);
+        });
         if (ms < best) { best = ms; bi = i; }
     }
     p->fwd_bx = shapes[bi][0];
@@ -1966,12 +1891,16 @@ extern "C" msf_status msf_projector_autotune(msf_projector* p, void* stream, int
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         nsm = 0;
     const dim3 g64 = adj_grid(p->dims, 64);
-    const bool deep64 = nsm > 0 && (double)g64.x * g64.y * g64.z >= 24.0 * 8.0 * nsm;
+    const double blocks64 = p->adj_planes ? (double)planes_adj_blocks(p->dims, 64) * p->dims.nt : (double)g64.x * g64.y * g64.z;
+    const bool deep64 = nsm > 0 && blocks64 >= 24.0 * 8.0 * nsm;
     best = 1e30f;
     int bz = 1;
     for (int i = 0; i < (deep64 ? 4 : 3); ++i) {
         p->adj_zb = zbs[i];
-        const float ms = time_it([&] { launch_adj_zb<ADJ_PLAIN>(p, p->d_sw, tmp, nullptr, nullptr, CgScalars{}, 0.0f, st); });
+        const float ms = time_it([&] {
+            if (p->adj_planes) planes_gather(p, p->d_sw, tmp, st);
+            else launch_adj_zb<ADJ_PLAIN>(p, p->d_sw, tmp, nullptr, nullptr, CgScalars{}, 0.0f, st);
+        });
         if (ms < best) { best = ms; bz = i; }
     }
     p->adj_zb = zbs[bz];
