@@ -2704,15 +2704,19 @@ __global__ void __launch_bounds__(256) wgrad_last_kernel(const float* __restrict
     const int lane8 = threadIdx.x & 7, row = threadIdx.x >> 3;    // 32 pixel rows x 8 channel groups
     float acc[3][8] = {};
     unsigned b = (p_lo + row) % W, a = (p_lo + row) / W % H;
-    // the loads of four pixels before their terms (a tap outside the image adds 0)
+    // the loads of four pixels before their terms (a tap outside the image adds 0 * 0: a
+    // non-finite gradient has no term there)
     for (unsigned p0 = p_lo + row; p0 < p_hi; p0 += 4 * 32) {
         float d[4];
+        bool left[4], right[4];
         uint4 u[4][3];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const unsigned p = p0 + 32 * j;
             const bool in = p < p_hi && (unsigned)((int)a + dy) < (unsigned)H;
             d[j] = in ? dR[p] : 0.0f;
+            left[j] = b > 0;
+            right[j] = b + 1 < (unsigned)W;
 #pragma unroll
             for (int dx = -1; dx <= 1; ++dx)
                 u[j][dx + 1] = in && (unsigned)((int)b + dx) < (unsigned)W ? act[((ptrdiff_t)p + dy * W + dx) * 8 + lane8]
@@ -2723,10 +2727,11 @@ __global__ void __launch_bounds__(256) wgrad_last_kernel(const float* __restrict
         for (int j = 0; j < 4; ++j)
 #pragma unroll
             for (int t = 0; t < 3; ++t) {
+                const float dt = t == 0 ? (left[j] ? d[j] : 0.0f) : t == 2 ? (right[j] ? d[j] : 0.0f) : d[j];
                 float f[8];
                 bf16x8_to_f32(u[j][t], f);
 #pragma unroll
-                for (int k = 0; k < 8; ++k) acc[t][k] = fmaf(d[j], f[k], acc[t][k]);
+                for (int k = 0; k < 8; ++k) acc[t][k] = fmaf(dt, f[k], acc[t][k]);
             }
     }
     // reduce the 32 rows through shared memory
