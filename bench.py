@@ -229,7 +229,7 @@ def algorithmic(scan, K1):
         "joseph_adj": ("hbm", 4.0 * (M + 2 * N)),
         # volume order <-> lines along z (two volumes each way)
         "transpose": ("hbm", 16.0 * N),
-        "volume": ("hbm", 12.0 * N),
+        "volume": ("hbm", 20.0 * N),
         "cg_residual": ("hbm", 12.0 * N),
         "cg_direction": ("hbm", 20.0 * N),
         # one colour of the ICD sweep: its voxels read/written, all neighbours read

@@ -136,25 +136,43 @@ __global__ void __launch_bounds__(256) lines_kernel(const float* __restrict__ in
     }
 }
 
-// x[nt][nz][ny][nx] = z (+ alpha_t p), z and p as lines (ADD: the last CG step).
+// x[nt][nz][ny][nx] = z (+ alpha_t p), z and p as lines (ADD: the last CG step, whose new
+// residual r - alpha_t q has no reader: squared and added by eights, as cg_residual_kernel
+// would, it raises the status flag if that is not finite).
 template <bool ADD>
 __global__ void __launch_bounds__(256) volume_kernel(const float* __restrict__ vz, const float* __restrict__ p,
-                                                     const double* __restrict__ alpha, float* __restrict__ out, int nx,
-                                                     int ny, int nz) {
+                                                     const float* __restrict__ r, const float* __restrict__ q,
+                                                     const double* __restrict__ alpha, float* __restrict__ out,
+                                                     int* __restrict__ status, int nx, int ny, int nz) {
     __shared__ float tile[LT][LT + 1];
     const int xt = (nx + LT - 1) / LT, ty = blockIdx.x / xt, t = ty / ny, y = ty % ny;
     const int x0 = blockIdx.x % xt * LT, z0 = blockIdx.y * LT;
     const int nzp = vz_pitch(nz);
     const int lo = threadIdx.x % LT, hi = threadIdx.x / LT;
     const float a = ADD ? (float)alpha[t] : 0.0f;
+    bool ok = true;
 #pragma unroll
-    for (int k = 0; k < LT / 4; ++k) {
-        const int x = x0 + 4 * k + hi, z = z0 + lo;
-        if (x < nx && z < nz) {
+    for (int k0 = 0; k0 < LT / 4; k0 += 8) {   // eight voxels' loads before their sums
+        float zv[8], pv[8], rv[8], qv[8], run = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int x = x0 + 4 * (k0 + k) + hi, z = z0 + lo;
+            const bool in = x < nx && z < nz;
             const size_t i = (((size_t)t * ny + y) * nx + x) * nzp + VZ_FRONT + z;
-            tile[lo][4 * k + hi] = ADD ? __fmaf_rn(a, p[i], vz[i]) : vz[i];
+            zv[k] = in ? vz[i] : 0.0f;
+            pv[k] = ADD && in ? p[i] : 0.0f;
+            rv[k] = ADD && in ? r[i] : 0.0f;
+            qv[k] = ADD && in ? q[i] : 0.0f;
         }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            tile[lo][4 * (k0 + k) + hi] = ADD ? __fmaf_rn(a, pv[k], zv[k]) : zv[k];
+            const float rn = __fmaf_rn(-a, qv[k], rv[k]);
+            run = __fmaf_rn(rn, rn, run);
+        }
+        ok = ok && isfinite(run);
     }
+    if (ADD && !ok) atomicExch(status, (int)MSF_ERR_NUMERIC);
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < LT / 4; ++k) {
@@ -1560,9 +1578,10 @@ extern "C" msf_status msf_prox_data(msf_dataprox* dp, const float* d_y, const fl
             MSF_LAUNCH_CHECK();
         }
     }
-    // the last step's z + alpha p, back in volume order (its r has no reader)
+    // the last step's z + alpha p, back in volume order
     MSF_PROF("volume", st);
-    volume_kernel<true><<<lines_grid(v), 256, 0, st>>>(z, dp->d_p, dp->d_alpha, d_x, v.nx, v.ny, v.nz);
+    volume_kernel<true><<<lines_grid(v), 256, 0, st>>>(z, dp->d_p, dp->d_r, dp->d_q, dp->d_alpha, d_x, dp->d_status, v.nx,
+                                                       v.ny, v.nz);
     MSF_LAUNCH_CHECK();
     return MSF_OK;
 }
@@ -1624,7 +1643,7 @@ extern "C" msf_status msf_prox_data_icd(msf_dataprox* dp, const float* d_y, cons
         }
     }
     MSF_PROF("volume", st);
-    volume_kernel<false><<<lines_grid(v), 256, 0, st>>>(z, nullptr, nullptr, d_x, v.nx, v.ny, v.nz);
+    volume_kernel<false><<<lines_grid(v), 256, 0, st>>>(z, nullptr, nullptr, nullptr, nullptr, d_x, nullptr, v.nx, v.ny, v.nz);
     MSF_LAUNCH_CHECK();
     return MSF_OK;
 }

@@ -34,3 +34,20 @@ def test_infinite_loss_gradient_at_a_corner_misses_the_taps_outside(M):
     g = M.unpack_params(c.get_grads())[0][9][0].reshape(64, 3, 3)
     assert np.isfinite(g[:, 0, :]).all() and np.isfinite(g[:, :, 0]).all()
     assert not np.isfinite(g[:, 1:, 1:]).any()
+
+
+@pytest.mark.parametrize("n_cg", [1, 2])
+def test_residual_that_overflows_in_the_last_step_is_reported(M, n_cg):
+    # readings of 1e12 with weights of 1e8: the residual's values are near 1e21, their
+    # squares beyond FP32, the state stays near 1e12
+    import torch
+    scan = synth.Scan(n=16, nt=2, nu=24, nv=22, views=5)
+    shape = (2, scan.nt, scan.n, scan.n, scan.n)
+    W, X = torch.zeros(shape, device="cuda"), torch.zeros(shape, device="cuda")
+    y = torch.full((scan.nt, scan.views, scan.nv, scan.nu), 1e12, device="cuda")
+    y *= 1 + torch.rand(y.shape, device="cuda", generator=torch.Generator("cuda").manual_seed(3))
+    m = M.Mace(M.Projector(scan), W, X, y, torch.full_like(y, 1e8), M.MSF_PRIOR_QGGMRF, mrf=M.msf_mrf(2.0, 1.2, 1.0, 0.1, 0.5))
+    with pytest.raises(M.MsfError) as e:
+        M.msf_mace_step(m, 0.5, 1.0, [0.5, 0.5], n_cg, 1)
+    assert e.value.status == 5 and "CG" in str(e.value)
+    assert n_cg > 1 or torch.isfinite(X).all()
