@@ -15,6 +15,7 @@ namespace msf {
 
 // Scale of the terms 1 + r whose product shares a reciprocal (qggmrf_pair).
 constexpr float MRF_SCALE = 0x1p-33f;
+enum MrfKind { MRF_USUAL = 0, MRF_NEAR = 1, MRF_APART = 2 };   // of arithmetic (qggmrf_pair)
 
 struct MrfDims {
     int nx, ny, nz, nt;
@@ -25,16 +26,21 @@ struct MrfDims {
     float pq;                    // p - q
     // surrogate coefficients of the face, edge, corner and temporal neighbours,
     // 2 b a(D) = w (k1 + k2 w) with w = 1 / (1 + r): 2 b (q/p) / (2 sigma_x^2) and
-    // 2 b (1 - q/p) / (2 sigma_x^2)  (p = 2); `usual`: w is 1 / MRF_SCALE times that, and k1 and k2
-    // MRF_SCALE and its square times
+    // 2 b (1 - q/p) / (2 sigma_x^2)  (p = 2); MRF_USUAL: w is 1 / MRF_SCALE times that, and k1 and
+    // k2 MRF_SCALE and its square times
     float k1[4], k2[4];
-    bool usual;
+    int kind;
     float bt;                    // temporal weight
 };
 
 __device__ __forceinline__ float lg2_ftz(float x) {
     float r;
     asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float lg2_full(float x) {   // of subnormal numbers too
+    float r;
+    asm("lg2.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
 __device__ __forceinline__ float ex2_ftz(float x) {
@@ -53,29 +59,33 @@ __device__ __forceinline__ float rcp_ftz(float x) {
 //   a(D) = 1/(2 sx^2) * (1 + (q/p) r)/(1 + r)^2,   r = |D/(T sx)|^(p-q),
 // in partial fractions of 1/(1 + r).  r is formed as exp2((p-q) log2 .) with the
 // hardware approximations (about 2^-21 relative, far inside the FP32 tolerance of
-// the agent; a term flushed to zero is below 2^-126 beside the 1).  USUAL: the two
-// share a reciprocal, since the special function unit bounds these kernels (28
-// neighbours, a logarithm, a power and a reciprocal each).  The terms are formed
-// MRF_SCALE times as large, so that their product stays a normal number for any FP32 r
-// beside one of 2^64: unscaled it passed 2^126 at two outliers of 2^63, and both
-// weights vanished, though with q = 1 an outlier's influence does not fall with its
-// distance.  Otherwise (coefficients that would lose bits to the scale) each term has a
-// reciprocal of its own.
-template <bool USUAL>
+// the agent).  The two share a reciprocal, since the special function unit bounds these
+// kernels (28 neighbours, a logarithm, a power and a reciprocal each).
+//   MRF_USUAL: p - q >= 0.2.  A ratio below 2^-126 is flushed to r = 0: its r is below
+//     2^-25, and the sum 1 either way.  The terms are formed MRF_SCALE times as large, so
+//     that their product stays a normal number for any FP32 r beside one of 2^64: unscaled
+//     it passed 2^126 at two outliers of 2^63, and both weights vanished, though with q = 1
+//     an outlier's influence does not fall with its distance.
+//   MRF_NEAR: p - q < 0.2.  r is at most 2^26, no product overflows; the logarithm takes
+//     subnormal ratios, which the power brings back to the size of the 1.
+//   MRF_APART: coefficients that would lose bits to the scale; a reciprocal each.
+template <int KIND>
 __device__ __forceinline__ f32x2 qggmrf_pair(f32x2 D, int kind, const MrfDims& m) {
     float r0 = 1.0f, r1 = 1.0f;
     if (m.pq != 0.0f) {
         float d0, d1;
         unpack2(mul2(D, pack2(m.inv_tsx, m.inv_tsx)), d0, d1);
-        unpack2(mul2(pack2(lg2_ftz(fabsf(d0)), lg2_ftz(fabsf(d1))), pack2(m.pq, m.pq)), d0, d1);
+        d0 = KIND == MRF_USUAL ? lg2_ftz(fabsf(d0)) : lg2_full(fabsf(d0));
+        d1 = KIND == MRF_USUAL ? lg2_ftz(fabsf(d1)) : lg2_full(fabsf(d1));
+        unpack2(mul2(pack2(d0, d1), pack2(m.pq, m.pq)), d0, d1);
         r0 = ex2_ftz(d0);
         r1 = ex2_ftz(d1);
     }
-    constexpr float S = USUAL ? MRF_SCALE : 1.0f;
+    constexpr float S = KIND == MRF_USUAL ? MRF_SCALE : 1.0f;
     float x, y;
     unpack2(fma2(pack2(r0, r1), pack2(S, S), pack2(S, S)), x, y);
     f32x2 w;
-    if (USUAL) {
+    if (KIND != MRF_APART) {
         const float rc = rcp_ftz(__fmul_rn(x, y));
         w = mul2(pack2(y, x), pack2(rc, rc));
     } else {
@@ -114,7 +124,7 @@ __device__ __forceinline__ bool inner(int iy, int iz, int t, const MrfDims& m) {
 }
 
 // The minimiser of voxel (ix, iy, iz) of frame t given its neighbours.
-template <bool USUAL>
+template <int KIND>
 __device__ __forceinline__ void icd_voxel(const float* __restrict__ v, float* z, int ix, int iy, int iz,
                                           int t, const MrfDims& m) {
     float* c = z + (((size_t)t * m.nz + iz) * m.ny + iy) * m.nx + ix;
@@ -123,7 +133,7 @@ __device__ __forceinline__ void icd_voxel(const float* __restrict__ v, float* z,
     auto pair = [&](ptrdiff_t o1, bool in1, ptrdiff_t o2, bool in2, int kind) {
         const f32x2 zr = pack2(in1 ? c[o1] : zs, in2 ? c[o2] : zs);
         float a1, a2;
-        unpack2(qggmrf_pair<USUAL>(sub2(pack2(zs, zs), zr), kind, m), a1, a2);
+        unpack2(qggmrf_pair<KIND>(sub2(pack2(zs, zs), zr), kind, m), a1, a2);
         const f32x2 a = pack2(in1 ? a1 : 0.0f, in2 ? a2 : 0.0f);
         num = fma2(a, zr, num);
         den = add2(den, a);
@@ -145,8 +155,9 @@ __device__ __forceinline__ void icd_voxel(const float* __restrict__ v, float* z,
 // -> 7.4e-8) 3.18, without bounds checks in y, z and t inside the volume 3.12, and, with
 // the scaled terms, twelve blocks per SM asked for (BLOCKS; 40 registers) 3.07 (3.38 at the
 // 48 that the compiler takes by itself, which a colour of few blocks, waiting for one
-// voxel's chain, is faster with: 33^3 x 4 133 against 170 us).
-template <bool USUAL, int BLOCKS>
+// voxel's chain, is faster with: 33^3 x 4 131 against 170 us, 64^3 x 4 180 against 197,
+// 110^3 x 3 329 against 326).
+template <int KIND, int BLOCKS>
 __global__ void __launch_bounds__(128, BLOCKS) icd_colour_kernel(const float* __restrict__ v,
                                                          float* __restrict__ z, MrfDims m) {
     const int hxv = blockIdx.x * 32 + threadIdx.x;
@@ -154,7 +165,7 @@ __global__ void __launch_bounds__(128, BLOCKS) icd_colour_kernel(const float* __
     const int hzv = blockIdx.z % m.hz;
     const int htv = blockIdx.z / m.hz;
     if (hxv >= m.hx || hyv >= m.hy) return;
-    icd_voxel<USUAL>(v, z, 2 * hxv + m.px, 2 * hyv + m.py, 2 * hzv + m.pz, 2 * htv + m.pt, m);
+    icd_voxel<KIND>(v, z, 2 * hxv + m.px, 2 * hyv + m.py, 2 * hzv + m.pz, 2 * htv + m.pt, m);
 }
 
 // All sweeps of a small volume in one launch: the CTAs of one cluster (8 SMs) take
@@ -163,7 +174,7 @@ __global__ void __launch_bounds__(128, BLOCKS) icd_colour_kernel(const float* __
 // 31 at 24^3, 64 at 24^3 x 4, the largest (3456 voxels per colour on 8 SMs).
 constexpr int ICD_CLUSTER = 8, ICD_SMALL_THREADS = 512;
 constexpr long long ICD_SMALL_VOXELS = (long long)ICD_CLUSTER * ICD_SMALL_THREADS;   // of the largest colour
-template <bool USUAL>
+template <int KIND>
 __global__ void __cluster_dims__(ICD_CLUSTER, 1, 1) __launch_bounds__(ICD_SMALL_THREADS)
     icd_small_kernel(const float* __restrict__ v, float* z, MrfDims m, int n_sweeps) {
     const int id = blockIdx.x * ICD_SMALL_THREADS + threadIdx.x;
@@ -172,7 +183,7 @@ __global__ void __cluster_dims__(ICD_CLUSTER, 1, 1) __launch_bounds__(ICD_SMALL_
         const int hx = (m.nx - px + 1) / 2, hy = (m.ny - py + 1) / 2, hz = (m.nz - pz + 1) / 2, ht = (m.nt - pt + 1) / 2;
         if (id < hx * hy * hz * ht) {
             const int x = id % hx, r = id / hx, y = r % hy, q = r / hy;
-            icd_voxel<USUAL>(v, z, 2 * x + px, 2 * y + py, 2 * (q % hz) + pz, 2 * (q / hz) + pt, m);
+            icd_voxel<KIND>(v, z, 2 * x + px, 2 * y + py, 2 * (q % hz) + pz, 2 * (q / hz) + pt, m);
         }
         // the colour's voxels, written by any CTA, before the next colour reads them
         asm volatile("barrier.cluster.arrive.release;" ::: "memory");
@@ -187,7 +198,7 @@ constexpr int MAP_BLOCKS = 152 * 8;
 // (L_a x)_s = sum_r b_sr a(anchor_s - anchor_r) (x_s - x_r) over the 26 spatial
 // and 2 temporal neighbours of s (free boundaries): half the gradient of the
 // prior's quadratic surrogate built at `anchor`.
-template <bool USUAL>
+template <int KIND>
 __device__ __forceinline__ float surrogate_lap(const float* __restrict__ anchor, const float* __restrict__ x,
                                                size_t s, int ix, int iy, int iz, int t, const MrfDims& m) {
     const float as = anchor[s], xs = x[s];
@@ -195,7 +206,7 @@ __device__ __forceinline__ float surrogate_lap(const float* __restrict__ anchor,
     neighbour_pairs<false>(ix, iy, iz, t, m, [&](ptrdiff_t o1, bool in1, ptrdiff_t o2, bool in2, int kind) {
         const f32x2 ar = pack2(in1 ? anchor[s + o1] : as, in2 ? anchor[s + o2] : as);
         const f32x2 xr = pack2(in1 ? x[s + o1] : xs, in2 ? x[s + o2] : xs);   // outside: a zero difference
-        acc = fma2(qggmrf_pair<USUAL>(sub2(pack2(as, as), ar), kind, m), sub2(pack2(xs, xs), xr), acc);
+        acc = fma2(qggmrf_pair<KIND>(sub2(pack2(as, as), ar), kind, m), sub2(pack2(xs, xs), xr), acc);
     });
     float a0, a1;
     unpack2(acc, a0, a1);
@@ -208,7 +219,7 @@ enum MapLapMode { MAP_INIT = 0, MAP_Q = 1 };
 //           d = r, partial r.r
 // MAP_Q:    q = data + 2 beta L_a d  (data = A^T Lambda A d held in q), partial d.q
 // One grid-stride pass over all voxels; per-block FP64 partials.
-template <int MODE, bool USUAL>
+template <int MODE, int KIND>
 __global__ void __launch_bounds__(256) map_lap_kernel(const float* __restrict__ anchor, const float* __restrict__ x,
                                                       float* __restrict__ out, float* __restrict__ out2,
                                                       float two_beta, MrfDims m, double* __restrict__ partial) {
@@ -220,7 +231,7 @@ __global__ void __launch_bounds__(256) map_lap_kernel(const float* __restrict__ 
         const int iz = (int)(r / sxy);
         const int rr = (int)(r - (size_t)iz * sxy);
         const int iy = rr / m.nx, ix = rr - iy * m.nx;
-        const float L = surrogate_lap<USUAL>(anchor, x, s, ix, iy, iz, t, m);
+        const float L = surrogate_lap<KIND>(anchor, x, s, ix, iy, iz, t, m);
         if (MODE == MAP_INIT) {
             const float v = fmaf(-two_beta, L, out[s]);
             out[s] = v;
@@ -234,6 +245,14 @@ __global__ void __launch_bounds__(256) map_lap_kernel(const float* __restrict__ 
     }
     const double b = block_sum_f64(dot);
     if (threadIdx.x == 0) partial[blockIdx.x] = b;
+}
+
+template <int MODE>
+static void launch_map_lap(const float* anchor, const float* x, float* out, float* out2, float two_beta, const MrfDims& m,
+                           double* partial, cudaStream_t st) {
+    auto* f = m.kind == MRF_USUAL ? map_lap_kernel<MODE, MRF_USUAL>
+              : m.kind == MRF_NEAR ? map_lap_kernel<MODE, MRF_NEAR> : map_lap_kernel<MODE, MRF_APART>;
+    f<<<MAP_BLOCKS, 256, 0, st>>>(anchor, x, out, out2, two_beta, m, partial);
 }
 
 // x += alpha d ; r -= alpha q ; partial r.r
@@ -379,8 +398,8 @@ static msf_status mrf_dims(const msf_vol* vol, const msf_mrf* prm, double sigma,
     const double b[4] = {1.0 / s, 1.0 / (sqrt(2.0) * s), 1.0 / (sqrt(3.0) * s), prm->b_temporal};
     // (a temporal weight so small that it loses bits is nothing beside the spatial ones)
     const double q1 = prm->q / prm->p;
-    m.usual = q1 == 1.0 || c * (1.0 - q1) >= 0x1p-54;
-    const double s1 = m.usual ? MRF_SCALE : 1.0;
+    m.kind = prm->p - prm->q < 0.2 ? MRF_NEAR : c * (1.0 - q1) >= 0x1p-54 ? MRF_USUAL : MRF_APART;
+    const double s1 = m.kind == MRF_USUAL ? MRF_SCALE : 1.0;
     for (int k = 0; k < 4; ++k) {
         m.k1[k] = (float)(b[k] * c * q1 * s1);
         m.k2[k] = (float)(b[k] * c * (1.0 - q1) * s1 * s1);
@@ -466,8 +485,7 @@ extern "C" msf_status msf_map_solve(msf_map* m, const msf_mrf* prm, double beta,
         MSF_TRY(msf_backproject(m->proj, m->d_s, m->d_r, sv));
         {
             MSF_PROF("map_lap", st);
-            (md.usual ? map_lap_kernel<MAP_INIT, true> : map_lap_kernel<MAP_INIT, false>)<<<MAP_BLOCKS, 256, 0, st>>>(
-                m->d_anchor, d_x, m->d_r, m->d_d, two_beta, md, m->d_part);
+            launch_map_lap<MAP_INIT>(m->d_anchor, d_x, m->d_r, m->d_d, two_beta, md, m->d_part, st);
             MSF_LAUNCH_CHECK();
         }
         {
@@ -486,8 +504,7 @@ extern "C" msf_status msf_map_solve(msf_map* m, const msf_mrf* prm, double beta,
             MSF_TRY(msf_backproject(m->proj, m->d_s, m->d_q, sv));
             {
                 MSF_PROF("map_lap", st);
-                (md.usual ? map_lap_kernel<MAP_Q, true> : map_lap_kernel<MAP_Q, false>)<<<MAP_BLOCKS, 256, 0, st>>>(
-                    m->d_anchor, m->d_d, m->d_q, nullptr, two_beta, md, m->d_part);
+                launch_map_lap<MAP_Q>(m->d_anchor, m->d_d, m->d_q, nullptr, two_beta, md, m->d_part, st);
                 MSF_LAUNCH_CHECK();
             }
             {
@@ -564,8 +581,9 @@ extern "C" msf_status msf_prox_qggmrf(const msf_vol* vol, const msf_mrf* prm, co
     const long long colour = (long long)((m.nx + 1) / 2) * ((m.ny + 1) / 2) * ((m.nz + 1) / 2) * ((m.nt + 1) / 2);
     if (colour <= ICD_SMALL_VOXELS) {
         MSF_PROF("qggmrf_icd", st);
-        (m.usual ? icd_small_kernel<true> : icd_small_kernel<false>)<<<ICD_CLUSTER, ICD_SMALL_THREADS, 0, st>>>(d_v, d_x, m,
-                                                                                                              n_sweeps);
+        auto* f = m.kind == MRF_USUAL ? icd_small_kernel<MRF_USUAL>
+                  : m.kind == MRF_NEAR ? icd_small_kernel<MRF_NEAR> : icd_small_kernel<MRF_APART>;
+        f<<<ICD_CLUSTER, ICD_SMALL_THREADS, 0, st>>>(d_v, d_x, m, n_sweeps);
         MSF_LAUNCH_CHECK();
         return MSF_OK;
     }
@@ -577,11 +595,12 @@ extern "C" msf_status msf_prox_qggmrf(const msf_vol* vol, const msf_mrf* prm, co
             if (m.hx <= 0 || m.hy <= 0 || m.hz <= 0 || m.ht <= 0) continue;
             dim3 grid((m.hx + 31) / 32, (m.hy + 3) / 4, m.hz * m.ht);
             MSF_PROF("qggmrf_icd", st);
-            // three waves of twelve blocks per SM: 128^3 x 6 (3.4) takes 542 us either way, 110^3 x 3 (1.7)
-            // 326 with twelve and 295 without
-            const bool deep = (long long)grid.x * grid.y * grid.z >= 3 * 12 * 152;
-            (!m.usual ? icd_colour_kernel<false, 1> : deep ? icd_colour_kernel<true, 12> : icd_colour_kernel<true, 1>)
-                <<<grid, dim3(32, 4), 0, st>>>(d_v, d_x, m);
+            // the twelve blocks of every SM
+            const bool deep = (long long)grid.x * grid.y * grid.z >= 12 * 152;
+            auto* f = m.kind == MRF_APART  ? icd_colour_kernel<MRF_APART, 1>
+                      : m.kind == MRF_NEAR ? (deep ? icd_colour_kernel<MRF_NEAR, 12> : icd_colour_kernel<MRF_NEAR, 1>)
+                                           : (deep ? icd_colour_kernel<MRF_USUAL, 12> : icd_colour_kernel<MRF_USUAL, 1>);
+            f<<<grid, dim3(32, 4), 0, st>>>(d_v, d_x, m);
             MSF_LAUNCH_CHECK();
         }
     }

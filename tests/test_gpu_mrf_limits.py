@@ -5,7 +5,7 @@ import pytest
 
 import oracle
 from paper_2008_01567_gb300 import synth
-from tests._problems import f32
+from tests._problems import I0, f32, measurement, rel_l2
 
 pytestmark = pytest.mark.gpu
 SHAPES = [(3, 5, 6, 40), (3, 18, 22, 70)]   # all sweeps in one launch, a launch per colour
@@ -45,3 +45,28 @@ def test_two_far_outliers_keep_their_influence(M, shape):
     # their influence, b / (2 sx) beside v / sigma^2, carries the logarithm's 2^-22 times
     # log2(1e32) times ln 2: 2e-5 of it, 1e-5 of a voxel
     assert np.abs(got - ref)[ok].max() <= 1e-5 * max(1.0, np.abs(ref[ok]).max())
+
+
+@pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "x".join(map(str, s)))
+@pytest.mark.parametrize("q", [1.8, 1.99, 2.0])
+def test_ratios_below_the_normal_numbers(M, shape, q):
+    # |D / (T sx)| near 1e-39, which p - q near 0 brings back to 0.4: 1e-5, the agent's bound
+    v, z = f32(1e-19 * synth.normal(55, shape)), f32(1e-19 * synth.normal(56, shape))
+    got = _sweeps(M, v, z, 1.0, q, 1e20, 1.0, 2)
+    assert rel_l2(1e19 * got, 1e19 * oracle.prox_qggmrf(v, z, 1.0, 2.0, q, 1e20, 1.0, 0.5, 2)) <= 1e-5
+
+
+def test_direct_map_with_ratios_below_the_normal_numbers(M):
+    # the surrogate's Laplacian of the direct MAP solve, T = 1e39; the bound of test_gpu_map.py
+    import torch
+    scan, n_outer, n_cg = synth.TINY, 2, 4
+    x0, counts, y, lam = measurement(scan, 51)
+    P, c = M.Projector(scan), torch.from_numpy(counts.astype(np.float32)).cuda()
+    yg, lg = torch.zeros_like(c), torch.zeros_like(c)
+    M.msf_weights(c, yg, lg, I0, I0)
+    xs = f32(0.5 * x0)
+    x = torch.from_numpy(xs.astype(np.float32)).cuda()
+    M.msf_map_solve(M.MapSolver(P), M.msf_mrf(2.0, 1.99, 1e39, 0.2, 0.5), 30.0, yg, lg, x, n_outer, n_cg)
+    ref = oracle.map_mm(f32(y), f32(lam), xs, scan, 2.0, 1.99, 1e39, 0.2, 0.5, 30.0, n_outer, n_cg)
+    assert rel_l2(x.cpu().numpy(), ref) <= 2 * n_outer * (n_cg + 1) * 1e-5
+    assert rel_l2(xs, ref) > 1e-2
