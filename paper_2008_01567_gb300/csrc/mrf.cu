@@ -123,9 +123,10 @@ __device__ __forceinline__ bool inner(int iy, int iz, int t, const MrfDims& m) {
     return iy > 0 && iy + 1 < m.ny && iz > 0 && iz + 1 < m.nz && t > 0 && t + 1 < m.nt;
 }
 
-// The minimiser of voxel (ix, iy, iz) of frame t given its neighbours.
+// The minimiser of voxel (ix, iy, iz) of frame t given its neighbours (v may be z: no
+// __restrict__, which would let loads of v miss the last sweep's values).
 template <int KIND>
-__device__ __forceinline__ void icd_voxel(const float* __restrict__ v, float* z, int ix, int iy, int iz,
+__device__ __forceinline__ void icd_voxel(const float* v, float* z, int ix, int iy, int iz,
                                           int t, const MrfDims& m) {
     float* c = z + (((size_t)t * m.nz + iz) * m.ny + iy) * m.nx + ix;
     const float zs = *c;
@@ -176,7 +177,7 @@ constexpr int ICD_CLUSTER = 8, ICD_SMALL_THREADS = 512;
 constexpr long long ICD_SMALL_VOXELS = (long long)ICD_CLUSTER * ICD_SMALL_THREADS;   // of the largest colour
 template <int KIND>
 __global__ void __cluster_dims__(ICD_CLUSTER, 1, 1) __launch_bounds__(ICD_SMALL_THREADS)
-    icd_small_kernel(const float* __restrict__ v, float* z, MrfDims m, int n_sweeps) {
+    icd_small_kernel(const float* v, float* z, MrfDims m, int n_sweeps) {
     const int id = blockIdx.x * ICD_SMALL_THREADS + threadIdx.x;
     for (int k = 0; k < 16 * n_sweeps; ++k) {
         const int px = k & 1, py = (k >> 1) & 1, pz = (k >> 2) & 1, pt = (k >> 3) & 1;

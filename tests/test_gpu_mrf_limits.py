@@ -56,6 +56,16 @@ def test_ratios_below_the_normal_numbers(M, shape, q):
     assert rel_l2(1e19 * got, 1e19 * oracle.prox_qggmrf(v, z, 1.0, 2.0, q, 1e20, 1.0, 0.5, 2)) <= 1e-5
 
 
+@pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "x".join(map(str, s)))
+def test_in_place_on_its_own_input(M, shape):
+    # d_v == d_x: every sweep takes the voxel's present value as v
+    z = f32(synth.normal(57, shape) + 1.0)
+    got, ref = _sweeps(M, z, z, 0.2, 1.2, 1.0, 0.1, 3, alias=True), z
+    for _ in range(3):
+        ref = oracle.prox_qggmrf(ref, ref, 0.2, 2.0, 1.2, 1.0, 0.1, 0.5, 1)
+    assert rel_l2(got, ref) <= 1e-5
+
+
 def test_direct_map_with_ratios_below_the_normal_numbers(M):
     # the surrogate's Laplacian of the direct MAP solve, T = 1e39; the bound of test_gpu_map.py
     import torch
