@@ -171,8 +171,11 @@ __global__ void __launch_bounds__(128, BLOCKS) icd_colour_kernel(const float* __
 
 // All sweeps of a small volume in one launch: the CTAs of one cluster (8 SMs) take
 // a colour's voxels, one each, and meet at the cluster's barrier between colours.
-// Launches set the time of such a volume, 16 a sweep (66 us): now 39 us at 8^3 x 2,
-// 31 at 24^3, 64 at 24^3 x 4, the largest (3456 voxels per colour on 8 SMs).
+// Issuing launches sets the time of such a volume, 16 a sweep (66 us; 33 with one frame): so
+// 39 us at 8^3 x 2, 29 at 24^3 and 32^3, 53 at 32^3 x 2, 64 at 24^3 x 4, 68 at 16^3 x 16 (the
+// largest, 4096 voxels per colour on 8 SMs).  Replayed from a graph sixteen launches cost
+// less than the cluster's barriers and few SMs (31 against 39 us at 8^3 x 2, 37 against 64 at
+// 24^3 x 4), so a captured call takes them.
 constexpr int ICD_CLUSTER = 8, ICD_SMALL_THREADS = 512;
 constexpr long long ICD_SMALL_VOXELS = (long long)ICD_CLUSTER * ICD_SMALL_THREADS;   // of the largest colour
 template <int KIND>
@@ -182,6 +185,7 @@ __global__ void __cluster_dims__(ICD_CLUSTER, 1, 1) __launch_bounds__(ICD_SMALL_
     for (int k = 0; k < 16 * n_sweeps; ++k) {
         const int px = k & 1, py = (k >> 1) & 1, pz = (k >> 2) & 1, pt = (k >> 3) & 1;
         const int hx = (m.nx - px + 1) / 2, hy = (m.ny - py + 1) / 2, hz = (m.nz - pz + 1) / 2, ht = (m.nt - pt + 1) / 2;
+        if (hx * hy * hz * ht == 0) continue;   // of a volume of one slice or frame, in every CTA
         if (id < hx * hy * hz * ht) {
             const int x = id % hx, r = id / hx, y = r % hy, q = r / hy;
             icd_voxel<KIND>(v, z, 2 * x + px, 2 * y + py, 2 * (q % hz) + pz, 2 * (q / hz) + pt, m);
@@ -580,7 +584,9 @@ extern "C" msf_status msf_prox_qggmrf(const msf_vol* vol, const msf_mrf* prm, co
     MSF_TRY(mrf_dims(vol, prm, sigma, &m));
     if (n_sweeps == 0) return MSF_OK;
     const long long colour = (long long)((m.nx + 1) / 2) * ((m.ny + 1) / 2) * ((m.nz + 1) / 2) * ((m.nt + 1) / 2);
-    if (colour <= ICD_SMALL_VOXELS) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) cudaGetLastError();   // (a launch will report it)
+    if (colour <= ICD_SMALL_VOXELS && capture == cudaStreamCaptureStatusNone) {
         MSF_PROF("qggmrf_icd", st);
         auto* f = m.kind == MRF_USUAL ? icd_small_kernel<MRF_USUAL>
                   : m.kind == MRF_NEAR ? icd_small_kernel<MRF_NEAR> : icd_small_kernel<MRF_APART>;

@@ -66,6 +66,26 @@ def test_in_place_on_its_own_input(M, shape):
     assert rel_l2(got, ref) <= 1e-5
 
 
+def test_captured_sweeps_equal_eager_ones(M):
+    # a captured call of a small volume takes a launch per colour, an eager one a launch for all:
+    # the same bits, also where colours are empty
+    import torch
+    for shape in ((1, 1, 9, 40), (2, 6, 7, 40), (1, 32, 32, 32)):
+        nt, nz, ny, nx = shape
+        vol, mrf = M.msf_vol(nx, ny, nz, nt, 1.0), M.msf_mrf(2.0, 1.2, 1.0, 0.1, 0.5)
+        g = torch.Generator("cuda").manual_seed(6)
+        v, z = (torch.randn(shape, device="cuda", generator=g) for _ in range(2))
+        a, b = z.clone(), z.clone()
+        M.msf_prox_qggmrf(vol, mrf, v, a, 0.2, 2)
+        graph, st = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+        torch.cuda.synchronize()
+        with torch.cuda.graph(graph, stream=st):
+            M.msf_prox_qggmrf(vol, mrf, v, b, 0.2, 2)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(a, b) and not torch.equal(a, z), shape
+
+
 def test_direct_map_with_ratios_below_the_normal_numbers(M):
     # the surrogate's Laplacian of the direct MAP solve, T = 1e39; the bound of test_gpu_map.py
     import torch
