@@ -114,10 +114,10 @@ size_t msf_projector_bytes(const msf_projector* p);
 /* Autotuner: times the forward projector with its three launch shapes, named
  * 32x4, 64x2 and 16x8 (in lines 4, 8 or 2 detector columns per block, one warp
  * each over sets of 32 rows; in planes columns x pairs of rows), and the gather
- * adjoint with the z-runs 8, 16 and 32 (in lines at most 2, 4 or 6 voxels per lane
- * of a block's lines, 32 lanes; in planes voxels per thread) and, when its grid is
- * still at least 24 waves of 8 blocks per SM deep, 64 (in lines at most 12), on
- * this plan's geometry, and keeps the fastest of each for the plan.
+ * adjoint with the z-runs 8, 16, 32 and 64 (in lines at most 2, 4, 6 or 12 voxels
+ * per lane of a block's lines, 32 lanes, each distinct launch once; in planes
+ * voxels per thread, 64 only when its grid is still at least 24 waves of 8 blocks
+ * per SM deep), on this plan's geometry, and keeps the fastest of each for the plan.
  * Results do not depend on the choice (same per-ray arithmetic and the same
  * per-voxel summation order).  Synchronises; allocates a temporary buffer.
  * h_choice (optional, 3 ints) receives {block columns, block rows, z-run}. */

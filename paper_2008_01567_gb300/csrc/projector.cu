@@ -1704,8 +1704,8 @@ static_assert(STATIC_MAX_VIEWS * 8 + STATIC_MAX_COLUMNS * 32 + STATIC_MAX_VIEWS 
 // explicit roundings (the lerp v00 + w_a (v01 - v00) along a, then along z,
 // and a round-to-nearest accumulation over increasing planes), and a plane
 // whose taps all lie outside the grid adds exactly zero in joseph_fwd_kernel,
-// so the result equals msf_project's bit for bit; only the addressing differs
-// (x-major rays read x-strided data here instead of the transposed copy).
+// so the result equals msf_project's bit for bit; only the addressing differs (the
+// volume's own order here instead of lines along z or planes of pairs).
 __global__ void __launch_bounds__(128) joseph_fwd_direct_kernel(const float* __restrict__ x,
                                                                 const float4* __restrict__ col,
                                                                 float* __restrict__ out, ProjDims d) {
@@ -1900,21 +1900,23 @@ extern "C" msf_status msf_projector_autotune(msf_projector* p, void* stream, int
     }
     p->fwd_bx = shapes[bi][0];
     p->fwd_by = shapes[bi][1];
-    // z-runs of 64 halve the gather's block count; they are tried only while
-    // their grid stays at least 24 waves deep (8 blocks per SM), because with a
-    // shallower grid, run beside other problems' kernels (a batch), the longer
-    // blocks measured slower although they won when timed alone
+    // Planes: z-runs of 64 halve the gather's block count; they are tried only while their grid
+    // stays at least 24 waves deep (8 blocks per SM), because with a shallower grid, run beside
+    // other problems' kernels (a batch), the longer blocks measured slower although they won when
+    // timed alone.  Lines: a run that gives a block the same voxels as one already timed is the
+    // same launch; otherwise what wins alone wins beside others, in shallow grids too (CG of
+    // 256^3 x 4 with runs of 32 and 64: 10.95 and 10.31 ms, four at once 42.0 and 39.4; 64^2 x 224 x 2,
+    // 512 blocks: 0.560 and 0.505, eight at once 3.07 and 2.94).
     const int zbs[4] = {8, 16, 32, 64};
     int nsm = 0, dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         nsm = 0;
-    const dim3 g64 = adj_grid(p->dims, 64);
-    const double blocks64 = p->adj_planes ? (double)planes_adj_blocks(p->dims, 64) * p->dims.nt : (double)g64.x * g64.y * g64.z;
-    const bool deep64 = nsm > 0 && blocks64 >= 24.0 * 8.0 * nsm;
+    const bool deep64 = nsm > 0 && (double)planes_adj_blocks(p->dims, 64) * p->dims.nt >= 24.0 * 8.0 * nsm;
     best = 1e30f;
-    int bz = 1;
-    for (int i = 0; i < (deep64 ? 4 : 3); ++i) {
+    int bz = 0;
+    for (int i = 0; i < 4; ++i) {
+        if (p->adj_planes ? i == 3 && !deep64 : i > 0 && adj_j(p->dims.nz, zbs[i]) == adj_j(p->dims.nz, zbs[i - 1])) continue;
         p->adj_zb = zbs[i];
         const float ms = time_it([&] {
             if (p->adj_planes) planes_gather(p, p->d_sw, tmp, st);
