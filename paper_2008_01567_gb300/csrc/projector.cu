@@ -649,9 +649,12 @@ __device__ __forceinline__ void gather_run(const float4* __restrict__ col, const
     }
 }
 
-// Blocks per SM that the register limit asks for: as measured fastest for each J
-// (384^3 x 2, J = 12: 1.81 ms with 4, 1.99 with 5, 2.47 with no limit; J = 6: 2.00
-// with 5, 2.22 with none; 128^3 x 8, J = 4: 0.67 with 6, 0.73 with none).
+// Blocks per SM that the register limit asks for, by A^T's time with 1 (no limit) / 4 / 5 / 6 / 8 of
+// them (us, 24 views): J = 1 (256^2 x 32 x 8) 1089-1094 with any; J = 2 (128^2 x 64 x 8) 327 / 327 / 328 /
+// 295 / 279; J = 3 (128^2 x 96 x 8) 401 / 401 / 368 / 348 / 348; J = 4 (128^3 x 8) 449 / 449 / 452 / 420 /
+// 416; J = 5 (160^3 x 4) 426 / 424 / 385 / 377 / 392; J = 6 (192^3 x 4) 649 / 640 / 582 / 605 / 614; J = 8
+// (256^3 x 2) 773 / 665 / 663 / 697 / 806; J = 10 (320^3) 699 / 636 / 692 / 731 / 964; J = 12 (384^3 x 2) 2768 /
+// 2076 / 2185 / 2519 / 3424 (with 3: 2164).
 __host__ __device__ constexpr int adj_min_blocks(int J) { return J >= 8 ? 4 : J >= 5 ? 5 : J >= 3 ? 6 : 8; }
 
 // Both phases of a block on the lines x0 + STR i, y0 + STR w, voxels z_lo + STR (lane
