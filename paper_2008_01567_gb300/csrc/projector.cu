@@ -1245,38 +1245,41 @@ static msf_status launch_adj(msf_projector* p, const float* e, float* out, const
 // detector columns or voxels along x, instead of rows or voxels along z.  The bounds below
 // were drawn through times of both on 480 shapes of 16^2 to 512^2 voxels, 1 to 200 slices,
 // 1 to 160 rows, 24 to 48 views and 2 to 12 frames (given here as planes' gain over lines).
-// Where lanes are spare, the work sets the time once there is enough of it (columns, or lines
-// of voxels, of all frames); before that a warp's walk does, and the lines' is the shorter.
-//   A: up to a set of 32 rows, from 8000 columns for one row (128^2 x 1, 85920 columns: 6.7
-//      times) to 34000 for 32 (128^2 x 8, 85920: 1.2; 64^2, 42720: 0.95); with two sets, the
-//      second of which is short up to 48 rows, by columns x planes (384^2, 51552 columns: 33 rows
-//      1.3 to 1.5, 48 rows 1.0 to 1.1; 48^2, 32160: 0.9).
-//   A^T and CG: up to 16 slices by the lines of voxels (A^T of 512^2 x 1 x 2: 3.7 to 7.3 times,
-//      256^2 x 8 x 4: 1.9, 96^2 x 16 x 12: 1.0, 128^2 x 8 x 4: 1.15, 96^2 x 8 x 4: 0.75), sooner the
-//      more rows a voxel has; above, where the rows are too few for the voxels beside a column
-//      (384^2 x 64, 40 rows: 1.1, 64 rows: 0.67), or where CG's slower A outweighs A^T (384^2 x 24,
-//      33 rows: CG 1.14, A^T 0.97).
-//   ICD: its three launches a step tell in favour of lines further (192^2 x 12, 16 rows: 0.42;
-//      256^2 x 16 x 4: 0.87; 384^2 x 16 x 4: 1.18); in a workspace for planes it needs lines of at
-//      most 1.5 times the volume, as from eight slices.
+// Where lanes are spare, the work sets the time once there is enough of it; before that a
+// warp's walk does, and the lines' is the shorter.
+//   A (the same bits either way): up to a set of 32 rows, from 8000 columns of all frames for
+//      one row (128^2 x 1, 85920 columns: 6.7 times) to 34000 for 32 (128^2 x 8, 85920: 1.2;
+//      64^2, 42720: 0.95); with two sets, the second of which is short up to 48 rows, by columns
+//      x planes (384^2, 51552 columns: 33 rows 1.3 to 1.5, 48 rows 1.0 to 1.1; 48^2, 32160: 0.9).
+//   A^T and CG: by the frame alone, since a voxel's terms are grouped otherwise, and a frame
+//      must not depend on how many others its problem has (a problem split by time-points
+//      equals the whole bit for bit).  The bounds are those of 12 frames, which no number up
+//      to that is slower with than the planes; fewer would be faster in lines near them.  Up
+//      to 16 slices by the frame's lines of voxels (512^2 x 1 x 2: 3.7 to 7.3 times, 96^2 x 8 x 12:
+//      1.4 to 1.7, 96^2 x 16 x 12: 1.0; 96^2 x 8 x 2: 0.50), sooner the more rows a voxel has; above,
+//      where the rows are too few for the voxels beside a column (384^2 x 64 x 4, 40 rows: 1.1, 64
+//      rows: 0.67), or where CG's slower A outweighs A^T (384^2 x 24 x 4, 33 rows: CG 1.14, A^T 0.97).
+//   ICD: its three launches a step tell in favour of lines further (128^2 x 8 x 12: 1.0 to 1.24,
+//      96^2 x 8 x 12: 0.76 to 0.96, 256^2 x 16 x 4: 0.87; 384^2 x 16 x 4: 1.18); in a workspace for planes
+//      it needs lines of at most 1.5 times the volume, as from eight slices.
 static void choose_routes(msf_projector* p) {
     const ProjDims& d = p->dims;
     if (!planes_fit(d)) return;
     const int nz = d.nz, nv = d.nv;
-    const double cols = (double)d.nt * d.views * d.nu, lines = (double)d.nt * d.nx * d.ny;
+    const double cols = (double)d.nt * d.views * d.nu, xy = (double)d.nx * d.ny;
     p->fwd_planes = nv <= 32 ? cols >= 8000.0 + (nz <= 2 ? 4.0 : 25.0) * nv * nv
                              : nv <= 48 && cols * std::max(d.nx, d.ny) >= 2e6 + 3.3e5 * (nv - 33);
     if (nz <= 16) {
-        p->adj_planes = lines >= (16000.0 + 4500.0 * nz) * (nv >= 8 * nz ? 0.6 : nv >= 2 * nz ? 0.72 : 1.0);
+        p->adj_planes = 12.0 * xy >= (16000.0 + 4500.0 * nz) * (nv >= 8 * nz ? 0.6 : nv >= 2 * nz ? 0.72 : 1.0);
     } else if (nz < 24) {
-        p->adj_planes = lines >= 200000.0;
+        p->adj_planes = 12.0 * xy >= 200000.0;
     } else {
         const int few = std::max(28, nz / 2 + (nz <= 64 ? 10 : 0));
-        p->adj_planes = (nv < few && lines >= (nz <= 64 ? 200000.0 : 130000.0)) ||
-                        (3 * nv < 2 * few && lines >= (nz <= 64 ? 50000.0 : 12000.0)) ||
-                        (p->fwd_planes && lines >= 400000.0 && (nz < 32 || (nz <= 40 && nv < 40)));
+        p->adj_planes = (nv < few && xy >= (nz <= 64 ? 50000.0 : 32500.0)) ||
+                        (3 * nv < 2 * few && xy >= (nz <= 64 ? 12500.0 : 3000.0)) ||
+                        (nv <= 48 && xy >= 100000.0 && (nz < 32 || (nz <= 40 && nv < 40)));
     }
-    p->icd_planes = p->adj_planes && (nz < 8 || nv < 8 || 2 * nv <= nz || lines >= 18000.0 * nz);
+    p->icd_planes = p->adj_planes && (nz < 8 || nv < 8 || 2 * nv <= nz || 12.0 * xy >= 18000.0 * nz);
 }
 
 static dim3 icd_grid(const ProjDims& d, int gx, int gy, int zrun) {

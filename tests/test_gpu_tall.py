@@ -110,6 +110,8 @@ def _icd(A, y, lam, v, z, sigma, sweeps, shape):
     for _ in range(sweeps):
         for g in range(8):
             on = group == g
+            if not on.any():
+                continue              # a volume of one slice
             th1 = np.where(on, -(A.T @ (lam * e)) + (z - v) / sigma ** 2, 0.0)
             d = -th1 / theta2
             ad = A @ d
