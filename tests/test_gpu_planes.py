@@ -159,3 +159,23 @@ def test_data_agents(M, shape, icd):
         out = got[-1].cpu().numpy().astype(np.float64).ravel()
         assert np.linalg.norm(out - ref) <= (2 * 8 if icd else 2 * 2) * 1e-5 * np.linalg.norm(ref)
         assert np.linalg.norm(xn - ref) > 1e-2 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("shape", [SHAPES[2], SHAPES[5], SHAPES[7]], ids=lambda s: "x".join(map(str, s)))
+def test_autotune_keeps_results(M, shape):
+    # plans of planes, of both layouts for the agents, and with A alone in planes
+    import torch
+    with _Plan(M, shape) as P:
+        g = torch.Generator("cuda").manual_seed(8)
+        x, e = torch.rand(P.volume().shape, device="cuda", generator=g), torch.rand(P.sino().shape, device="cuda", generator=g)
+        outs, choice = [], (ctypes.c_int * 3)()
+        for tuned in (False, True):
+            if tuned:
+                assert P.L.msf_projector_autotune(P.h, None, choice) == 0
+                assert choice[0] * choice[1] == 128 and choice[2] in (8, 16, 32, 64)
+            y, b = P.sino(), P.volume()
+            assert P.L.msf_project(P.h, x.data_ptr(), y.data_ptr(), None) == 0
+            assert P.L.msf_backproject(P.h, e.data_ptr(), b.data_ptr(), None) == 0
+            torch.cuda.synchronize()
+            outs.append((y, b))
+        assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
